@@ -23,7 +23,7 @@
 #include <algorithm>
 #include <vector>
 
-#include "hpg_internal.cuh"
+#include "stencil.cuh"
 
 namespace hpg {
 
@@ -47,28 +47,6 @@ __device__ __forceinline__ void ld_n(const float* p, float (&v)[N]) {
     v[0] = ld_dep(p);
   }
 }
-// The same through the read-only path (ld.global.nc), for a kernel that is
-// never launched programmatically: every writer of the vector has completed
-// before it starts, and its successors write only after their wait, so the
-// vector is constant while it runs (the multi-RHS SpMV: measured 782 -> 776
-// ms for the 64 x 8 batch against ld_n).
-template <int N>
-__device__ __forceinline__ void ldnc_n(const float* p, float (&v)[N]) {
-  if constexpr (N == 8) {
-    const float4 a = __ldg(reinterpret_cast<const float4*>(p));
-    const float4 b = __ldg(reinterpret_cast<const float4*>(p) + 1);
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-  } else if constexpr (N == 4) {
-    const float4 a = __ldg(reinterpret_cast<const float4*>(p));
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-  } else if constexpr (N == 2) {
-    const float2 a = __ldg(reinterpret_cast<const float2*>(p));
-    v[0] = a.x; v[1] = a.y;
-  } else {
-    v[0] = __ldg(p);
-  }
-}
 template <int N>
 __device__ __forceinline__ void st_n(float* p, const float (&v)[N]) {
   if constexpr (N == 8) {
@@ -84,34 +62,6 @@ __device__ __forceinline__ void st_n(float* p, const float (&v)[N]) {
 }
 
 // ------------------------------------------------- multi-RHS stencil kernels
-// Y = A X (Sec. 3.2.2) for R right-hand sides.  Never launched
-// programmatically (mspmv_t), so X is gathered through the read-only path.
-template <int R, int LPR>
-__global__ void __launch_bounds__(256)
-mspmv_kernel(const float* __restrict__ vals, const int* __restrict__ cols, long long ns,
-             const float* __restrict__ x, float* __restrict__ y) {
-  constexpr int RL = R / LPR;
-  pdl_trigger();
-  pdl_wait();
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const long long row = t / LPR;
-  const int lane = (int)(t % LPR);
-  if (row >= ns) return;
-  float acc[RL];
-#pragma unroll
-  for (int r = 0; r < RL; ++r) acc[r] = 0.0f;
-#pragma unroll
-  for (int s = 0; s < kSlots; ++s) {
-    const float a = ld_stream(vals + s * ns + row);
-    const int c = ld_stream(cols + s * ns + row);
-    float xv[RL];
-    ldnc_n<RL>(x + (long long)c * R + lane * RL, xv);
-#pragma unroll
-    for (int r = 0; r < RL; ++r) acc[r] = fma(a, xv[r], acc[r]);
-  }
-  st_n<RL>(y + row * R + lane * RL, acc);
-}
-
 // One Gauss-Seidel colour phase (Sec. 3.2.1) for R right-hand sides: rows
 // [row0, row0 + nrows) of one colour block; entries j >= valid_end read as
 // zero (first forward sweep from z = 0).  MC selects the slots loaded:
@@ -168,39 +118,6 @@ mgs_phase_kernel(const float* __restrict__ vals, const int* __restrict__ cols, l
 #pragma unroll
   for (int r = 0; r < RL; ++r) acc[r] = acc[r] / a[kCentre];
   st_n<RL>(z + row * R + lane * RL, acc);
-}
-
-// Fused residual + injection restriction (Sec. 3.2.4) for R right-hand sides;
-// MODE as for mgs_phase_kernel.
-template <int R, int MODE>
-__global__ void __launch_bounds__(256)
-mrestrict_kernel(const __grid_constant__ Geom gf, const __grid_constant__ Geom gc,
-                 const float* __restrict__ vals, const int* __restrict__ cols,
-                 const float* __restrict__ rhs, const float* __restrict__ z,
-                 float* __restrict__ rc) {
-  pdl_trigger();
-  pdl_wait();
-  const int cx = gf.cdx[kCoarseColour], cy = gf.cdy[kCoarseColour];
-  const long long cnt = (long long)cx * cy * gf.cdz[kCoarseColour];
-  const long long ns = gf.n_store;
-  const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (p >= cnt) return;
-  const long long row = gf.off[kCoarseColour] + p;
-  float acc[R];
-  ld_n<R>(rhs + row * R, acc);
-#pragma unroll
-  for (int s = 0; s < kSlots; ++s) {
-    const float a = ld_mat<MODE>(vals + s * ns + row);
-    const int c = ld_mat<MODE>(cols + s * ns + row);
-    float xv[R];
-    ld_n<R>(z + (long long)c * R, xv);
-#pragma unroll
-    for (int r = 0; r < R; ++r) acc[r] = fma(-a, xv[r], acc[r]);
-  }
-  const int I = (int)(p % cx);
-  const int J = (int)((p / cx) % cy);
-  const int K = (int)(p / ((long long)cx * cy));
-  st_n<R>(rc + store_index(gc, I, J, K) * R, acc);
 }
 
 // Prolongation and correction z_{f_c(I)} += zc_I (eq. (3) transposed).
@@ -499,25 +416,10 @@ static int msymgs(hpg_problem* h, int level, const float* rhs, float* z, bool fr
   return HPG_OK;
 }
 
-template <int R, int LPR>
-static cudaError_t mspmv_launch(hpg_problem* h, const Level& L, int block, cudaStream_t s,
-                                const float* x, float* y) {
-  return kl(h, mspmv_kernel<R, LPR>, grid_for(L.g.n_store * LPR, block), block, s, L.v32, L.cols,
-            L.g.n_store, x, y);
-}
-
-template <int R>
-static int mspmv_t(hpg_problem* h, int level, const float* x, float* y, cudaStream_t s) {
-  const Level& L = h->lev[level];
-  const Shape sh = shape_of(h, level, kShapeSpmv, R);
-  constexpr int L2 = R >= 2 ? 2 : 1;
-  return launch(h, K_SPMV, level, HPG_FP32, L.g.n_store * (27.0 * 8 + 2.0 * 4 * R), s,
-                "mspmv_kernel", [&] {
-                  h->pdl_next = false;   // required by the read-only gathers of X
-                  if (sh.lpr == 1) return mspmv_launch<R, 1>(h, L, sh.block, s, x, y);
-                  if (sh.lpr == 2) return mspmv_launch<R, L2>(h, L, sh.block, s, x, y);
-                  return mspmv_launch<R, R>(h, L, sh.block, s, x, y);
-                });
+// Y = A X on R-vectors; the tuned shape's block size, lanes per row do not apply.
+static int run_mspmv(hpg_problem* h, int R, int level, const float* x, float* y,
+                     cudaStream_t s) {
+  return stencil_spmv(h, level, R, x, y, s, shape_of(h, level, kShapeSpmv, R).block);
 }
 
 // z = M^{-1} r for R right-hand sides: the V-cycle of sparse.cu, phase for
@@ -540,15 +442,7 @@ static int mvcycle_t(hpg_problem* h, int l, const float* rhs, float* z, cudaStre
   float* zcv = bs->zc[l + 1];
   const long long cnt = (long long)L.g.cdx[kCoarseColour] * L.g.cdy[kCoarseColour] *
                         L.g.cdz[kCoarseColour];
-  rc = launch(h, K_RESTRICT, l, HPG_FP32, cnt * (27.0 * 8 + 3.0 * 4 * R), s, "mrestrict_kernel",
-              [&] {
-                const int mode = mmat_mode(L);
-                auto kern = mode == kMatStream     ? mrestrict_kernel<R, kMatStream>
-                            : mode == kMatResident ? mrestrict_kernel<R, kMatResident>
-                                                   : mrestrict_kernel<R, kMatCached>;
-                return kl(h, kern, grid_for(cnt, 256), 256, s, L.g, C.g, L.v32, L.cols, rhs, z,
-                          rcv);
-              });
+  rc = stencil_restrict(h, l, R, rhs, z, rcv, (float*)nullptr, s);
   if (rc) return rc;
   if ((rc = mvcycle_t<R>(h, l + 1, rcv, zcv, s))) return rc;
   rc = launch(h, K_PROLONG, l, HPG_FP32, cnt * 3.0 * 4 * R, s, "mprolong_kernel", [&] {
@@ -568,16 +462,6 @@ static int run_mvcycle(hpg_problem* h, int R, int level, const float* rhs, float
     case 2: return mvcycle_t<2>(h, level, rhs, z, s);
     case 4: return mvcycle_t<4>(h, level, rhs, z, s);
     default: return mvcycle_t<8>(h, level, rhs, z, s);
-  }
-}
-
-static int run_mspmv(hpg_problem* h, int R, int level, const float* x, float* y,
-                     cudaStream_t s) {
-  switch (R) {
-    case 1: return mspmv_t<1>(h, level, x, y, s);
-    case 2: return mspmv_t<2>(h, level, x, y, s);
-    case 4: return mspmv_t<4>(h, level, x, y, s);
-    default: return mspmv_t<8>(h, level, x, y, s);
   }
 }
 
@@ -949,39 +833,36 @@ mupdate_x_kernel(double* __restrict__ x, const float* __restrict__ d, long long 
 }
 
 // r = b - A x (FP64, Algorithm 3 outer residual) and ||r_r||^2 per
-// right-hand side, one thread per storage row.
+// right-hand side.  A thread meets one right-hand side only: lines, strides
+// and blocks of an R-vector are multiples of R.
 template <int R>
 __global__ void __launch_bounds__(kBThreads)
-mresidual_kernel(const double* __restrict__ vals, const int* __restrict__ cols, long long ns,
+mresidual_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<double> c,
+                 const __grid_constant__ RowPlan pl, const double* diag,
                  const double* __restrict__ b, const double* __restrict__ x,
                  double* __restrict__ res, double* partials, double* gpart,
                  unsigned int* counter, double* __restrict__ out) {
   pdl_trigger();
   pdl_wait();
-  double acc[R];
-#pragma unroll
-  for (int r = 0; r < R; ++r) acc[r] = 0.0;
-  const long long stride = (long long)gridDim.x * kBThreads;
-  for (long long row = blockIdx.x * (long long)kBThreads + threadIdx.x; row < ns;
-       row += stride) {
-    double v[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = ld_dep(b + row * R + r);
-#pragma unroll
-    for (int s = 0; s < kSlots; ++s) {
-      const double a = ld_stream(vals + s * ns + row);
-      const int c = ld_stream(cols + s * ns + row);
-#pragma unroll
-      for (int r = 0; r < R; ++r) v[r] = fma(-a, ld_dep(x + (long long)c * R + r), v[r]);
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      res[row * R + r] = v[r];
-      acc[r] = fma(v[r], v[r], acc[r]);
+  double acc[1] = {0.0};
+  auto take = [&](unsigned p, double v) {
+    res[p] = v;
+    acc[0] = fma(v, v, acc[0]);
+  };
+  const unsigned stride = gridDim.x * kBThreads;
+  for (unsigned t = blockIdx.x * kBThreads + threadIdx.x; t < pl.threads + pl.pad; t += stride) {
+    if (t < pl.threads) {
+      const unsigned e = t % (unsigned)g.we, q = t / (unsigned)g.we;
+      stencil_rows<double, -1, 1>(g, c, x, diag, (int)e, (int)(q % pl.groups),
+                                  (int)(q / pl.groups), [&](unsigned p) { return ld_dep(b + p); },
+                                  take);
+    } else {
+      const unsigned p = pad_element(g, t - pl.threads);
+      take(p, ld_dep(b + p) - ld_dep(x + p));
     }
   }
   __shared__ double sums[R];
-  if (mblock_partials_last<1, R>(acc, R, partials, gpart, counter, sums) && threadIdx.x < R)
+  if (mblock_partials_last<R, 1>(acc, 1, partials, gpart, counter, sums) && threadIdx.x < R)
     out[threadIdx.x] = sums[threadIdx.x];
 }
 
@@ -1207,7 +1088,7 @@ static int enqueue_mstep(hpg_problem* h, int k, unsigned long long next, cudaStr
   const long long len = bs->ns * R;
   int rc;
   if ((rc = mvcycle_t<R>(h, 0, bs->Q + k * len, bs->z, s))) return rc;
-  if ((rc = mspmv_t<R>(h, 0, bs->z, bs->w, s))) return rc;
+  if ((rc = run_mspmv(h, R, 0, bs->z, bs->w, s))) return rc;
   const int ncol = k + 1;
   float* qnew = bs->Q + (k + 1) * len;
   if ((rc = launch_mpass<R, kBGemvT>(h, ncol, nullptr, bs->h1, 0ULL, s))) return rc;
@@ -1244,13 +1125,12 @@ template <int R>
 static int enqueue_mouter(hpg_problem* h, unsigned long long loop, cudaStream_t s) {
   BatchSpace* bs = h->batch;
   const Level& L = h->lev[0];
-  int rc = launch(h, K_RESIDUAL, 0, HPG_FP64, L.n * (27.0 * 12.0 + 3.0 * 8.0 * R), s,
-                  "mresidual_kernel", [&] {
-                    return kl(h, mresidual_kernel<R>, bs->G, kBThreads, s, (const double*)L.v64,
-                              (const int*)L.cols, bs->ns, (const double*)bs->b,
-                              (const double*)bs->x, bs->r, bs->partials, gpart_of(bs),
-                              bs->counter, bs->rho2);
-                  });
+  const SGeom g = make_sgeom(L.g, R);
+  int rc = launch(h, K_RESIDUAL, 0, HPG_FP64, L.n * 3.0 * 8.0 * R, s, "mresidual_kernel", [&] {
+    return kl(h, mresidual_kernel<R>, bs->G, kBThreads, s, g, make_coef<double>(h->beta),
+              make_row_plan(g, 1), level_diag<double>(L), (const double*)bs->b,
+              (const double*)bs->x, bs->r, bs->partials, gpart_of(bs), bs->counter, bs->rho2);
+  });
   if (rc) return rc;
   return launch(h, K_NORM, 0, HPG_FP64, 0.0, s, "mouter_check_kernel", [&] {
     return kl(h, mouter_check_kernel<R>, 1, 32, s, (const double*)bs->rho2, bs->st, loop);
@@ -1562,7 +1442,7 @@ static int tune_t(hpg_problem* h, int reps, cudaStream_t s) {
             h->pdl_next = false;
             BSweep sw;
             rc = kind == kShapeGs ? msymgs<R>(h, l, a, b, false, sw, s)
-                                  : mspmv_t<R>(h, l, a, b, s);
+                                  : run_mspmv(h, R, l, a, b, s);
           }
           if (rc) break;
           if (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||

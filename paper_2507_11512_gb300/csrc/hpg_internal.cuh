@@ -162,13 +162,6 @@ __device__ __forceinline__ V ld_dep(const V* p) {
   return __ldca(p);
 }
 
-// Bulk prefetch of [p, p + bytes) into L2 by the TMA engine (no registers,
-// no completion to wait for).  p must be 16-byte aligned, bytes a multiple
-// of 16.
-__device__ __forceinline__ void prefetch_l2_bulk(const void* p, unsigned bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
 // ------------------------------------------------- TMA bulk copies, mbarriers
 // 1-D bulk copies global -> shared by the TMA engine, completion counted in
 // bytes on a shared-memory mbarrier.  Addresses must be 16-byte aligned and
@@ -229,20 +222,6 @@ __host__ __device__ constexpr unsigned gs_slot_mask(int c, bool from_zero) {
     if (nc < c) m |= 1u << s;
   }
   return m;
-}
-
-// One thread of the block prefetches the block's slice [row, row + rows) of
-// the 27 value and index slots of a slot-major ELL matrix.  row and rows are
-// multiples of 4 (colour blocks start on 32-row boundaries), so every range
-// starts on a 16-byte boundary and has a multiple-of-16 size.
-template <typename TV>
-__device__ __forceinline__ void prefetch_ell_rows(const TV* vals, const int* cols, long long ns,
-                                                  long long row, int rows) {
-  if (threadIdx.x != 0 || rows <= 0) return;
-  for (int s = 0; s < 27; ++s) {
-    prefetch_l2_bulk(vals + s * ns + row, (unsigned)(rows * sizeof(TV)));
-    prefetch_l2_bulk(cols + s * ns + row, (unsigned)(rows * sizeof(int)));
-  }
 }
 
 // ------------------------------------------------------------ host objects
@@ -367,8 +346,6 @@ void dev_free(void* p);
 // an error code and counts its launches in h->launches.
 int launch_spmv(hpg_problem* h, int level, hpg_prec prec, const void* x, void* y,
                 cudaStream_t s);
-int launch_residual64(hpg_problem* h, const double* b, const double* x, double* r,
-                      cudaStream_t s);
 // c0_done: z already holds the first sweep's colour-0 phase, z_i = r_i / a_ii
 // on colour block 0 (written by the kernel that produced r).
 int run_vcycle(hpg_problem* h, int level, hpg_prec prec, const void* r, void* z,

@@ -15,7 +15,7 @@
 
 #include <algorithm>
 
-#include "hpg_internal.cuh"
+#include "stencil.cuh"
 
 namespace hpg {
 
@@ -30,48 +30,6 @@ template <> struct Prec<double> {
 };
 
 // ------------------------------------------------------------------ kernels
-// y = A x over all storage rows (Sec. 3.2.2; Algorithm 3 SpMV).
-template <typename T>
-__global__ void __launch_bounds__(256)
-spmv_kernel(const T* __restrict__ vals, const int* __restrict__ cols, long long ns,
-            const T* __restrict__ x, T* __restrict__ y) {
-  pdl_trigger();
-  const long long row0 = blockIdx.x * (long long)blockDim.x;
-  prefetch_ell_rows(vals, cols, ns, row0, (int)min((long long)blockDim.x, ns - row0));
-  pdl_wait();
-  const long long row = row0 + threadIdx.x;
-  if (row >= ns) return;
-  T acc = T(0);
-#pragma unroll
-  for (int s = 0; s < kSlots; ++s) {
-    const T a = ld_stream(vals + s * ns + row);
-    const int c = ld_stream(cols + s * ns + row);
-    acc = fma(a, ld_dep(x + c), acc);
-  }
-  y[row] = acc;
-}
-
-// r = b - A x in FP64 (Algorithm 3, outer residual).
-__global__ void __launch_bounds__(256)
-residual64_kernel(const double* __restrict__ vals, const int* __restrict__ cols, long long ns,
-                  const double* __restrict__ b, const double* __restrict__ x,
-                  double* __restrict__ r) {
-  pdl_trigger();
-  const long long row0 = blockIdx.x * (long long)blockDim.x;
-  prefetch_ell_rows(vals, cols, ns, row0, (int)min((long long)blockDim.x, ns - row0));
-  pdl_wait();
-  const long long row = row0 + threadIdx.x;
-  if (row >= ns) return;
-  double acc = ld_dep(b + row);
-#pragma unroll
-  for (int s = 0; s < kSlots; ++s) {
-    const double a = ld_stream(vals + s * ns + row);
-    const int c = ld_stream(cols + s * ns + row);
-    acc = fma(-a, ld_dep(x + c), acc);
-  }
-  r[row] = acc;
-}
-
 // Rows a thread of a bandwidth-variant Gauss-Seidel phase takes, and the
 // 16-byte vector types that load one slot of them at once.
 template <typename T> struct PhaseRows;
@@ -598,48 +556,6 @@ gs_pipeline_kernel(const T* __restrict__ vals, const int* __restrict__ cols, lon
   }
 }
 
-// Fused residual + injection restriction (Sec. 3.2.4, last equation):
-// rc_I = r_{f_c(I)} - sum_j A_{f_c(I) j} z_j for every coarse point I.  The
-// coarse-coincident fine points are exactly fine colour block 7, stored in the
-// same lexicographic order as the coarse grid, so threads walk that block
-// contiguously and scatter into the coarse colour blocks.
-//
-// zc0 (optional): the coarse level's first forward sweep from zero starts
-// with colour 0, whose rows have no neighbour of a lower colour, so that
-// phase is z_I = rc_I / a_II; with zc0 set it is done here, for the coarse
-// points of colour 0, and the sweep skips the phase (same values).
-// 32 registers (8 CTAs per SM, a 128^3 level-0 restriction is one wave):
-// measured 0.15 % faster 128^3 solves than the 34-register build.
-template <typename T, int MODE>
-__global__ void __launch_bounds__(256, 8)
-restrict_kernel(const __grid_constant__ Geom gf, const __grid_constant__ Geom gc,
-                const T* __restrict__ vals, const int* __restrict__ cols,
-                const T* __restrict__ r, const T* __restrict__ z, T* __restrict__ rc,
-                T* __restrict__ zc0, const T* __restrict__ cdiag) {
-  pdl_trigger();
-  const int cx = gf.cdx[kCoarseColour], cy = gf.cdy[kCoarseColour];
-  const long long cnt = (long long)cx * cy * gf.cdz[kCoarseColour];
-  const long long ns = gf.n_store;
-  const long long p0 = blockIdx.x * (long long)blockDim.x;
-  pdl_wait();
-  const long long p = p0 + threadIdx.x;
-  if (p >= cnt) return;
-  const long long row = gf.off[kCoarseColour] + p;
-  T acc = ld_dep(r + row);
-#pragma unroll
-  for (int s = 0; s < kSlots; ++s) {
-    const T a = ld_mat<MODE>(vals + s * ns + row);
-    const int c = ld_mat<MODE>(cols + s * ns + row);
-    acc = fma(-a, ld_dep(z + c), acc);
-  }
-  const int I = (int)(p % cx);
-  const int J = (int)((p / cx) % cy);
-  const int K = (int)(p / ((long long)cx * cy));
-  const long long R = store_index(gc, I, J, K);
-  rc[R] = acc;
-  if (zc0 && colour_of(I, J, K) == 0) zc0[R] = acc / cdiag[R];
-}
-
 // Prolongation P = R^T and correction (Fig. 1, eq. (3) transposed):
 // z_{f_c(I)} += zc_I.
 template <typename T>
@@ -673,50 +589,10 @@ static int mat_mode(const Level& L) {
                                                                         : kMatResident;
 }
 
-template <typename T>
-static auto restrict_fn(const Level& L) -> decltype(&restrict_kernel<T, kMatStream>) {
-  switch (mat_mode(L)) {
-    case kMatStream: return restrict_kernel<T, kMatStream>;
-    case kMatCached: return restrict_kernel<T, kMatCached>;
-    default: return restrict_kernel<T, kMatResident>;
-  }
-}
-
-// Algorithmic DRAM bytes per row (ELL with 27 padded slots, int32 indices;
-// every vector entry read or written once).  sv / sx: value / vector bytes.
-static double bytes_spmv_row(double sv, double sx) { return 27.0 * (sv + 4.0) + 2.0 * sx; }
-// GS phase, per row reading k off-diagonal slots: k + 1 values, k indices
-// (the diagonal's is implied), r_i, the new x_i, and x gathered once (in
-// proportion to the slots read).
-static double bytes_restrict_row(double sv, double sx) { return 27.0 * (sv + 4.0) + 3.0 * sx; }
-
-template <typename T>
-static int spmv_t(hpg_problem* h, int level, const T* x, T* y, cudaStream_t s) {
-  const Level& L = h->lev[level];
-  const long long ns = L.g.n_store;
-  const T* vals = Prec<T>::vals(L);
-  return launch(h, K_SPMV, level, Prec<T>::idx == 0 ? HPG_FP64 : HPG_FP32,
-                L.n * bytes_spmv_row(sizeof(T), sizeof(T)), s, "spmv_kernel", [&] {
-                  return kl(h, spmv_kernel<T>, grid_for(ns, kThreads), kThreads, s, vals, L.cols,
-                            ns, x, y);
-                });
-}
-
 int launch_spmv(hpg_problem* h, int level, hpg_prec prec, const void* x, void* y,
                 cudaStream_t s) {
-  if (prec == HPG_FP64) return spmv_t<double>(h, level, (const double*)x, (double*)y, s);
-  return spmv_t<float>(h, level, (const float*)x, (float*)y, s);
-}
-
-int launch_residual64(hpg_problem* h, const double* b, const double* x, double* r,
-                      cudaStream_t s) {
-  const Level& L = h->lev[0];
-  const long long ns = L.g.n_store;
-  return launch(h, K_RESIDUAL, 0, HPG_FP64, L.n * (27.0 * 12.0 + 3.0 * 8.0), s,
-                "residual64_kernel", [&] {
-                  return kl(h, residual64_kernel, grid_for(ns, kThreads), kThreads, s, L.v64,
-                            L.cols, ns, b, x, r);
-                });
+  if (prec == HPG_FP64) return stencil_spmv(h, level, 1, (const double*)x, (double*)y, s);
+  return stencil_spmv(h, level, 1, (const float*)x, (float*)y, s);
 }
 
 // State of the sweeps on one level: the colour of the most recent phase when
@@ -1092,13 +968,7 @@ static int vcycle_t(hpg_problem* h, int l, const T* r, T* z, cudaStream_t s,
   const long long cnt = (long long)L.g.cdx[kCoarseColour] * L.g.cdy[kCoarseColour] *
                         L.g.cdz[kCoarseColour];
   const int prec = Prec<T>::idx == 0 ? HPG_FP64 : HPG_FP32;
-  const T* vals = Prec<T>::vals(L);
-  rc = launch(h, K_RESTRICT, l, prec, cnt * bytes_restrict_row(sizeof(T), sizeof(T)), s,
-              "restrict_kernel", [&] {
-                return kl(h, restrict_fn<T>(L), grid_for(cnt, kThreads), kThreads, s, L.g,
-                          C.g, vals, L.cols, r, z, rc_vec, fuse ? zc_vec : (T*)nullptr,
-                          Prec<T>::vals(C) + kCentre * C.g.n_store);
-              });
+  rc = stencil_restrict(h, l, 1, r, z, rc_vec, fuse ? zc_vec : (T*)nullptr, s);
   if (rc) return rc;
   if ((rc = vcycle_t<T>(h, l + 1, rc_vec, zc_vec, s, fuse))) return rc;
   rc = launch(h, K_PROLONG, l, prec, cnt * 3.0 * sizeof(T), s, "prolong_kernel", [&] {
@@ -1256,13 +1126,7 @@ static int vcycle_noalloc_t(hpg_problem* h, int l, const T* r, T* z, T* const* c
   const long long cnt = (long long)L.g.cdx[kCoarseColour] * L.g.cdy[kCoarseColour] *
                         L.g.cdz[kCoarseColour];
   const int prec = Prec<T>::idx == 0 ? HPG_FP64 : HPG_FP32;
-  const T* vals = Prec<T>::vals(L);
-  rc = launch(h, K_RESTRICT, l, prec, cnt * bytes_restrict_row(sizeof(T), sizeof(T)), s,
-              "restrict_kernel", [&] {
-                return kl(h, restrict_fn<T>(L), grid_for(cnt, kThreads), kThreads, s, L.g,
-                          C.g, vals, L.cols, r, z, rc_vec, fuse ? zc_vec : (T*)nullptr,
-                          Prec<T>::vals(C) + kCentre * C.g.n_store);
-              });
+  rc = stencil_restrict(h, l, 1, r, z, rc_vec, fuse ? zc_vec : (T*)nullptr, s);
   if (rc) return rc;
   if ((rc = vcycle_noalloc_t<T>(h, l + 1, rc_vec, zc_vec, crhs, csol, s, fuse))) return rc;
   rc = launch(h, K_PROLONG, l, prec, cnt * 3.0 * sizeof(T), s, "prolong_kernel", [&] {

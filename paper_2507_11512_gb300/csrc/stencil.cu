@@ -1,0 +1,151 @@
+// Products with the 27-point operator evaluated straight from the grid: SpMV
+// and the fused residual-restriction, for one right-hand side and for
+// R-vectors.
+//
+// See stencil.cuh for what they read and why their values equal the ELL
+// kernels' bit for bit.
+
+#include <algorithm>
+
+#include "stencil.cuh"
+
+namespace hpg {
+
+// ------------------------------------------------------------------ product
+// y = A x (Sec. 3.2.2).  Bound by the vectors' traffic (8 bytes per FP32 row)
+// on large grids, by latency on small ones; FP64 by the FP64 rate (27 FMAs a
+// row).  A thread takes a point pair of LINES consecutive x-lines, so that a
+// warp's loads run along x and neighbour lines are reused in registers.
+template <typename T, int LINES>
+__global__ void __launch_bounds__(256)
+stencil_spmv_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T> c,
+                    const __grid_constant__ RowPlan pl, const T* x, const T* diag, T* y) {
+  pdl_trigger();
+  pdl_wait();
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < pl.threads) {
+    const unsigned e = t % (unsigned)g.we, q = t / (unsigned)g.we;
+    const unsigned grp = q % pl.groups, k = q / pl.groups;
+    stencil_rows<T, 1, LINES>(g, c, x, diag, (int)e, (int)grp * LINES, (int)k,
+                              [](unsigned) { return T(0); },
+                              [&](unsigned p, T v) { y[p] = v; });
+  } else if (t - pl.threads < pl.pad) {
+    const unsigned p = pad_element(g, t - pl.threads);
+    y[p] = ld_dep(x + p);
+  }
+}
+
+RowPlan make_row_plan(const SGeom& g, int lines) {
+  RowPlan p;
+  p.lines = lines;
+  p.groups = (unsigned)((g.ny + lines - 1) / lines);
+  p.threads = (unsigned)g.we * p.groups * (unsigned)g.nz;
+  p.pad = 0;
+  for (int c = 0; c < kColours; ++c) p.pad += g.end[c] - g.off[c] - g.cnt[c];
+  return p;
+}
+
+template <typename T>
+static int spmv_t(hpg_problem* h, int level, int R, const T* x, T* y, cudaStream_t s,
+                  int block) {
+  const Level& L = h->lev[level];
+  const SGeom g = make_sgeom(L.g, R);
+  // four lines a thread once that leaves every SM several 256-thread blocks
+  const bool big = (long long)g.we * g.ny * g.nz >= (long long)kRowLines * 4 * 256 * h->num_sms;
+  const RowPlan pl = make_row_plan(g, big ? kRowLines : 1);
+  const T* diag = level_diag<T>(L);
+  const int grid = grid_for((long long)pl.threads + pl.pad, block);
+  return launch(h, K_SPMV, level, sizeof(T) == 8 ? HPG_FP64 : HPG_FP32,
+                (double)L.n * R * 2.0 * sizeof(T) + (diag ? L.n * (double)sizeof(T) : 0.0), s,
+                "stencil_spmv_kernel", [&] {
+                  return kl(h, big ? stencil_spmv_kernel<T, kRowLines>
+                                   : stencil_spmv_kernel<T, 1>,
+                            grid, block, s, g, make_coef<T>(h->beta), pl, x, diag, y);
+                });
+}
+int stencil_spmv(hpg_problem* h, int level, int R, const float* x, float* y, cudaStream_t s,
+                 int block) {
+  return spmv_t<float>(h, level, R, x, y, s, block);
+}
+int stencil_spmv(hpg_problem* h, int level, int R, const double* x, double* y, cudaStream_t s,
+                 int block) {
+  return spmv_t<double>(h, level, R, x, y, s, block);
+}
+
+// -------------------------------------------------------------- restriction
+// Fused residual + injection restriction (Sec. 3.2.4): rc_I = r_f - (A z)_f at
+// the fine points f = 2I, which are colour block 7 in the coarse grid's own
+// order.  One thread per coarse element; slot order as the product's.
+// zc0 (optional): the coarse level's first phase from zero on its colour-0
+// points, z_I = rc_I / a_II (see symgs).
+template <typename T>
+__global__ void __launch_bounds__(256)
+stencil_restrict_kernel(const __grid_constant__ SGeom gf, const __grid_constant__ Geom gc,
+                        const __grid_constant__ Coef<T> c, const T* r, const T* z,
+                        const T* fdiag, const T* cdiag, T* rc, T* zc0) {
+  pdl_trigger();
+  pdl_wait();
+  const unsigned p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= gf.cnt[kCoarseColour]) return;
+  const unsigned e = p % (unsigned)gf.we, q = p / (unsigned)gf.we;
+  const int J = (int)(q % (unsigned)gf.he), K = (int)(q / (unsigned)gf.he);
+  const unsigned row = gf.off[kCoarseColour] + p;
+  const int j = 2 * J, k = 2 * K;
+  T l[9], m[9], rr[9];
+#pragma unroll
+  for (int u = 0; u < 9; ++u) {
+    const int jj = j + u % 3 - 1, kk = k + u / 3 - 1;
+    l[u] = m[u] = rr[u] = T(0);
+    if ((unsigned)jj < (unsigned)gf.ny && (unsigned)kk < (unsigned)gf.nz) {
+      const T* od = z + line_base(gf, 1, jj, kk) + e;
+      m[u] = ld_dep(z + line_base(gf, 0, jj, kk) + e);
+      if ((int)e >= gf.R && (int)e - gf.R < gf.wo) l[u] = ld_dep(od - gf.R);
+      if ((int)e < gf.wo) rr[u] = ld_dep(od);
+    }
+  }
+  T acc = ld_dep(r + row);
+  const unsigned I = e / (unsigned)gf.R;
+  const T d = fdiag ? fdiag[row / (unsigned)gf.R] : (T)kDiag;
+#pragma unroll
+  for (int u = 0; u < 9; ++u) {
+    const int dyz = u % 3 - 1 + u / 3 - 1;
+    if (u == 4) {
+      acc = fma(-c.a[2], l[u], acc);
+      acc = fma(-d, m[u], acc);
+      acc = fma(-c.a[4], rr[u], acc);
+      if (on_boundary(gf, 2 * (int)I, j, k)) acc = fma(T(0), m[u], acc);
+    } else {
+      acc = line_sum<T, -1>(c, dyz, l[u], m[u], rr[u], acc);
+    }
+  }
+  const long long Rc = store_index(gc, (int)I, J, K);
+  rc[Rc * gf.R + (e - I * gf.R)] = acc;
+  if (zc0 && colour_of((int)I, J, K) == 0)
+    zc0[Rc * gf.R + (e - I * gf.R)] = acc / (cdiag ? cdiag[Rc] : (T)kDiag);
+}
+
+template <typename T>
+static int restrict_t(hpg_problem* h, int level, int R, const T* r, const T* z, T* rc, T* zc0,
+                      cudaStream_t s) {
+  const Level& L = h->lev[level];
+  const Level& C = h->lev[level + 1];
+  const SGeom g = make_sgeom(L.g, R);
+  const double cnt = (double)g.cnt[kCoarseColour];
+  // z is read once, r and rc once per coarse row
+  return launch(h, K_RESTRICT, level, sizeof(T) == 8 ? HPG_FP64 : HPG_FP32,
+                ((double)L.n * R + 2.0 * cnt) * sizeof(T), s, "stencil_restrict_kernel", [&] {
+                  return kl(h, stencil_restrict_kernel<T>, grid_for((long long)cnt, 256), 256, s,
+                            g, C.g, make_coef<T>(h->beta), r, z, level_diag<T>(L),
+                            level_diag<T>(C), rc, zc0);
+                });
+}
+int stencil_restrict(hpg_problem* h, int level, int R, const float* r, const float* z, float* rc,
+                     float* zc0, cudaStream_t s) {
+  return restrict_t<float>(h, level, R, r, z, rc, zc0, s);
+}
+int stencil_restrict(hpg_problem* h, int level, int R, const double* r, const double* z,
+                     double* rc, double* zc0, cudaStream_t s) {
+  return restrict_t<double>(h, level, R, r, z, rc, zc0, s);
+}
+
+}  // namespace hpg
