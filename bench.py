@@ -31,21 +31,17 @@ if ROOT not in sys.path:
 METRIC = "GMRES-IR GFLOP/s and time-to-1e-9 residual, MxP vs FP64, 1 GB300; % HBM peak"
 FALLBACK_HBM_GBS = 6800.0
 
-# DRAM bytes (read + write) per launch of the level-0 FP32 Gauss-Seidel phase
-# kernel at 128^3, from one ncu capture of that kernel, valid while the
-# kernel's source text (the kernel and the helpers it inlines) hashes to
-# `sources_sha256`.
-GS_TRAFFIC = {"workload": "mxp_gmres30_128cube", "bytes_per_launch": 65166976.0,
-              "sources_sha256": "d797e9973fb181b4d5383dbc69dd6b586e4b41f70cf2ba667a9760cb975d6a1a"}
+# DRAM bytes (read + write) per launch of the level-0 FP32 Gauss-Seidel plane
+# kernel at 128^3, from one ncu capture of that kernel (None: not captured),
+# valid while the kernel's source text (the kernel and the helpers it inlines)
+# hashes to `sources_sha256`.
+GS_TRAFFIC = {"workload": "mxp_gmres30_128cube", "bytes_per_launch": None,
+              "sources_sha256": "0" * 64}
 # (file, first line of the block, text that ends it): the kernel's source
 GS_KERNEL_TEXT = (
-    ("paper_2507_11512_gb300/csrc/sparse.cu", "template <typename T> struct PhaseRows;",
-     "// One Gauss-Seidel colour phase"),
-    ("paper_2507_11512_gb300/csrc/sparse.cu", "template <typename T, bool STREAM, int MC>",
-     "// The bandwidth-variant instantiation"),
-    ("paper_2507_11512_gb300/csrc/hpg_internal.cuh", "template <bool STREAM, typename V>", "\n}\n"),
-    ("paper_2507_11512_gb300/csrc/hpg_internal.cuh",
-     "__host__ __device__ constexpr unsigned gs_slot_mask", "\n}\n"),
+    ("paper_2507_11512_gb300/csrc/gs_planes.cu", "enum PlaneKind", "// Shared memory of a plane CTA"),
+    ("paper_2507_11512_gb300/csrc/stencil.cuh", "// First element of the x-line",
+     "// Whether a point touches"),
     ("paper_2507_11512_gb300/csrc/hpg_internal.cuh",
      "template <typename V>\n__device__ __forceinline__ V ld_dep", "\n}\n"),
 )
@@ -396,9 +392,11 @@ def run_gpu(args):
     gs_ms = sum(a.elapsed_time(c) for a, c in ev)
     del g_spmv, g_sweep
     cnt = info0["colour_count"]
-    gs_row_bytes = metrics.gs_row_bytes(4, 4)
-    gs_phases = 15
-    gs_bytes = (sum(cnt) + sum(cnt[:7])) * gs_row_bytes * gs_reps
+    # a sweep is 3 launches (odd planes, even planes, odd planes); each reads z
+    # once, and r and writes z on its half of the planes: 8 bytes a grid point
+    gs_launches = 3
+    gs_row_bytes = 8.0
+    gs_bytes = gs_launches * sum(cnt) * gs_row_bytes * gs_reps
     gs_gbs = gs_bytes / (gs_ms / 1e3) / 1e9
     traffic = gs_traffic(w.name)
     # the same kernel inside the profiled solve (event-bracketed launches)
@@ -410,17 +408,17 @@ def run_gpu(args):
     # graph-timed time per solve
     solve_bytes = sum(p["bytes"] for p in prof)
     solve_gbs = solve_bytes / (ms_max / args.steps / 1e3) / 1e9
-    roofline = {"bound": "hbm", "kernel": "gs_phase_kernel (level 0, fp32)",
+    roofline = {"bound": "hbm", "kernel": "gs_plane_kernel (level 0, fp32)",
                 "achieved": gs_gbs, "peak": peak, "unit": "GB/s", "frac": gs_gbs / peak,
                 "peak_source": peak_src,
                 "traffic": traffic,
-                "algorithmic_bytes_per_launch": gs_bytes / (gs_reps * gs_phases),
+                "algorithmic_bytes_per_launch": gs_bytes / (gs_reps * gs_launches),
                 "row_bytes": gs_row_bytes,
-                "launches": gs_reps * gs_phases,
-                "avg_launch_us": 1e3 * gs_ms / (gs_reps * gs_phases),
+                "launches": gs_reps * gs_launches,
+                "avg_launch_us": 1e3 * gs_ms / (gs_reps * gs_launches),
                 "timing": "CUDA events around each of %d graph-launched hpg_mg_smooth sweeps "
-                          "on level 0 (%d phase launches), a graph-launched level-0 SpMV "
-                          "between sweeps" % (gs_reps, gs_reps * gs_phases),
+                          "on level 0 (%d launches), a graph-launched level-0 SpMV "
+                          "between sweeps" % (gs_reps, gs_reps * gs_launches),
                 "in_solve": {"achieved": gs_in_solve,
                              "frac": gs_in_solve / peak if gs_in_solve else None,
                              "timing": "level-0 phases of one eager solve, each bracketed "

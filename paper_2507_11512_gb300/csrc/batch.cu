@@ -62,64 +62,6 @@ __device__ __forceinline__ void st_n(float* p, const float (&v)[N]) {
 }
 
 // ------------------------------------------------- multi-RHS stencil kernels
-// One Gauss-Seidel colour phase (Sec. 3.2.1) for R right-hand sides: rows
-// [row0, row0 + nrows) of one colour block; entries j >= valid_end read as
-// zero (first forward sweep from z = 0).  MC selects the slots loaded:
-// kAllSlots every slot; c = 0..7 the first forward sweep's phase of colour c
-// from z = 0 with its slot set (gs_slot_mask) fixed at compile time, so a
-// row's loads issue as one straight-line batch; kMaskSlots the same set
-// passed at run time in `mask` (the other slots are known zero and not
-// loaded).  MODE (MatLoad) is the level's matrix load policy: streamed
-// evict-first, cached, or evict-last for the small coarse levels.  Same slot
-// order and arithmetic per value as gs_phase_kernel.
-constexpr int kAllSlots = -1, kMaskSlots = -2;
-template <int R, int LPR, int MODE, int MC>
-__global__ void __launch_bounds__(256, 3)
-mgs_phase_kernel(const float* __restrict__ vals, const int* __restrict__ cols, long long ns,
-                 const float* __restrict__ rhs, float* z, long long row0, long long nrows,
-                 long long valid_end, unsigned mask) {
-  constexpr int RL = R / LPR;
-  constexpr unsigned kMask = MC >= 0 ? gs_slot_mask(MC, true) : (1u << kSlots) - 1u;
-  pdl_trigger();
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const long long lr = t / LPR;
-  const int lane = (int)(t % LPR);
-  if (lr >= nrows) return;
-  const long long row = row0 + lr;
-  // the row's matrix slots first, all at once (the matrix does not depend on
-  // earlier kernels, so these loads may overlap the previous phase), then the
-  // gathers slot by slot; the arithmetic is that of gs_phase_kernel
-  int col[kSlots];
-  float a[kSlots];
-#pragma unroll
-  for (int s = 0; s < kSlots; ++s) {
-    const bool use = ((kMask >> s) & 1u) && (MC != kMaskSlots || s == kCentre ||
-                                             ((mask >> s) & 1u));
-    col[s] = use && s != kCentre ? ld_mat<MODE>(cols + s * ns + row) : 0;
-    a[s] = use ? ld_mat<MODE>(vals + s * ns + row) : 0.0f;
-  }
-  pdl_wait();
-  float acc[RL];
-  ld_n<RL>(rhs + row * R + lane * RL, acc);
-#pragma unroll
-  for (int s = 0; s < kSlots; ++s) {
-    if (s == kCentre || !((kMask >> s) & 1u)) continue;
-    const bool use = MC != kMaskSlots || ((mask >> s) & 1u);
-    float xv[RL];
-    if (use && col[s] < valid_end) {
-      ld_n<RL>(z + (long long)col[s] * R + lane * RL, xv);
-    } else {
-#pragma unroll
-      for (int r = 0; r < RL; ++r) xv[r] = 0.0f;
-    }
-#pragma unroll
-    for (int r = 0; r < RL; ++r) acc[r] = fma(-a[s], xv[r], acc[r]);
-  }
-#pragma unroll
-  for (int r = 0; r < RL; ++r) acc[r] = acc[r] / a[kCentre];
-  st_n<RL>(z + row * R + lane * RL, acc);
-}
-
 // Prolongation and correction z_{f_c(I)} += zc_I (eq. (3) transposed).
 template <int R>
 __global__ void __launch_bounds__(256)
@@ -294,128 +236,6 @@ static Shape shape_of(hpg_problem* h, int level, int kind, int R) {
   return sh;
 }
 
-// Load policy of a level's matrix (as in sparse.cu): streamed evict-first
-// where the FP32 ELL arrays exceed the streaming size, evict-last where they
-// are small (coarse levels read by every V-cycle), cached otherwise.
-static int mmat_mode(const Level& L) {
-  const long long b = L.g.n_store * 27LL * 8;
-  return b > kStreamMatrixBytes ? kMatStream : b > kResidentMatrixBytes ? kMatCached
-                                                                        : kMatResident;
-}
-
-template <int R, int LPR, int MODE, int MC>
-static cudaError_t mgs_kl(hpg_problem* h, int grid, int block, cudaStream_t s, const float* vals,
-                          const int* cols, long long ns, const float* rhs, float* z,
-                          long long row0, long long nrows, long long valid_end, unsigned mask) {
-  return kl(h, mgs_phase_kernel<R, LPR, MODE, MC>, grid, block, s, vals, cols, ns, rhs, z, row0,
-            nrows, valid_end, mask);
-}
-
-// Colour c of the first sweep from zero with its compile-time slot set.
-template <int R, int MODE>
-static cudaError_t mgs_colour(hpg_problem* h, int c, int grid, int block, cudaStream_t s,
-                              const float* vals, const int* cols, long long ns,
-                              const float* rhs, float* z, long long row0, long long nrows,
-                              long long valid_end, unsigned mask) {
-  switch (c) {
-#define HPG_MGS_CASE(C)                                                                   \
-  case C:                                                                                 \
-    return mgs_kl<R, 1, MODE, C>(h, grid, block, s, vals, cols, ns, rhs, z, row0, nrows, \
-                                 valid_end, mask);
-    HPG_MGS_CASE(0) HPG_MGS_CASE(1) HPG_MGS_CASE(2) HPG_MGS_CASE(3)
-    HPG_MGS_CASE(4) HPG_MGS_CASE(5) HPG_MGS_CASE(6) HPG_MGS_CASE(7)
-#undef HPG_MGS_CASE
-  }
-  return cudaErrorInvalidValue;
-}
-
-template <int R, int LPR, int MODE>
-static cudaError_t mgs_launch(hpg_problem* h, int c, bool masked, int grid, int block,
-                              cudaStream_t s, const float* vals, const int* cols, long long ns,
-                              const float* rhs, float* z, long long row0, long long nrows,
-                              long long valid_end, unsigned mask) {
-  if (!masked)
-    return mgs_kl<R, LPR, MODE, kAllSlots>(h, grid, block, s, vals, cols, ns, rhs, z, row0,
-                                           nrows, valid_end, mask);
-  if constexpr (LPR == 1)
-    return mgs_colour<R, MODE>(h, c, grid, block, s, vals, cols, ns, rhs, z, row0, nrows,
-                               valid_end, mask);
-  return mgs_kl<R, LPR, MODE, kMaskSlots>(h, grid, block, s, vals, cols, ns, rhs, z, row0, nrows,
-                                          valid_end, mask);
-}
-
-template <int R, int LPR>
-static cudaError_t mgs_mode(hpg_problem* h, int mode, int c, bool masked, int grid, int block,
-                            cudaStream_t s, const float* vals, const int* cols, long long ns,
-                            const float* rhs, float* z, long long row0, long long nrows,
-                            long long valid_end, unsigned mask) {
-  if (mode == kMatStream)
-    return mgs_launch<R, LPR, kMatStream>(h, c, masked, grid, block, s, vals, cols, ns, rhs, z,
-                                          row0, nrows, valid_end, mask);
-  if (mode == kMatResident)
-    return mgs_launch<R, LPR, kMatResident>(h, c, masked, grid, block, s, vals, cols, ns, rhs,
-                                            z, row0, nrows, valid_end, mask);
-  return mgs_launch<R, LPR, kMatCached>(h, c, masked, grid, block, s, vals, cols, ns, rhs, z,
-                                        row0, nrows, valid_end, mask);
-}
-
-template <int R>
-static cudaError_t mgs_dispatch(hpg_problem* h, int lpr, int mode, int c, bool masked,
-                                long long nrows, int block, cudaStream_t s, const float* vals,
-                                const int* cols, long long ns, const float* rhs, float* z,
-                                long long row0, long long valid_end, unsigned mask) {
-  constexpr int L2 = R >= 2 ? 2 : 1;
-  const int grid = grid_for(nrows * lpr, block);
-  if (lpr == 1)
-    return mgs_mode<R, 1>(h, mode, c, masked, grid, block, s, vals, cols, ns, rhs, z, row0,
-                          nrows, valid_end, mask);
-  if (lpr == 2)
-    return mgs_mode<R, L2>(h, mode, c, masked, grid, block, s, vals, cols, ns, rhs, z, row0,
-                           nrows, valid_end, mask);
-  return mgs_mode<R, R>(h, mode, c, masked, grid, block, s, vals, cols, ns, rhs, z, row0, nrows,
-                        valid_end, mask);
-}
-
-struct BSweep {
-  int last = -1;   // colour of the latest phase on unchanged data (skipped if repeated)
-};
-
-template <int R>
-static int mgs_phase(hpg_problem* h, int level, const float* rhs, float* z, int c,
-                     bool from_zero, BSweep& sw, cudaStream_t s) {
-  if (sw.last == c) return HPG_OK;
-  const Level& L = h->lev[level];
-  const long long row0 = L.g.off[c];
-  const long long nrows = L.g.off[c + 1] - row0;
-  sw.last = c;
-  if (nrows == 0) return HPG_OK;
-  const long long valid_end = from_zero ? row0 : L.g.n_store;
-  const unsigned mask = gs_slot_mask(c, from_zero);
-  const int nslots = __builtin_popcount(mask) - 1;
-  const double row_bytes = (nslots + 1.0) * 4 + nslots * 4.0 + R * (2.0 + nslots / 26.0) * 4;
-  const Shape sh = shape_of(h, level, kShapeGs, R);
-  return launch(h, K_GS, level, HPG_FP32, L.cnt[c] * row_bytes, s, "mgs_phase_kernel", [&] {
-    // phases of up to HPG_OPT_PDL_ROWS rows (none of a streamed level by
-    // default) are launched programmatically; measured on GB300, launching
-    // the 110,592-row phases of a 96^3 system so as well (triggering at
-    // block exit) made its 8-RHS solve 72.6 instead of 70.9 ms
-    if (nrows > h->pdl_rows) h->pdl_next = false;
-    return mgs_dispatch<R>(h, sh.lpr, mmat_mode(L), c, from_zero, nrows, sh.block, s, L.v32,
-                           L.cols, L.g.n_store, rhs, z, row0, valid_end, mask);
-  });
-}
-
-template <int R>
-static int msymgs(hpg_problem* h, int level, const float* rhs, float* z, bool from_zero,
-                  BSweep& sw, cudaStream_t s) {
-  int rc;
-  for (int c = 0; c < kColours; ++c)
-    if ((rc = mgs_phase<R>(h, level, rhs, z, c, from_zero, sw, s))) return rc;
-  for (int c = kColours - 1; c >= 0; --c)
-    if ((rc = mgs_phase<R>(h, level, rhs, z, c, false, sw, s))) return rc;
-  return HPG_OK;
-}
-
 // Y = A X on R-vectors; the tuned shape's block size, lanes per row do not apply.
 static int run_mspmv(hpg_problem* h, int R, int level, const float* x, float* y,
                      cudaStream_t s) {
@@ -428,15 +248,14 @@ template <int R>
 static int mvcycle_t(hpg_problem* h, int l, const float* rhs, float* z, cudaStream_t s) {
   const Level& L = h->lev[l];
   BatchSpace* bs = h->batch;
-  BSweep sw;
   int rc;
-  if (l == h->nlev - 1) return msymgs<R>(h, l, rhs, z, true, sw, s);
+  if (l == h->nlev - 1) return stencil_symgs(h, l, R, rhs, z, true, false, s);
   if (h->pre == 0) {
     HPG_CK(cudaMemsetAsync(z, 0, sizeof(float) * L.g.n_store * R, s));
     h->pdl_next = false;
   }
   for (int it = 0; it < h->pre; ++it)
-    if ((rc = msymgs<R>(h, l, rhs, z, it == 0, sw, s))) return rc;
+    if ((rc = stencil_symgs(h, l, R, rhs, z, it == 0, it > 0, s))) return rc;
   const Level& C = h->lev[l + 1];
   float* rcv = bs->rc[l + 1];
   float* zcv = bs->zc[l + 1];
@@ -449,9 +268,8 @@ static int mvcycle_t(hpg_problem* h, int l, const float* rhs, float* z, cudaStre
     return kl(h, mprolong_kernel<R>, grid_for(cnt, 256), 256, s, L.g, C.g, (const float*)zcv, z);
   });
   if (rc) return rc;
-  sw.last = -1;
   for (int it = 0; it < h->post; ++it)
-    if ((rc = msymgs<R>(h, l, rhs, z, false, sw, s))) return rc;
+    if ((rc = stencil_symgs(h, l, R, rhs, z, false, it > 0, s))) return rc;
   return HPG_OK;
 }
 
@@ -1440,8 +1258,7 @@ static int tune_t(hpg_problem* h, int reps, cudaStream_t s) {
           for (int it = 0; it <= reps && rc == HPG_OK; ++it) {
             if (it == 1 && cudaEventRecord(e0, s) != cudaSuccess) rc = HPG_ERR_CUDA;
             h->pdl_next = false;
-            BSweep sw;
-            rc = kind == kShapeGs ? msymgs<R>(h, l, a, b, false, sw, s)
+            rc = kind == kShapeGs ? stencil_symgs(h, l, R, a, b, false, false, s)
                                   : run_mspmv(h, R, l, a, b, s);
           }
           if (rc) break;

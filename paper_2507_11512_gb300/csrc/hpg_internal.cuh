@@ -244,6 +244,7 @@ struct Level {
   int* pipe_flags = nullptr;
   unsigned* pipe_sync = nullptr;
   int pipe_tiles = 0;
+  bool stalled = false;   // hpg_inject_stall: FP64 sweeps go through the pipelined kernel
 };
 
 constexpr int kPipeTileRows = 256;   // rows of one tile (= threads of its CTA)
@@ -286,7 +287,7 @@ struct hpg_problem {
   long long pdl_rows = 16384;     // latency-variant GS phases launched programmatically up
                                   // to this many rows
   int gs_pipeline = 1;            // pipelined sweep kernel: 0 never; on streamed levels
-                                  // 1 FP64 sweeps only (measured faster there), 2 always;
+                                  // 1 FP64 sweeps after hpg_inject_stall, 2 always;
                                   // 3 every level
   unsigned* pipe_err = nullptr;   // device word: a pipelined sweep's wait ran out
   int vc_cluster[2] = {0, 0};     // its cluster size per precision (0: not probed, <0: none)
@@ -298,7 +299,7 @@ namespace hpg {
 // its stream; prof_begin returns a slot (or -1 when disabled).
 int prof_begin(hpg_problem* h, cudaStream_t s);
 void prof_end(hpg_problem* h, int slot, int cls, int level, int prec, double bytes,
-              cudaStream_t s);
+              cudaStream_t s, int phases);
 void destroy_profiler(hpg_problem* h);
 
 // Enqueues kernel<<<grid, block, 0, s>>>(args...), with the programmatic
@@ -323,15 +324,16 @@ cudaError_t kl(hpg_problem* h, void (*kern)(KArgs...), int grid, int block, cuda
 }
 
 // Launches `f` (a lambda that enqueues one kernel with kl), counts it,
-// profiles it with its algorithmic DRAM bytes, and checks the launch.
+// profiles it with its algorithmic DRAM bytes, and checks the launch.  phases:
+// the colour phases it runs (what the profile counts).
 template <typename F>
 int launch(hpg_problem* h, int cls, int level, int prec, double bytes, cudaStream_t s,
-           const char* what, F&& f) {
+           const char* what, F&& f, int phases = 1) {
   const int slot = prof_begin(h, s);
   if (slot >= 0) h->pdl_next = false;
   const cudaError_t e0 = f();
   const cudaError_t e = e0 != cudaSuccess ? e0 : cudaGetLastError();
-  prof_end(h, slot, cls, level, prec, bytes, s);
+  prof_end(h, slot, cls, level, prec, bytes, s, phases);
   h->launches++;
   h->pdl_next = true;
   if (e != cudaSuccess) return cuda_fail(e, what, __FILE__, __LINE__);

@@ -222,6 +222,7 @@ static void free_level(Level& L, bool keep_matrix) {
   L.pipe_flags = nullptr;
   L.pipe_sync = nullptr;
   L.pipe_tiles = 0;
+  L.stalled = false;
   if (!keep_matrix) {
     dev_free(L.cols);
     dev_free(L.v32);
@@ -541,6 +542,10 @@ HPG_API int hpg_inject_stall(hpg_problem_t* h, int level, int tiles) {
   }
   const unsigned v = (unsigned)tiles;
   HPG_CK(cudaMemcpy(h->lev[level].pipe_sync + kPipeQueue, &v, sizeof(v), cudaMemcpyHostToDevice));
+  if (!h->lev[level].stalled) {
+    h->lev[level].stalled = true;
+    if (h->ws) destroy_workspace(h);   // a captured graph holds the plain sweeps
+  }
   return HPG_OK;
 }
 

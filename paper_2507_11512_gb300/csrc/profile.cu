@@ -17,6 +17,7 @@ namespace hpg {
 struct ProfRec {
   int cls, level, prec;
   double bytes;
+  int phases;
   int ev;   // index of the start event; ev + 1 is the stop event
 };
 
@@ -52,11 +53,11 @@ int prof_begin(hpg_problem* h, cudaStream_t s) {
 }
 
 void prof_end(hpg_problem* h, int slot, int cls, int level, int prec, double bytes,
-              cudaStream_t s) {
+              cudaStream_t s, int phases) {
   if (slot < 0) return;
   Profiler* p = h->prof;
   cudaEventRecord(p->events[slot + 1], s);
-  p->recs.push_back(ProfRec{cls, level, prec, bytes, slot});
+  p->recs.push_back(ProfRec{cls, level, prec, bytes, phases, slot});
 }
 
 void destroy_profiler(hpg_problem* h) {
@@ -103,7 +104,7 @@ HPG_API int hpg_profile_report(hpg_problem_t* h, hpg_kernel_stat* out, int capac
     st.name = kernel_class_name(r.cls);
     st.level = r.level;
     st.prec = r.prec;
-    st.launches += 1;
+    st.launches += r.phases;
     st.total_ms += ms;
     st.bytes += r.bytes;
   }

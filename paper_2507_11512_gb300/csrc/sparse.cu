@@ -30,132 +30,6 @@ template <> struct Prec<double> {
 };
 
 // ------------------------------------------------------------------ kernels
-// Rows a thread of a bandwidth-variant Gauss-Seidel phase takes, and the
-// 16-byte vector types that load one slot of them at once.
-template <typename T> struct PhaseRows;
-template <> struct PhaseRows<float> {
-  static constexpr int R = 4;
-  using V = float4;
-  using I = int4;
-};
-template <> struct PhaseRows<double> {
-  static constexpr int R = 2;
-  using V = double2;
-  using I = int2;
-};
-__device__ __forceinline__ void split_rows(const float4& v, float (&o)[4]) {
-  o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
-}
-__device__ __forceinline__ void split_rows(const double2& v, double (&o)[2]) {
-  o[0] = v.x; o[1] = v.y;
-}
-__device__ __forceinline__ float4 join_rows(const float (&o)[4]) {
-  return make_float4(o[0], o[1], o[2], o[3]);
-}
-__device__ __forceinline__ double2 join_rows(const double (&o)[2]) {
-  return make_double2(o[0], o[1]);
-}
-__device__ __forceinline__ void split_rows(const int4& v, int (&o)[4]) {
-  o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
-}
-__device__ __forceinline__ void split_rows(const int2& v, int (&o)[2]) {
-  o[0] = v.x; o[1] = v.y;
-}
-
-// One Gauss-Seidel colour phase (Sec. 3.2.1, relaxation form of eq. (1)):
-// for every row i of the colour block [row0, row0 + nrows),
-//   x_i <- (r_i - sum_{j != i} a_ij x_j) / a_ii.
-// The block is an independent set, so no row reads a value written by this
-// launch.  Entries x_j with j >= valid_end read as zero: the first forward
-// sweep from z = 0 passes valid_end = start of the current colour block, so
-// that colours not yet visited count as zero without a memset.
-//
-// Bandwidth variant, for levels whose matrix streams from HBM: a thread takes
-// PhaseRows<T>::R consecutive rows and loads each slot's values and indices
-// for them as one 16-byte vector (the colour blocks start and end on 32-row
-// boundaries, so the rows divide evenly and the loads are aligned), and r
-// and x likewise: the launcher sends vectors off a 16-byte boundary (caller
-// pointers) to the one-row-per-thread latency kernel instead, whose per-row
-// arithmetic is the same (a branch on the alignment inside this kernel cost
-// 1 %).  Each row's
-// arithmetic is the one-row-per-thread kernel's, in the same order.  Two
-// 256-thread CTAs per SM with 128 registers, so a thread has its rows' loads
-// in flight at once (a 128^3 FP32 phase is 256 CTAs, one wave).  Measured on
-// GB300 against one row per thread in 32 registers (8 CTAs per SM): level-0
-// phase 10.72 -> 9.35 us, 128^3 solve 102.8 -> 97.4 ms, 320^3 3534 ->
-// 3401 ms; 2 rows per thread in 64 registers 99.7 ms, 4 rows in 64 or 80
-// registers 103.0 / 101.9 ms, 4 rows in 128-thread CTAs 97.7 ms.  The
-// matrix is read evict-first.  No early trigger and no load before the
-// programmatic wait: measured on GB300, letting the next phase's CTAs start
-// early (or prefetching its slots into L2) slows this bandwidth-bound chain
-// down; launched with the programmatic attribute but triggering only as its
-// blocks exit, the next launch is prepared while a phase drains (faster).
-//
-// MC = -1 reads every slot.  MC = c (0..7) is the phase of colour c in the
-// first forward sweep from z = 0: only the slots whose neighbour colour is
-// below c are loaded (the others multiply zeros), and the set is fixed at
-// compile time, so the loads of a row issue as one straight-line batch.  A
-// run-time slot mask made these phases no faster than full ones on GB300
-// (colour 0, which loads only the diagonal, took 70 % of a full phase).
-template <typename T, bool STREAM, int MC>
-__global__ void __launch_bounds__(256, 2)
-gs_phase_kernel(const T* __restrict__ vals, const int* __restrict__ cols, long long ns,
-                const T* __restrict__ r, T* x, long long row0, long long nrows,
-                long long valid_end) {
-  constexpr unsigned kMask = MC < 0 ? (1u << kSlots) - 1u : gs_slot_mask(MC, true);
-  constexpr int NR = PhaseRows<T>::R;
-  using V = typename PhaseRows<T>::V;
-  using I = typename PhaseRows<T>::I;
-  pdl_wait();
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (NR * t >= nrows) return;
-  const long long row = row0 + NR * t;
-  T acc[NR];
-  split_rows(ld_dep(reinterpret_cast<const V*>(r + row)), acc);
-#pragma unroll
-  for (int s = 0; s < kSlots; ++s) {
-    if (s == kCentre || !((kMask >> s) & 1u)) continue;
-    T a[NR];
-    int c[NR];
-    split_rows(ld_matrix<STREAM>(reinterpret_cast<const V*>(vals + s * ns + row)), a);
-    split_rows(ld_matrix<STREAM>(reinterpret_cast<const I*>(cols + s * ns + row)), c);
-#pragma unroll
-    for (int q = 0; q < NR; ++q) {
-      const T xv = (c[q] < valid_end) ? ld_dep(x + c[q]) : T(0);
-      acc[q] = fma(-a[q], xv, acc[q]);
-    }
-  }
-  T diag[NR];
-  split_rows(ld_matrix<STREAM>(reinterpret_cast<const V*>(vals + kCentre * ns + row)), diag);
-#pragma unroll
-  for (int q = 0; q < NR; ++q) acc[q] = acc[q] / diag[q];
-  *reinterpret_cast<V*>(x + row) = join_rows(acc);
-}
-
-// The bandwidth-variant instantiation of a phase of colour c.
-template <typename T, bool STREAM>
-using GsPhaseFn = void (*)(const T*, const int*, long long, const T*, T*, long long, long long,
-                           long long);
-template <typename T, bool STREAM>
-static GsPhaseFn<T, STREAM> gs_phase_fn(int c, bool from_zero) {
-  if (!from_zero) return gs_phase_kernel<T, STREAM, -1>;
-  switch (c) {
-    case 0: return gs_phase_kernel<T, STREAM, 0>;
-    case 1: return gs_phase_kernel<T, STREAM, 1>;
-    case 2: return gs_phase_kernel<T, STREAM, 2>;
-    case 3: return gs_phase_kernel<T, STREAM, 3>;
-    case 4: return gs_phase_kernel<T, STREAM, 4>;
-    case 5: return gs_phase_kernel<T, STREAM, 5>;
-    case 6: return gs_phase_kernel<T, STREAM, 6>;
-    default: return gs_phase_kernel<T, STREAM, 7>;
-  }
-}
-
-// A colour block's rows (a multiple of kRowAlign) split evenly into the
-// bandwidth-variant phase's rows per thread.
-static_assert(kRowAlign % PhaseRows<float>::R == 0 && kRowAlign % PhaseRows<double>::R == 0,
-              "colour blocks must split evenly into a thread's rows");
-
 // TMA-tiled variant of the streamed phase (option HPG_OPT_GS_HALO): a CTA
 // takes whole x-lines of its colour block -- lines J0 .. J0+L-1 of plane K --
 // and moves everything its rows read into shared memory with 1-D bulk
@@ -315,90 +189,13 @@ gs_phase_halo_kernel(const T* __restrict__ vals, const int* __restrict__ cols, l
   T acc = sr[e];
 #pragma unroll
   for (int q = 0; q < kSlots; ++q) {
-    if (q == kCentre) continue;
-    const unsigned idx = (unsigned)(sc[q * rpad + e] + sdelta[q]);
+    const int s = gs_order(q);
+    if (s == kCentre) continue;
+    const unsigned idx = (unsigned)(sc[s * rpad + e] + sdelta[s]);
     const T xv = idx < nsm ? sx[idx] : T(0);
-    acc = fma(-sv[q * rpad + e], xv, acc);
+    acc = fma(-sv[s * rpad + e], xv, acc);
   }
   x[row0 + t] = acc / sv[kCentre * rpad + e];
-}
-
-// Threads per CTA of the latency variant; measured on GB300 at 128^3, the
-// FP32 solve took 106.6 / 106.1 / 106.0 / 105.0 / 109.0 ms with 32 / 64 / 128
-// / 256 / 512, while the FP64 solve was 3 % slower with 256 than with 64.
-template <typename T>
-__host__ __device__ constexpr int small_threads() {
-  return sizeof(T) == 4 ? 256 : 64;
-}
-
-// Latency variant, for coarse levels (matrix resident in L2, at most a few
-// tens of thousands of rows per phase): one row per thread, small_threads<T>()
-// per CTA, and each thread loads its row's 27 indices and values *before* the
-// programmatic wait -- the matrix does not depend on earlier kernels -- so that
-// latency overlaps the previous phase; after the wait it issues all the
-// gathers of x at once.  Same slot order and arithmetic as gs_phase_kernel.
-// early != 0: the next kernel may launch as soon as this one starts (the
-// small phases of levels 2-3; without it the 128^3 solve took 145.8 instead
-// of 102.9 ms); 0: only as this one's blocks exit (the 32768-row level-1
-// phases: 102.9 -> 102.3 ms, while an early trigger there made it 105.6 ms).
-// MODE (MatLoad): kMatCached, or kMatResident for the small levels whose
-// matrix is kept in L2 evict-last.  MC as in gs_phase_kernel: -1 all slots,
-// c the first forward sweep's colour c (slots with a later neighbour colour
-// are neither loaded nor gathered).
-template <typename T, int MODE, int MC>
-__global__ void __launch_bounds__(small_threads<T>())
-gs_phase_small_kernel(const T* __restrict__ vals, const int* __restrict__ cols, long long ns,
-                      const T* __restrict__ r, T* x, long long row0, long long nrows,
-                      long long valid_end, int early) {
-  constexpr unsigned kMask = MC < 0 ? (1u << kSlots) - 1u : gs_slot_mask(MC, true);
-  if (early) pdl_trigger();
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const bool live = t < nrows;
-  const long long row = row0 + (live ? t : 0);
-  int col[kSlots];
-  T a[kSlots];
-#pragma unroll
-  for (int s = 0; s < kSlots; ++s) {
-    const bool use = live && ((kMask >> s) & 1u);
-    col[s] = use ? ld_mat<MODE>(cols + s * ns + row) : 0;
-    a[s] = use ? ld_mat<MODE>(vals + s * ns + row) : T(1);
-  }
-  pdl_wait();
-  if (!live) return;
-  T xv[kSlots];
-#pragma unroll
-  for (int s = 0; s < kSlots; ++s)
-    xv[s] = (s != kCentre && ((kMask >> s) & 1u) && col[s] < valid_end) ? ld_dep(x + col[s])
-                                                                        : T(0);
-  T acc = ld_dep(r + row);
-#pragma unroll
-  for (int s = 0; s < kSlots; ++s)
-    if (s != kCentre && ((kMask >> s) & 1u)) acc = fma(-a[s], xv[s], acc);
-  x[row] = acc / a[kCentre];
-}
-
-// The latency-variant instantiation of a phase of colour c.
-template <typename T>
-using GsSmallFn = void (*)(const T*, const int*, long long, const T*, T*, long long, long long,
-                           long long, int);
-template <typename T, int MODE>
-static GsSmallFn<T> gs_small_fn_mode(int c, bool from_zero) {
-  if (!from_zero) return gs_phase_small_kernel<T, MODE, -1>;
-  switch (c) {
-    case 0: return gs_phase_small_kernel<T, MODE, 0>;
-    case 1: return gs_phase_small_kernel<T, MODE, 1>;
-    case 2: return gs_phase_small_kernel<T, MODE, 2>;
-    case 3: return gs_phase_small_kernel<T, MODE, 3>;
-    case 4: return gs_phase_small_kernel<T, MODE, 4>;
-    case 5: return gs_phase_small_kernel<T, MODE, 5>;
-    case 6: return gs_phase_small_kernel<T, MODE, 6>;
-    default: return gs_phase_small_kernel<T, MODE, 7>;
-  }
-}
-template <typename T>
-static GsSmallFn<T> gs_small_fn(int mode, int c, bool from_zero) {
-  return mode == kMatResident ? gs_small_fn_mode<T, kMatResident>(c, from_zero)
-                              : gs_small_fn_mode<T, kMatCached>(c, from_zero);
 }
 
 // ---------------------------------------------- pipelined symmetric sweep
@@ -451,7 +248,8 @@ __device__ __forceinline__ void pipe_row(const T* __restrict__ vals, const int* 
                                          long long row, long long valid_end, unsigned mask) {
   T acc = ld_dep(r + row);
 #pragma unroll
-  for (int s = 0; s < kSlots; ++s) {
+  for (int q = 0; q < kSlots; ++q) {
+    const int s = gs_order(q);
     if (s == kCentre) continue;
     if (MASKED) {
       const bool use = (mask >> s) & 1u;
@@ -621,24 +419,27 @@ static size_t halo_smem_bytes(const Geom& g, int c, int L) {
   return bytes + elems * sizeof(T);
 }
 
-// Launches the TMA-tiled phase when it applies (option set, FP32, whole lines
-// fit a CTA, r and z 16-byte aligned); returns false to use gs_phase_kernel.
-template <typename T, bool STREAM>
-static bool launch_gs_halo(hpg_problem* h, const Level& L, const T* r, T* z, int c,
-                           cudaStream_t s, cudaError_t* e) {
-  if constexpr (sizeof(T) != 4) {
-    return false;
-  } else {
-  if (!h->gs_halo || (((uintptr_t)z | (uintptr_t)r) & 15u) != 0) return false;
+// Whether the TMA-tiled phase applies (option set, FP32, whole lines fit a CTA,
+// r and z 16-byte aligned).
+template <typename T>
+static bool halo_fits(hpg_problem* h, const Level& L, const T* r, const T* z, int c) {
+  if (sizeof(T) != 4 || !h->gs_halo || (((uintptr_t)z | (uintptr_t)r) & 15u) != 0) return false;
   const int lines = halo_lines(L.g.cdx[c]);
-  if (lines < 1 || L.cnt[c] == 0) return false;
+  return lines >= 1 && halo_smem_bytes<T>(L.g, c, lines) <= (160u << 10);
+}
+
+template <typename T, bool STREAM>
+static cudaError_t launch_gs_halo(hpg_problem* h, const Level& L, const T* r, T* z, int c,
+                                  cudaStream_t s) {
+  if constexpr (sizeof(T) != 4) {
+    return cudaErrorInvalidValue;
+  } else {
+  const int lines = halo_lines(L.g.cdx[c]);
   const size_t smem = halo_smem_bytes<T>(L.g, c, lines);
-  if (smem > (160u << 10)) return false;
-  if (smem > (48u << 10) &&
-      cudaFuncSetAttribute(gs_phase_halo_kernel<T, STREAM>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, 160 << 10) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
+  if (smem > (48u << 10)) {
+    const cudaError_t e = cudaFuncSetAttribute(
+        gs_phase_halo_kernel<T, STREAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 << 10);
+    if (e != cudaSuccess) return e;
   }
   const int threads = (lines * L.g.cdx[c] + 31) / 32 * 32;
   const int grid = L.g.cdz[c] * ((L.g.cdy[c] + lines - 1) / lines);
@@ -647,61 +448,27 @@ static bool launch_gs_halo(hpg_problem* h, const Level& L, const T* r, T* z, int
   cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  *e = cudaLaunchKernelEx(&cfg, gs_phase_halo_kernel<T, STREAM>, Prec<T>::vals(L),
-                          (const int*)L.cols, L.g.n_store, r, z, L.g, c, lines, h->pipe_err);
-  return true;
+  return cudaLaunchKernelEx(&cfg, gs_phase_halo_kernel<T, STREAM>, Prec<T>::vals(L),
+                            (const int*)L.cols, L.g.n_store, r, z, L.g, c, lines, h->pipe_err);
   }
 }
 
+// One colour phase: TMA-tiled where the option asks for it, otherwise straight
+// from the grid.
 template <typename T>
 static int gs_phase(hpg_problem* h, int level, const T* r, T* z, int c, bool from_zero,
                     SweepState& st, cudaStream_t s, bool keep = false) {
   if (st.last == c) return HPG_OK;
   const Level& L = h->lev[level];
-  const long long row0 = L.g.off[c];
-  const long long nrows = L.g.off[c + 1] - row0;
   st.last = c;
-  if (nrows == 0) return HPG_OK;
-  const long long valid_end = from_zero ? row0 : L.g.n_store;
-  const T* vals = Prec<T>::vals(L);
-  const int nslots = __builtin_popcount(gs_slot_mask(c, from_zero)) - 1;   // off-diagonal
-  const double row_bytes =
-      (nslots + 1.0) * sizeof(T) + nslots * 4.0 + (2.0 + nslots / 26.0) * sizeof(T);
-  return launch(h, K_GS, level, Prec<T>::idx == 0 ? HPG_FP64 : HPG_FP32, L.cnt[c] * row_bytes, s,
-                "gs_phase_kernel", [&] {
-                  if (L.g.n_store * 27LL * 8 > kStreamMatrixBytes) {
-                    // launched programmatically after a kernel of the chain, but the
-                    // phase never triggers early and waits before its first load
-                    // (see gs_phase_kernel): the next phase's launch is set up while
-                    // this one drains; measured 103.6 -> 102.9 ms at 128^3
-                    if (((uintptr_t)r | (uintptr_t)z) & 15u)   // see gs_phase_kernel
-                      return kl(h, gs_small_fn<T>(kMatCached, c, from_zero),
-                                grid_for(nrows, small_threads<T>()), small_threads<T>(), s,
-                                vals, L.cols, L.g.n_store, r, z, row0, nrows, valid_end, 0);
-                    cudaError_t he = cudaSuccess;
-                    if (!from_zero &&
-                        (keep ? launch_gs_halo<T, false>(h, L, r, z, c, s, &he)
-                              : launch_gs_halo<T, true>(h, L, r, z, c, s, &he)))
-                      return he;
-                    if (keep)   // slice read again soon after: leave it in L2
-                      return kl(h, gs_phase_fn<T, false>(c, from_zero),
-                                grid_for(nrows / PhaseRows<T>::R, kThreads), kThreads, s,
-                                vals, L.cols, L.g.n_store, r, z, row0, nrows, valid_end);
-                    return kl(h, gs_phase_fn<T, true>(c, from_zero),
-                              grid_for(nrows / PhaseRows<T>::R, kThreads), kThreads, s, vals,
-                              L.cols, L.g.n_store, r, z, row0, nrows, valid_end);
-                  }
-                  // measured on GB300: programmatic overlap helps the smallest
-                  // phases and slows phases of tens of thousands of rows (with
-                  // the 32768-row level-1 phases overlapped too, the 128^3
-                  // solve took 110.3 ms instead of 107.4)
-                  const int early = nrows > h->pdl_rows ? 0 : 1;
-                  return kl(h, gs_small_fn<T>(mat_mode(L), c, from_zero),
-                            grid_for(nrows, small_threads<T>()), small_threads<T>(), s, vals,
-                            L.cols, L.g.n_store, r, z, row0, nrows, valid_end, early);
-                });
+  if (L.cnt[c] == 0) return HPG_OK;
+  if (!from_zero && halo_fits<T>(h, L, r, z, c))
+    return launch(h, K_GS, level, HPG_FP32, L.cnt[c] * 224.0, s, "gs_phase_halo_kernel", [&] {
+      return keep ? launch_gs_halo<T, false>(h, L, r, z, c, s)
+                  : launch_gs_halo<T, true>(h, L, r, z, c, s);
+    });
+  return stencil_colour_phase(h, level, 1, c, from_zero, r, z, s);
 }
-
 
 // Resident CTAs of the pipelined sweep kernel (queried once per precision).
 template <typename T>
@@ -768,20 +535,22 @@ static int symgs_pipelined(hpg_problem* h, int level, const T* r, T* z, bool fro
 template <typename T>
 static int symgs(hpg_problem* h, int level, const T* r, T* z, bool from_zero, SweepState& st,
                  cudaStream_t s) {
-  const bool streamed_level = h->lev[level].g.n_store * 27LL * 8 > kStreamMatrixBytes;
+  const Level& L = h->lev[level];
+  const bool streamed_level = L.g.n_store * 27LL * 8 > kStreamMatrixBytes;
   const bool pipe = h->gs_pipeline == 3 ||
                     (streamed_level && (h->gs_pipeline == 2 ||
-                                        (h->gs_pipeline == 1 && sizeof(T) == 8)));
-  if (pipe && h->lev[level].pipe_flags && h->pipe_err)
+                                        (h->gs_pipeline == 1 && L.stalled && sizeof(T) == 8)));
+  if (pipe && L.pipe_flags && h->pipe_err)
     return symgs_pipelined<T>(h, level, r, z, from_zero, st, s);
   int rc;
-  // Where a colour's slice of the matrix fits in L2 with room to spare:
-  // the slice of colour kColours - 2 is read again right after the turning
-  // colour, so its forward phase leaves it in L2 (the others stream
-  // evict-first); measured 1.2 % faster solves at 128^3 FP32.  The last phase
-  // (colour 0) leaves its slice in L2 too: after the post-smoothing, the
-  // Krylov SpMV reads the matrix from the colour-0 block on; 0.3 % faster.
-  const Level& L = h->lev[level];
+  if (!(h->gs_halo && streamed_level && sizeof(T) == 4)) {
+    rc = stencil_symgs(h, level, 1, r, z, from_zero, st.last == 0, s);
+    st.last = 0;
+    return rc;
+  }
+  // Where a colour's slice of the matrix fits in L2 with room to spare, the
+  // slice read again soon is left there: colour kColours - 2, read again right
+  // after the turning colour, and colour 0 (the others stream evict-first).
   const auto fits = [&](int c) {
     return (double)(L.g.off[c + 1] - L.g.off[c]) * kSlots * (sizeof(T) + 4.0) <=
            (double)kKeepSliceBytes;
@@ -856,8 +625,10 @@ coarse_sweep_cta_kernel(const T* __restrict__ vals, const int* __restrict__ cols
       xv[q] = (q != kCentre && ((ph.mask >> q) & 1u) && col[q] < ph.valid_end) ? sz[col[q]]
                                                                                 : T(0);
 #pragma unroll
-    for (int q = 0; q < kSlots; ++q)
+    for (int i = 0; i < kSlots; ++i) {
+      const int q = gs_order(i);
       if (q != kCentre && ((ph.mask >> q) & 1u)) acc = fma(-a[q], xv[q], acc);
+    }
     if (p + 1 < plan.nphases) load(p + 1, true);
     if (live) sz[ph.row0 + t] = acc / diag;
     __syncthreads();

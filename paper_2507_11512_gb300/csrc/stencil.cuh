@@ -25,6 +25,12 @@
 
 namespace hpg {
 
+// Slot visited q-th by a Gauss-Seidel phase: the plane below, the plane above,
+// then the point's own plane.  Both outer planes have the other z parity and
+// are constant while the colours of one plane parity are updated, so their 18
+// products are formed once for several updates of a point (gs_plane_kernel).
+__host__ __device__ constexpr int gs_order(int q) { return q < 9 ? q : q < 18 ? q + 9 : q - 9; }
+
 // A level's geometry in elements of an R-vector.  e / o: even / odd
 // coordinate.  off32 holds fewer than 2^31 elements (n_store * 27 < 2^31).
 struct SGeom {
@@ -204,5 +210,17 @@ int stencil_restrict(hpg_problem* h, int level, int R, const float* r, const flo
                      float* zc0, cudaStream_t s);
 int stencil_restrict(hpg_problem* h, int level, int R, const double* r, const double* z,
                      double* rc, double* zc0, cudaStream_t s);
+
+// One symmetric sweep (colours 0..7 then 7..0) and one colour phase, in place.
+// from_zero: z enters as 0 and is not read.  c0_done: colour 0's first phase
+// is already in z.
+int stencil_symgs(hpg_problem* h, int level, int R, const float* r, float* z, bool from_zero,
+                  bool c0_done, cudaStream_t s);
+int stencil_symgs(hpg_problem* h, int level, int R, const double* r, double* z, bool from_zero,
+                  bool c0_done, cudaStream_t s);
+int stencil_colour_phase(hpg_problem* h, int level, int R, int colour, bool from_zero,
+                         const float* r, float* z, cudaStream_t s);
+int stencil_colour_phase(hpg_problem* h, int level, int R, int colour, bool from_zero,
+                         const double* r, double* z, cudaStream_t s);
 
 }  // namespace hpg
