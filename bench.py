@@ -41,7 +41,7 @@ GS_TRAFFIC = {"workload": "mxp_gmres30_128cube", "bytes_per_launch": None,
 GS_KERNEL_TEXT = (
     ("paper_2507_11512_gb300/csrc/gs_planes.cu", "enum PlaneKind", "// Shared memory of a plane CTA"),
     ("paper_2507_11512_gb300/csrc/stencil.cuh", "// First element of the x-line",
-     "// Whether a point touches"),
+     "// Whether element e of an x-line"),
     ("paper_2507_11512_gb300/csrc/hpg_internal.cuh",
      "template <typename V>\n__device__ __forceinline__ V ld_dep", "\n}\n"),
 )

@@ -651,36 +651,38 @@ mupdate_x_kernel(double* __restrict__ x, const float* __restrict__ d, long long 
 }
 
 // r = b - A x (FP64, Algorithm 3 outer residual) and ||r_r||^2 per
-// right-hand side.  A thread meets one right-hand side only: lines, strides
-// and blocks of an R-vector are multiples of R.
+// right-hand side, one thread per storage row (g: geometry of one vector).
 template <int R>
 __global__ void __launch_bounds__(kBThreads)
 mresidual_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<double> c,
-                 const __grid_constant__ RowPlan pl, const double* diag,
-                 const double* __restrict__ b, const double* __restrict__ x,
-                 double* __restrict__ res, double* partials, double* gpart,
-                 unsigned int* counter, double* __restrict__ out) {
+                 long long ns, const double* diag, const double* __restrict__ b,
+                 const double* __restrict__ x, double* __restrict__ res, double* partials,
+                 double* gpart, unsigned int* counter, double* __restrict__ out) {
   pdl_trigger();
   pdl_wait();
-  double acc[1] = {0.0};
-  auto take = [&](unsigned p, double v) {
-    res[p] = v;
-    acc[0] = fma(v, v, acc[0]);
-  };
-  const unsigned stride = gridDim.x * kBThreads;
-  for (unsigned t = blockIdx.x * kBThreads + threadIdx.x; t < pl.threads + pl.pad; t += stride) {
-    if (t < pl.threads) {
-      const unsigned e = t % (unsigned)g.we, q = t / (unsigned)g.we;
-      stencil_rows<double, -1, 1>(g, c, x, diag, (int)e, (int)(q % pl.groups),
-                                  (int)(q / pl.groups), [&](unsigned p) { return ld_dep(b + p); },
-                                  take);
-    } else {
-      const unsigned p = pad_element(g, t - pl.threads);
-      take(p, ld_dep(b + p) - ld_dep(x + p));
+  double acc[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) acc[r] = 0.0;
+  const long long stride = (long long)gridDim.x * kBThreads;
+  for (long long row = blockIdx.x * (long long)kBThreads + threadIdx.x; row < ns;
+       row += stride) {
+    double v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = ld_dep(b + row * R + r);
+    const bool point = for_row_slots(g, (unsigned)row, [&](int s, int ci, bool in, unsigned q) {
+      const double a = s == kCentre ? (diag ? diag[row] : kDiag) : in ? c.a[ci] : 0.0;
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[r] = fma(-a, ld_dep(x + (long long)q * R + r), v[r]);
+    });
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (!point) v[r] = v[r] - ld_dep(x + row * R + r);   // padding row: identity
+      res[row * R + r] = v[r];
+      acc[r] = fma(v[r], v[r], acc[r]);
     }
   }
   __shared__ double sums[R];
-  if (mblock_partials_last<R, 1>(acc, 1, partials, gpart, counter, sums) && threadIdx.x < R)
+  if (mblock_partials_last<1, R>(acc, R, partials, gpart, counter, sums) && threadIdx.x < R)
     out[threadIdx.x] = sums[threadIdx.x];
 }
 
@@ -943,10 +945,9 @@ template <int R>
 static int enqueue_mouter(hpg_problem* h, unsigned long long loop, cudaStream_t s) {
   BatchSpace* bs = h->batch;
   const Level& L = h->lev[0];
-  const SGeom g = make_sgeom(L.g, R);
   int rc = launch(h, K_RESIDUAL, 0, HPG_FP64, L.n * 3.0 * 8.0 * R, s, "mresidual_kernel", [&] {
-    return kl(h, mresidual_kernel<R>, bs->G, kBThreads, s, g, make_coef<double>(h->beta),
-              make_row_plan(g, 1), level_diag<double>(L), (const double*)bs->b,
+    return kl(h, mresidual_kernel<R>, bs->G, kBThreads, s, make_sgeom(L.g, 1),
+              make_coef<double>(h->beta), bs->ns, level_diag<double>(L), (const double*)bs->b,
               (const double*)bs->x, bs->r, bs->partials, gpart_of(bs), bs->counter, bs->rho2);
   });
   if (rc) return rc;

@@ -38,8 +38,7 @@ gs_colour_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T
   const int i = 2 * (e / g.R) + px;
   T acc = ld_dep(r + row);
 #pragma unroll
-  for (int q = 0; q < kSlots; ++q) {
-    const int s = gs_order(q);
+  for (int s = 0; s < kSlots; ++s) {
     const int dx = s % 3 - 1, dy = (s / 3) % 3 - 1, dz = s / 9 - 1;
     if (s == kCentre) continue;
     const int nc = colour ^ ((dx & 1) | ((dy & 1) << 1) | ((dz & 1) << 2));
@@ -50,7 +49,8 @@ gs_colour_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T
                        ((px + dx) >> 1) * g.R);
     acc = fma(-c.a[dx + dy + dz + 3], v, acc);
   }
-  if (!from_zero && on_boundary(g, i, j, k)) acc = fma(T(0), ld_dep(z + row), acc);
+  if (!from_zero && (x_edge(g, px, e) || j == 0 || j == g.ny - 1 || k == 0 || k == g.nz - 1))
+    acc = fma(T(0), ld_dep(z + row), acc);
   z[row] = acc / (diag ? diag[row / (unsigned)g.R] : (T)kDiag);
 }
 
@@ -61,24 +61,29 @@ gs_colour_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T
 //   kOddFwd   colours 0 1 2 3          on the odd planes
 //   kEven     colours 4 5 6 7 6 5 4    on the even planes
 //   kOddBwd   colours 3 2 1 0          on the odd planes
-// is a whole symmetric sweep (15 phases) in 3 launches.  The 18 products with
-// the two planes above and below, constant meanwhile, are formed once per
-// point (streamed in lines, neighbour lines reused in registers) and kept in
-// shared memory; a phase then only adds the 8 products of its own plane, from
-// shared memory.
+// is a whole symmetric sweep (15 phases) in 3 launches.  A CTA holds its part
+// of the plane in shared memory; the planes above and below, constant
+// meanwhile, are read where they are (L1 holds the lines two phases share).
+// The products of a row keep slot order -- plane below, own plane, plane above --
+// so values equal the one-launch-per-colour sweep's bit for bit.
 //
 // A cluster of `cs` CTAs shares a plane, each owning `lines` x-lines of it.
 // A CTA recomputes the one to three lines beyond its own that its last phases
 // need, from old values it loads itself, so CTAs exchange nothing; the only
 // hazard is that they update z in place, and one cluster barrier -- all old
-// values loaded before the first store -- settles it, hidden behind the
-// streamed products.
+// values loaded before the first store -- settles it: a CTA arrives once its
+// loads are done and waits only before it stores, after its last phase.
+//
+// Large grids are bound by the vectors' traffic and by instruction issue (R
+// and the loads' offsets are compile-time, two FP32 elements share loads and
+// addresses for that reason), FP64 by the FP64 rate; small ones by the chain of
+// load, phases and store.
 enum PlaneKind { kOddFwd = 0, kEven = 1, kOddBwd = 2 };
 
 struct PlanePlan {
   int lines;    // x-lines per CTA (even)
   int cs;       // CTAs per plane (cluster size)
-  int bx, by;   // threads along x, lines in flight
+  int bx, by;   // threads along x, line groups in flight
   size_t smem;
 };
 
@@ -89,158 +94,271 @@ __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-constexpr int kPlaneThreads = 512;
+// Asynchronous copy of one element global -> shared (L1-coherent like ld_dep),
+// completed by copy_wait().
+__device__ __forceinline__ void copy_async(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copy_async(double* dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copy_async2(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copy_wait() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
 
-template <typename T, int KIND, bool ZERO>
+// Threads of a plane CTA, at most (a line's element groups must fit); two such
+// CTAs of the FP32 kernels fit an SM.
+constexpr int kPlaneThreads = 384;
+// Shared-memory layout of a CTA: z of the lines a-2 .. b+2, each as
+//   [pad | even part | pad | odd part | pad]   (pads zero, parts rounded to V)
+template <int R, int V> struct PlaneLayout {
+  int part, pitch, odd;
+  __host__ __device__ explicit PlaneLayout(const SGeom& g) {
+    part = (g.we + V - 1) / V * V;
+    odd = 2 * pad() + part;
+    pitch = 2 * part + 3 * pad();
+  }
+  static __host__ __device__ constexpr int pad() { return R > V ? R : V; }
+  __host__ __device__ size_t elems(int lines) const { return (size_t)(lines + 5) * pitch; }
+};
+
+template <typename T, int V>
+__device__ __forceinline__ void lds(const T* p, T (&a)[V]) {
+  unpack(*reinterpret_cast<const typename VecOf<T, V>::type*>(p), a);
+}
+
+// What a thread's elements touch on one line in shared memory.
+template <typename T, int R, int V>
+__device__ __forceinline__ LinePts<T, V> smem_line(const T* ev, const T* od) {
+  LinePts<T, V> p;
+  lds<T, V>(ev, p.e);
+  lds<T, V>(od, p.o);
+  if constexpr (R % V == 0) {
+    lds<T, V>(od - R, p.l);
+    lds<T, V>(ev + R, p.r);
+  } else {
+    p.l[0] = od[-1];
+    p.r[V - 1] = ev[V];
+#pragma unroll
+    for (int v = 1; v < V; ++v) {
+      p.l[v] = p.o[v - 1];
+      p.r[v - 1] = p.e[v];
+    }
+  }
+  return p;
+}
+
+template <typename T, int R, bool VEC, int KIND, bool ZERO>
 __global__ void __launch_bounds__(kPlaneThreads, sizeof(T) == 4 ? 2 : 1)
 gs_plane_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T> c,
                 const __grid_constant__ PlanePlan pl, const T* r, const T* diag, T* z,
                 int c0_done) {
   extern __shared__ __align__(16) unsigned char plane_smem[];
-  const int R = g.R, we = g.we, wo = g.wo;
-  const int pitch = we + wo + 4 * R;      // a line: [R zeros | even | R zeros][R | odd | R]
-  const int oddp = we + 3 * R;            // first odd element of a line
-  T* sz = reinterpret_cast<T*>(plane_smem);          // z of lines a-2 ..
-  T* sp = sz + (pl.lines + 5) * pitch;               // r minus the outer planes, lines a-1 ..
-  T* sd = sp + (pl.lines + 3) * (we + wo);           // diagonal (only with diag)
+  constexpr int V = row_elems<T>();
+  const PlaneLayout<R, V> lay(g);
+  const int we = g.we, wo = g.wo;
+  T* sz = reinterpret_cast<T*>(plane_smem);
   const int rank = (int)(blockIdx.x % (unsigned)pl.cs);
   const int k = 2 * (int)(blockIdx.x / (unsigned)pl.cs) + (KIND == kEven ? 0 : 1);
   const int a = rank * pl.lines, b = min(a + pl.lines, g.ny);
-  const int tx = threadIdx.x % pl.bx;
-  const int ty0 = threadIdx.x / pl.bx;
-  const int ty = ty0 < pl.by ? ty0 : (1 << 24);      // threads past the last line row idle
+  const int top = g.ny - 1;
+  const int x = (int)(threadIdx.x % (unsigned)pl.bx) * V;
+  const int ty0 = (int)(threadIdx.x / (unsigned)pl.bx);
+  const int ty = ty0 < pl.by ? ty0 : (1 << 24);      // threads past the last row idle
+  const XMask<R, V, VEC> m(g, x);
   pdl_trigger();
+  // zeros outside the parts
+  {
+    const int n = lay.pitch - we - wo;
+    for (int q = threadIdx.x; q < (pl.lines + 5) * n; q += blockDim.x) {
+      const int l = q / n;
+      int e = q - l * n;
+      if (e >= lay.pad()) e += we;
+      if (e >= lay.odd) e += wo;
+      sz[l * lay.pitch + e] = T(0);
+    }
+  }
   pdl_wait();
 
   // old values of the own plane (zero outside the grid, and before they are
-  // first computed in a sweep from zero)
-  for (int q = threadIdx.x; q < (pl.lines + 5) * R; q += blockDim.x) {
-    T* ln = sz + q / R * pitch + q % R;
-    ln[0] = T(0);
-    ln[R + we] = T(0);
-    ln[2 * R + we] = T(0);
-    ln[3 * R + we + wo] = T(0);
-  }
+  // first computed in a sweep from zero): the lines zlo .. zhi
+  const int zlo = max(KIND == kOddBwd ? a - 1 : a - 2, 0);
+  const int zhi = min(KIND == kOddFwd ? b : KIND == kEven ? b + 2 : b + 1, top);
+  const PlanePtr<T> pz(z, g, k, x);
   for (int l = ty; l < pl.lines + 5; l += pl.by) {
     const int j = a - 2 + l;
-    // lines a-2..b (forward odd planes), a-2..b+2 (even), a-1..b+1 (backward)
-    const bool in = j >= (KIND == kOddBwd ? max(a - 1, 0) : 0) && j < g.ny &&
-                    j <= b + (KIND == kOddFwd ? 0 : KIND == kEven ? 2 : 1) &&
-                    (!ZERO || (KIND == kOddFwd && c0_done && (j & 1)));
-    const T* ev = in ? z + line_base(g, 0, j, k) : z;
-    const T* od = in ? z + line_base(g, 1, j, k) : z;
-    T* ln = sz + l * pitch;
-    for (int e = tx; e < we; e += pl.bx) ln[R + e] = in && !ZERO ? ld_dep(ev + e) : T(0);
-    for (int e = tx; e < wo; e += pl.bx) ln[oddp + e] = in ? ld_dep(od + e) : T(0);
-  }
-  __syncwarp();
-  if (pl.cs > 1) cluster_arrive();
-
-  // r minus the products with the planes k-1 and k+1
-  {
-    const int plo = KIND == kOddBwd ? a : max(a - 1, 0);
-    const int phi = min(KIND == kEven ? b + 1 : KIND == kOddBwd ? b : b - 1, g.ny - 1);
-    const int chunk = (phi - plo + pl.by) / pl.by;
-    const int j0 = ty < pl.by ? plo + ty * chunk : g.ny;
-    const int j1 = min(j0 + chunk - 1, phi);
-    for (int e = tx; e < we && j0 <= j1; e += pl.bx) {
-      LinePts<T> lo[3], up[3];
-      if (!(ZERO && KIND == kOddFwd)) {
-        lo[1] = load_line(z, g, j0 - 1, k - 1, e);
-        up[1] = load_line(z, g, j0 - 1, k + 1, e);
-        lo[2] = load_line(z, g, j0, k - 1, e);
-        up[2] = load_line(z, g, j0, k + 1, e);
-      }
-      for (int j = j0; j <= j1; ++j) {
-        const unsigned pe = line_base(g, 0, j, k) + e, po = line_base(g, 1, j, k) + e;
-        T ae = ld_dep(r + pe), ao = e < wo ? ld_dep(r + po) : T(0);
-        T* sl = sp + (j - (a - 1)) * (we + wo);
-        if (diag) {
-          T* dl = sd + (j - (a - 1)) * (we + wo);
-          dl[e] = diag[pe / (unsigned)R];
-          if (e < wo) dl[we + e] = diag[po / (unsigned)R];
-        }
-        if (!(ZERO && KIND == kOddFwd)) {
-          lo[0] = lo[1];
-          lo[1] = lo[2];
-          lo[2] = load_line(z, g, j + 1, k - 1, e);
-          up[0] = up[1];
-          up[1] = up[2];
-          up[2] = load_line(z, g, j + 1, k + 1, e);
+    const bool in = j >= zlo && j <= zhi && (!ZERO || (KIND == kOddFwd && c0_done && (j & 1)));
+    T* le = sz + l * lay.pitch + lay.pad() + x;
+    T* lo = sz + l * lay.pitch + lay.odd + x;
+    if (in) {
+      const T* ev = pz.ev[j & 1] + (j >> 1) * we;
+      const T* od = pz.od[j & 1] + (j >> 1) * wo;
+      if constexpr (VEC && V == 2) {
+        if (!ZERO && m.e[0]) copy_async2(le, ev);
+        if (m.o[0]) copy_async2(lo, od);
+      } else {
 #pragma unroll
-          for (int dy = -1; dy <= 1; ++dy) {
-            const LinePts<T>& p = lo[dy + 1];
-            ae = line_sum<T, -1>(c, dy - 1, p.l, p.e, p.o, ae);
-            ao = line_sum<T, -1>(c, dy - 1, p.e, p.o, p.r, ao);
-          }
-#pragma unroll
-          for (int dy = -1; dy <= 1; ++dy) {
-            const LinePts<T>& p = up[dy + 1];
-            ae = line_sum<T, -1>(c, dy + 1, p.l, p.e, p.o, ae);
-            ao = line_sum<T, -1>(c, dy + 1, p.e, p.o, p.r, ao);
-          }
+        for (int v = 0; v < V; ++v) {
+          if (!ZERO && m.e[v]) copy_async(le + v, ev + v);
+          if (m.o[v]) copy_async(lo + v, od + v);
         }
-        sl[e] = ae;
-        if (e < wo) sl[we + e] = ao;
       }
     }
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      if (m.e[v] && (ZERO || !in)) le[v] = T(0);
+      if (m.o[v] && !in) lo[v] = T(0);
+    }
+  }
+  const PlanePtr<T> pr(r, g, k, x), pb(z, g, k > 0 ? k - 1 : k, x),
+      pa(z, g, k + 1 < g.nz ? k + 1 : k, x);
+  bool ready = false;   // whether the copies have been waited for
+
+  // Colours of the lines lo, lo + 2, .. <= hi (one line parity), in the order
+  // x odd (ODD1), x even, x odd again (ODD2): the products up to the line before
+  // and the loads of the line and the plane after, once, then the updates.
+  auto colours = [&](auto odd1, auto odd2, bool skip, int lo, int hi) {
+    constexpr bool ODD1 = decltype(odd1)::value, ODD2 = decltype(odd2)::value;
+    constexpr bool outer = !(ZERO && KIND == kOddFwd);   // the other planes are not zero
+    for (int jb = lo; jb <= hi; jb += 2 * pl.by) {
+      const int j = jb + 2 * ty;
+      const bool on = j <= hi;
+      const int p = jb & 1, J = j >> 1;
+      T ae[V] = {}, ao[V] = {};
+      LinePts<T, V> w[3];
+      if (on) {
+        load_elems<T, V, VEC>(pr.ev[p] + J * we, m.e, ae);
+        load_elems<T, V, VEC>(pr.od[p] + J * wo, m.o, ao);
+        if (outer) {
+          LinePts<T, V> w0[3];
+#pragma unroll
+          for (int u = 0; u < 3; ++u) {   // the lines j - 1, j, j + 1
+            const int pu = (p + u + 1) & 1, Ju = J + (p ? u >> 1 : (u + 1) / 2 - 1);
+            const bool in = j + u >= 1 && j + u <= top + 1;
+            w0[u] = load_line<T, R, V, VEC>(pb.ev[pu] + Ju * we, pb.od[pu] + Ju * wo,
+                                            in && k > 0, m);
+            w[u] = load_line<T, R, V, VEC>(pa.ev[pu] + Ju * we, pa.od[pu] + Ju * wo,
+                                           in && k + 1 < g.nz, m);
+          }
+#pragma unroll
+          for (int u = 0; u < 3; ++u) line_sum<T, -1, V>(c, u - 2, w0[u], ae, ao);
+        }
+      }
+      if (!ready) {   // the own plane's old values
+        copy_wait();
+        __syncwarp();
+        if (pl.cs > 1) cluster_arrive();
+        __syncthreads();
+        ready = true;
+      }
+      T* le = sz + (on ? j - (a - 2) : 1) * lay.pitch + lay.pad() + x;
+      T* lod = le - lay.pad() + lay.odd;
+      LinePts<T, V> after;
+      T de[V], dd[V];
+      bool bnd = false;
+      if (on) {
+        line_sum<T, -1, V>(c, -1, smem_line<T, R, V>(le - lay.pitch, lod - lay.pitch), ae, ao);
+        after = smem_line<T, R, V>(le + lay.pitch, lod + lay.pitch);
+        bnd = j == 0 || j == top || k == 0 || k == g.nz - 1 || x < R || x + V > wo - R;
+        if (diag) {
+#pragma unroll
+          for (int v = 0; v < V; ++v) {
+            de[v] = m.e[v] ? diag[(pr.ev[p] + J * we - r + v) / R] : T(1);
+            dd[v] = m.o[v] ? diag[(pr.od[p] + J * wo - r + v) / R] : T(1);
+          }
+        }
+      }
+      // x odd: neighbours even[x], even[x + R]; x even: odd[x - R], odd[x]
+      auto update = [&](auto xodd) {
+        constexpr bool XO = decltype(xodd)::value;
+        if (on) {
+          T l[V], q[V], u[V];
+          T* own = XO ? lod : le;
+          if constexpr (XO) {
+            lds<T, V>(le, l);
+            if constexpr (R % V == 0) {
+              lds<T, V>(le + R, q);
+            } else {
+#pragma unroll
+              for (int v = 0; v + 1 < V; ++v) q[v] = l[v + 1];
+              q[V - 1] = le[V];
+            }
+          } else {
+            lds<T, V>(lod, q);
+            if constexpr (R % V == 0) {
+              lds<T, V>(lod - R, l);
+            } else {
+              l[0] = lod[-1];
+#pragma unroll
+              for (int v = 1; v < V; ++v) l[v] = q[v - 1];
+            }
+          }
+#pragma unroll
+          for (int v = 0; v < V; ++v) {
+            u[v] = fma(-c.a[4], q[v], fma(-c.a[2], l[v], XO ? ao[v] : ae[v]));
+            u[v] = half_sum<T, XO>(c, 1, after, v, u[v]);
+            if (outer) {
+#pragma unroll
+              for (int d = 0; d < 3; ++d) u[v] = half_sum<T, XO>(c, d, w[d], v, u[v]);
+            }
+          }
+          if (bnd) {
+            T v0[V];
+            lds<T, V>(own, v0);
+            const bool edge = j == 0 || j == top || k == 0 || k == g.nz - 1;
+#pragma unroll
+            for (int v = 0; v < V; ++v)
+              if (edge || x_edge(g, XO ? 1 : 0, x + v)) u[v] = fma(T(0), v0[v], u[v]);
+          }
+#pragma unroll
+          for (int v = 0; v < V; ++v) {
+            u[v] = diag ? u[v] / (XO ? dd[v] : de[v]) : div_diag(u[v]);
+            if (XO ? m.o[v] : m.e[v]) own[v] = u[v];
+          }
+        }
+        __syncthreads();
+      };
+      if (ODD1 && !skip) update(std::true_type());
+      update(std::false_type());
+      if (ODD2) update(std::true_type());
+    }
+  };
+  using Yes = std::true_type;
+  using No = std::false_type;
+  if (KIND == kOddFwd) {
+    colours(Yes(), No(), c0_done != 0, a > 0 ? a - 1 : 1, b - 1);   // odd lines a-1 ..
+    colours(Yes(), No(), false, a, b - 1);
+  } else if (KIND == kEven) {
+    colours(Yes(), No(), false, a > 0 ? a - 1 : 1, min(b + 1, top));
+    colours(Yes(), Yes(), false, a, min(b, top));
+    colours(No(), Yes(), false, a + 1, b - 1);
+  } else {
+    colours(No(), Yes(), false, a, min(b, top));
+    colours(No(), Yes(), false, a + 1, b - 1);
+  }
+  if (!ready) {   // no line of this CTA has a phase
+    copy_wait();
+    __syncwarp();
+    if (pl.cs > 1) cluster_arrive();
+    __syncthreads();
   }
   __syncwarp();
   if (pl.cs > 1) cluster_wait();
-  __syncthreads();
-
-  // one phase: points of x parity XP on the lines lo, lo + 2, .. <= hi; the
-  // last update of an own line goes to memory
-  auto phase = [&](auto xp, int lo, int hi, bool store) {
-    constexpr int XP = decltype(xp)::value;
-    const int w = XP ? wo : we;
-    for (int j = lo + 2 * ty; j <= hi; j += 2 * pl.by) {
-      T* ln = sz + (j - (a - 2)) * pitch;
-      const T* su = sp + (j - (a - 1)) * (we + wo) + (XP ? we : 0);
-      const bool edge = j == 0 || j == g.ny - 1 || k == 0 || k == g.nz - 1;
-      T* out = z + line_base(g, XP, j, k);
-      const bool st = store && j >= a && j < b;
-      for (int e = tx; e < w; e += pl.bx) {
-        // offsets of x-1, x, x+1 in a line
-        const int m = (XP ? oddp : R) + e;
-        const int xl = XP ? R + e : oddp + e - R, xr = XP ? R + e + R : oddp + e;
-        T acc = su[e];
-        acc = line_sum<T, -1>(c, -1, ln[xl - pitch], ln[m - pitch], ln[xr - pitch], acc);
-        acc = fma(-c.a[2], ln[xl], acc);
-        acc = fma(-c.a[4], ln[xr], acc);
-        acc = line_sum<T, -1>(c, 1, ln[xl + pitch], ln[m + pitch], ln[xr + pitch], acc);
-        const int i = 2 * (e / R) + XP;
-        if (edge || i == 0 || i == g.nx - 1) acc = fma(T(0), ln[m], acc);
-        acc = diag ? acc / sd[(j - (a - 1)) * (we + wo) + (XP ? we : 0) + e] : acc / (T)kDiag;
-        ln[m] = acc;
-        if (st) out[e] = acc;
-      }
+  {
+    for (int j = a + ty; j < b; j += pl.by) {
+      const T* ln = sz + (j - (a - 2)) * lay.pitch + x;
+      T v[V];
+      lds<T, V>(ln + lay.pad(), v);
+      store_elems<T, V, VEC>(const_cast<T*>(pz.ev[j & 1]) + (j >> 1) * we, m.e, v);
+      lds<T, V>(ln + lay.odd, v);
+      store_elems<T, V, VEC>(const_cast<T*>(pz.od[j & 1]) + (j >> 1) * wo, m.o, v);
     }
-    __syncthreads();
-  };
-  using Even = std::integral_constant<int, 0>;
-  using Odd = std::integral_constant<int, 1>;
-  const int top = g.ny - 1;
-  if (KIND == kOddFwd) {
-    const int lo = a > 0 ? a - 1 : 1;   // odd lines a-1 .. b-1
-    if (!c0_done) phase(Odd(), lo, b - 1, true);
-    phase(Even(), lo, b - 1, true);
-    phase(Odd(), a, b - 1, true);
-    phase(Even(), a, b - 1, true);
-  } else if (KIND == kEven) {
-    const int lo = a > 0 ? a - 1 : 1;
-    phase(Odd(), lo, min(b + 1, top), false);
-    phase(Even(), lo, min(b + 1, top), false);
-    phase(Odd(), a, min(b, top), false);
-    phase(Even(), a, min(b, top), true);
-    phase(Odd(), a, min(b, top), true);
-    phase(Even(), a + 1, b - 1, true);
-    phase(Odd(), a + 1, b - 1, true);
-  } else {
-    phase(Even(), a, min(b, top), true);
-    phase(Odd(), a, min(b, top), true);
-    phase(Even(), a + 1, b - 1, true);
-    phase(Odd(), a + 1, b - 1, true);
   }
   // padding rows (identity) of these planes' colours
   if (blockIdx.x == 0) {
@@ -257,40 +375,53 @@ gs_plane_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T>
 
 // Shared memory of a plane CTA with `lines` own lines.
 template <typename T>
-static size_t plane_smem(const SGeom& g, int lines, bool diag) {
-  const size_t row = (size_t)g.we + g.wo;
-  return sizeof(T) * ((lines + 5) * (row + 4 * g.R) + (lines + 3) * row * (diag ? 2 : 1));
+static size_t plane_smem(const SGeom& g, int lines) {
+  constexpr int V = row_elems<T>();
+  const size_t n = g.R == 1   ? PlaneLayout<1, V>(g).elems(lines)
+                   : g.R == 2 ? PlaneLayout<2, V>(g).elems(lines)
+                   : g.R == 4 ? PlaneLayout<4, V>(g).elems(lines)
+                              : PlaneLayout<8, V>(g).elems(lines);
+  return sizeof(T) * n;
 }
 
 constexpr size_t kMaxPlaneSmem = 227u << 10;
-constexpr int kMaxPlaneCtas = 8;   // portable cluster size
+constexpr size_t kPlaneSmemGoal = 50u << 10;   // four CTAs per SM
+constexpr int kMaxPlaneCtas = 8;               // portable cluster size
 
-// How a level's planes are split: cs CTAs per plane so that about two CTAs
-// per SM are busy, with at least 8 lines each (a CTA recomputes up to 3 more),
-// more if a CTA's lines would not fit shared memory.  False: no split fits.
+// How a level's planes are split.  Up to 4 CTAs per plane while that makes at
+// most two CTAs per SM, with at least 8 lines each (a CTA recomputes up to 3
+// more); up to 8 where a CTA's lines would take more shared memory than four
+// CTAs per SM have (measured, 320^3 FP32 sweep: 775 us at one or two CTAs per SM,
+// 589 us at four; FP64 sweeps pay for the recomputed lines: 96^3 with 4 CTAs per
+// plane 197 us, with 8 213 us).  False: a line has more element groups than a
+// CTA threads, or its lines do not fit shared memory even so.
 template <typename T>
-static bool plane_plan(const SGeom& g, int num_sms, bool diag, PlanePlan* out) {
+static bool plane_plan(const SGeom& g, int num_sms, PlanePlan* out) {
+  constexpr int V = row_elems<T>();
   const int planes = std::max(g.de, 1);
   int cs = 1;
   auto lines_for = [&](int n) { return std::max(2, ((g.ny + n - 1) / n + 1) / 2 * 2); };
-  while (cs < kMaxPlaneCtas && planes * (cs + 1) <= 2 * num_sms && lines_for(cs + 1) >= 8) ++cs;
-  while (cs <= kMaxPlaneCtas && plane_smem<T>(g, lines_for(cs), diag) > kMaxPlaneSmem) ++cs;
-  if (cs > kMaxPlaneCtas) return false;
+  while (cs < 4 && planes * (cs + 1) <= 2 * num_sms && lines_for(cs + 1) >= 8) ++cs;
+  while (cs < kMaxPlaneCtas && plane_smem<T>(g, lines_for(cs)) > kPlaneSmemGoal) ++cs;
+  if (plane_smem<T>(g, lines_for(cs)) > kMaxPlaneSmem) return false;
   PlanePlan p;
   p.lines = lines_for(cs);
   p.cs = (g.ny + p.lines - 1) / p.lines;
-  const int pieces = (g.we + 127) / 128;
-  p.bx = (g.we + pieces - 1) / pieces;
-  p.by = std::max(1, std::min(kPlaneThreads / p.bx, p.lines + 3));
-  p.smem = plane_smem<T>(g, p.lines, diag);
+  p.bx = (g.we + V - 1) / V;
+  if (p.bx > kPlaneThreads) return false;
+  // a phase has up to lines / 2 + 2 lines
+  const int rows = p.lines / 2 + 2, fit = std::max(1, kPlaneThreads / p.bx);
+  const int passes = (rows + fit - 1) / fit;
+  p.by = (rows + passes - 1) / passes;
+  p.smem = plane_smem<T>(g, p.lines);
   *out = p;
   return true;
 }
 
-template <typename T, int KIND, bool ZERO>
-static cudaError_t plane_launch(hpg_problem* h, const SGeom& g, const PlanePlan& pl, const T* r,
-                                const T* diag, T* z, int c0_done, cudaStream_t s) {
-  auto kern = gs_plane_kernel<T, KIND, ZERO>;
+template <typename T, int R, bool VEC, int KIND, bool ZERO>
+static cudaError_t plane_launch_r(hpg_problem* h, const SGeom& g, const PlanePlan& pl, const T* r,
+                                  const T* diag, T* z, int c0_done, cudaStream_t s) {
+  auto kern = gs_plane_kernel<T, R, VEC, KIND, ZERO>;
   if (pl.smem > (48u << 10)) {
     const cudaError_t e = cudaFuncSetAttribute(
         kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxPlaneSmem);
@@ -318,6 +449,19 @@ static cudaError_t plane_launch(hpg_problem* h, const SGeom& g, const PlanePlan&
   cfg.attrs = attr;
   cfg.numAttrs = na;
   return cudaLaunchKernelEx(&cfg, kern, g, make_coef<T>(h->beta), pl, r, diag, z, c0_done);
+}
+
+template <typename T, int KIND, bool ZERO>
+static cudaError_t plane_launch(hpg_problem* h, const SGeom& g, const PlanePlan& pl, const T* r,
+                                const T* diag, T* z, int c0_done, cudaStream_t s) {
+  if constexpr (sizeof(T) == 4) {   // R-vectors are FP32
+    if (g.R == 8) return plane_launch_r<T, 8, true, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s);
+    if (g.R == 4) return plane_launch_r<T, 4, true, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s);
+    if (g.R == 2) return plane_launch_r<T, 2, true, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s);
+    if (!whole_groups<T, row_elems<T>()>(g, r, z))
+      return plane_launch_r<T, 1, false, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s);
+  }
+  return plane_launch_r<T, 1, true, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s);
 }
 
 template <typename T>
@@ -354,7 +498,7 @@ static int symgs_t(hpg_problem* h, int level, int R, const T* r, T* z, bool from
   const T* diag = level_diag<T>(L);
   int rc;
   PlanePlan pl;
-  if (!plane_plan<T>(g, h->num_sms, diag != nullptr, &pl)) {
+  if (!plane_plan<T>(g, h->num_sms, &pl)) {
     for (int c = c0_done ? 1 : 0; c < kColours; ++c)
       if ((rc = stencil_colour_phase(h, level, R, c, from_zero, r, z, s))) return rc;
     for (int c = kColours - 2; c >= 0; --c)

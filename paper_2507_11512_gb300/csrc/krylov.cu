@@ -785,29 +785,25 @@ update_x_kernel(double* __restrict__ x, const T* __restrict__ d, long long ns) {
 // 2-byte basis).
 __global__ void __launch_bounds__(kRedThreads)
 residual_norm_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<double> c,
-                     const __grid_constant__ RowPlan pl, const double* diag,
-                     const double* __restrict__ b, const double* __restrict__ x,
-                     double* __restrict__ r, double* __restrict__ partials,
-                     unsigned int* counter, double* __restrict__ out) {
+                     long long ns, const double* diag, const double* __restrict__ b,
+                     const double* __restrict__ x, double* __restrict__ r,
+                     double* __restrict__ partials, unsigned int* counter,
+                     double* __restrict__ out) {
   pdl_trigger();
   pdl_wait();
   double acc[2] = {0.0, 0.0};
-  auto take = [&](unsigned p, double v) {
-    r[p] = v;
+  const long long stride = (long long)gridDim.x * kRedThreads;
+  for (long long row = blockIdx.x * (long long)kRedThreads + threadIdx.x; row < ns;
+       row += stride) {
+    double v = ld_dep(b + row);
+    const bool point = for_row_slots(g, (unsigned)row, [&](int s, int ci, bool in, unsigned q) {
+      const double a = s == kCentre ? (diag ? diag[row] : kDiag) : in ? c.a[ci] : 0.0;
+      v = fma(-a, ld_dep(x + q), v);
+    });
+    if (!point) v = v - ld_dep(x + row);   // padding row: identity
+    r[row] = v;
     acc[0] = fma(v, v, acc[0]);
     acc[1] = fmax(acc[1], fabs(v));
-  };
-  const unsigned stride = gridDim.x * kRedThreads;
-  for (unsigned t = blockIdx.x * kRedThreads + threadIdx.x; t < pl.threads + pl.pad; t += stride) {
-    if (t < pl.threads) {
-      const unsigned e = t % (unsigned)g.we, q = t / (unsigned)g.we;
-      stencil_rows<double, -1, 1>(g, c, x, diag, (int)e, (int)(q % pl.groups),
-                                  (int)(q / pl.groups), [&](unsigned p) { return ld_dep(b + p); },
-                                  take);
-    } else {
-      const unsigned p = pad_element(g, t - pl.threads);
-      take(p, ld_dep(b + p) - ld_dep(x + p));
-    }
   }
   __shared__ double sums[2];
   if (block_partials_last<double, 2, true>(acc, 2, partials, counter, sums) && threadIdx.x < 2)
@@ -1070,11 +1066,11 @@ static int enqueue_cycle_update(hpg_problem* h, hpg_prec prec, int k_model, cuda
 static int enqueue_outer(hpg_problem* h, unsigned long long loop, cudaStream_t s) {
   Workspace* ws = h->ws;
   const Level& L = h->lev[0];
-  const SGeom g = make_sgeom(L.g, 1);
   int rc = launch(h, K_RESIDUAL, 0, HPG_FP64, L.n * 3.0 * 8.0, s, "residual_norm_kernel", [&] {
-    return kl(h, residual_norm_kernel, ws->G, kRedThreads, s, g, make_coef<double>(h->beta),
-              make_row_plan(g, 1), level_diag<double>(L), (const double*)ws->b,
-              (const double*)ws->x, ws->r, ws->partials, ws->counter, ws->rho2);
+    return kl(h, residual_norm_kernel, ws->G, kRedThreads, s, make_sgeom(L.g, 1),
+              make_coef<double>(h->beta), L.g.n_store, level_diag<double>(L),
+              (const double*)ws->b, (const double*)ws->x, ws->r, ws->partials, ws->counter,
+              ws->rho2);
   });
   if (rc) return rc;
   return launch(h, K_NORM, 0, HPG_FP64, 0.0, s, "outer_check_kernel", [&] {

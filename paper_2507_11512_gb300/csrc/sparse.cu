@@ -189,11 +189,10 @@ gs_phase_halo_kernel(const T* __restrict__ vals, const int* __restrict__ cols, l
   T acc = sr[e];
 #pragma unroll
   for (int q = 0; q < kSlots; ++q) {
-    const int s = gs_order(q);
-    if (s == kCentre) continue;
-    const unsigned idx = (unsigned)(sc[s * rpad + e] + sdelta[s]);
+    if (q == kCentre) continue;
+    const unsigned idx = (unsigned)(sc[q * rpad + e] + sdelta[q]);
     const T xv = idx < nsm ? sx[idx] : T(0);
-    acc = fma(-sv[s * rpad + e], xv, acc);
+    acc = fma(-sv[q * rpad + e], xv, acc);
   }
   x[row0 + t] = acc / sv[kCentre * rpad + e];
 }
@@ -248,8 +247,7 @@ __device__ __forceinline__ void pipe_row(const T* __restrict__ vals, const int* 
                                          long long row, long long valid_end, unsigned mask) {
   T acc = ld_dep(r + row);
 #pragma unroll
-  for (int q = 0; q < kSlots; ++q) {
-    const int s = gs_order(q);
+  for (int s = 0; s < kSlots; ++s) {
     if (s == kCentre) continue;
     if (MASKED) {
       const bool use = (mask >> s) & 1u;
@@ -625,10 +623,8 @@ coarse_sweep_cta_kernel(const T* __restrict__ vals, const int* __restrict__ cols
       xv[q] = (q != kCentre && ((ph.mask >> q) & 1u) && col[q] < ph.valid_end) ? sz[col[q]]
                                                                                 : T(0);
 #pragma unroll
-    for (int i = 0; i < kSlots; ++i) {
-      const int q = gs_order(i);
+    for (int q = 0; q < kSlots; ++q)
       if (q != kCentre && ((ph.mask >> q) & 1u)) acc = fma(-a[q], xv[q], acc);
-    }
     if (p + 1 < plan.nphases) load(p + 1, true);
     if (live) sz[ph.row0 + t] = acc / diag;
     __syncthreads();

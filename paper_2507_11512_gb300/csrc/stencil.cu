@@ -12,37 +12,57 @@
 namespace hpg {
 
 // ------------------------------------------------------------------ product
-// y = A x (Sec. 3.2.2).  Bound by the vectors' traffic (8 bytes per FP32 row)
-// on large grids, by latency on small ones; FP64 by the FP64 rate (27 FMAs a
-// row).  A thread takes a point pair of LINES consecutive x-lines, so that a
-// warp's loads run along x and neighbour lines are reused in registers.
-template <typename T, int LINES>
+// y = A x (Sec. 3.2.2).  FP32: instruction issue first, then the vectors'
+// traffic (8 bytes a row); FP64: the FP64 rate (27 FMAs a row).  A thread takes
+// an element group of LINES consecutive x-lines, so that a warp's loads run
+// along x, neighbour lines are reused in registers and two FP32 elements share
+// loads and addresses.
+template <typename T, int R, bool VEC, int LINES>
 __global__ void __launch_bounds__(256)
 stencil_spmv_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T> c,
                     const __grid_constant__ RowPlan pl, const T* x, const T* diag, T* y) {
+  constexpr int V = row_elems<T>();
   pdl_trigger();
   pdl_wait();
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t < pl.threads) {
-    const unsigned e = t % (unsigned)g.we, q = t / (unsigned)g.we;
+    const unsigned e = t % pl.across, q = t / pl.across;
     const unsigned grp = q % pl.groups, k = q / pl.groups;
-    stencil_rows<T, 1, LINES>(g, c, x, diag, (int)e, (int)grp * LINES, (int)k,
-                              [](unsigned) { return T(0); },
-                              [&](unsigned p, T v) { y[p] = v; });
+    stencil_rows<T, 1, R, V, VEC, LINES>(
+        g, c, x, diag, (int)e * V, (int)grp * LINES, (int)k,
+        [](unsigned, const bool (&)[V], T (&a)[V]) {
+#pragma unroll
+          for (int v = 0; v < V; ++v) a[v] = T(0);
+        },
+        [&](unsigned p, const bool (&m)[V], const T (&a)[V]) {
+          store_elems<T, V, VEC>(y + p, m, a);
+        });
   } else if (t - pl.threads < pl.pad) {
     const unsigned p = pad_element(g, t - pl.threads);
     y[p] = ld_dep(x + p);
   }
 }
 
-RowPlan make_row_plan(const SGeom& g, int lines) {
+RowPlan make_row_plan(const SGeom& g, int elems, int lines) {
   RowPlan p;
-  p.lines = lines;
+  p.across = (unsigned)((g.we + elems - 1) / elems);
   p.groups = (unsigned)((g.ny + lines - 1) / lines);
-  p.threads = (unsigned)g.we * p.groups * (unsigned)g.nz;
+  p.threads = p.across * p.groups * (unsigned)g.nz;
   p.pad = 0;
   for (int c = 0; c < kColours; ++c) p.pad += g.end[c] - g.off[c] - g.cnt[c];
   return p;
+}
+
+template <typename T, int R, bool VEC>
+static cudaError_t spmv_launch(hpg_problem* h, const SGeom& g, const T* x, const T* diag, T* y,
+                               int block, cudaStream_t s) {
+  constexpr int V = row_elems<T>();
+  // four lines a thread once that leaves every SM several 256-thread blocks
+  const bool big = (long long)g.we / V * g.ny * g.nz >= (long long)kRowLines * 2 * 256 * h->num_sms;
+  const RowPlan pl = make_row_plan(g, V, big ? kRowLines : 1);
+  return kl(h, big ? stencil_spmv_kernel<T, R, VEC, kRowLines> : stencil_spmv_kernel<T, R, VEC, 1>,
+            grid_for((long long)pl.threads + pl.pad, block), block, s, g, make_coef<T>(h->beta),
+            pl, x, diag, y);
 }
 
 template <typename T>
@@ -50,17 +70,18 @@ static int spmv_t(hpg_problem* h, int level, int R, const T* x, T* y, cudaStream
                   int block) {
   const Level& L = h->lev[level];
   const SGeom g = make_sgeom(L.g, R);
-  // four lines a thread once that leaves every SM several 256-thread blocks
-  const bool big = (long long)g.we * g.ny * g.nz >= (long long)kRowLines * 4 * 256 * h->num_sms;
-  const RowPlan pl = make_row_plan(g, big ? kRowLines : 1);
   const T* diag = level_diag<T>(L);
-  const int grid = grid_for((long long)pl.threads + pl.pad, block);
   return launch(h, K_SPMV, level, sizeof(T) == 8 ? HPG_FP64 : HPG_FP32,
                 (double)L.n * R * 2.0 * sizeof(T) + (diag ? L.n * (double)sizeof(T) : 0.0), s,
                 "stencil_spmv_kernel", [&] {
-                  return kl(h, big ? stencil_spmv_kernel<T, kRowLines>
-                                   : stencil_spmv_kernel<T, 1>,
-                            grid, block, s, g, make_coef<T>(h->beta), pl, x, diag, y);
+                  const bool vec = whole_groups<T, row_elems<T>()>(g, x, y);
+                  if constexpr (sizeof(T) == 4) {   // R-vectors are FP32
+                    if (R == 8) return spmv_launch<T, 8, true>(h, g, x, diag, y, block, s);
+                    if (R == 4) return spmv_launch<T, 4, true>(h, g, x, diag, y, block, s);
+                    if (R == 2) return spmv_launch<T, 2, true>(h, g, x, diag, y, block, s);
+                    if (!vec) return spmv_launch<T, 1, false>(h, g, x, diag, y, block, s);
+                  }
+                  return spmv_launch<T, 1, true>(h, g, x, diag, y, block, s);
                 });
 }
 int stencil_spmv(hpg_problem* h, int level, int R, const float* x, float* y, cudaStream_t s,
@@ -78,6 +99,11 @@ int stencil_spmv(hpg_problem* h, int level, int R, const double* x, double* y, c
 // order.  One thread per coarse element; slot order as the product's.
 // zc0 (optional): the coarse level's first phase from zero on its colour-0
 // points, z_I = rc_I / a_II (see symgs).
+template <typename T>
+__device__ __forceinline__ T sub_line(const Coef<T>& c, int dyz, T l, T m, T r, T acc) {
+  return fma(-c.a[dyz + 4], r, fma(-c.a[dyz + 3], m, fma(-c.a[dyz + 2], l, acc)));
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256)
 stencil_restrict_kernel(const __grid_constant__ SGeom gf, const __grid_constant__ Geom gc,
@@ -113,9 +139,10 @@ stencil_restrict_kernel(const __grid_constant__ SGeom gf, const __grid_constant_
       acc = fma(-c.a[2], l[u], acc);
       acc = fma(-d, m[u], acc);
       acc = fma(-c.a[4], rr[u], acc);
-      if (on_boundary(gf, 2 * (int)I, j, k)) acc = fma(T(0), m[u], acc);
+      if (x_edge(gf, 0, (int)e) || j == 0 || j == gf.ny - 1 || k == 0 || k == gf.nz - 1)
+        acc = fma(T(0), m[u], acc);
     } else {
-      acc = line_sum<T, -1>(c, dyz, l[u], m[u], rr[u], acc);
+      acc = sub_line(c, dyz, l[u], m[u], rr[u], acc);
     }
   }
   const long long Rc = store_index(gc, (int)I, J, K);

@@ -25,12 +25,6 @@
 
 namespace hpg {
 
-// Slot visited q-th by a Gauss-Seidel phase: the plane below, the plane above,
-// then the point's own plane.  Both outer planes have the other z parity and
-// are constant while the colours of one plane parity are updated, so their 18
-// products are formed once for several updates of a point (gs_plane_kernel).
-__host__ __device__ constexpr int gs_order(int q) { return q < 9 ? q : q < 18 ? q + 9 : q - 9; }
-
 // A level's geometry in elements of an R-vector.  e / o: even / odd
 // coordinate.  off32 holds fewer than 2^31 elements (n_store * 27 < 2^31).
 struct SGeom {
@@ -71,80 +65,207 @@ __device__ __forceinline__ unsigned line_base(const SGeom& g, int px, int j, int
   return g.off[c] + (unsigned)w * ((unsigned)(j >> 1) + (unsigned)h * (unsigned)(k >> 1));
 }
 
-// What the two points at element e of line (j, k) -- x = 2I and x = 2I + 1 --
-// touch on that line: x = 2I-1, 2I, 2I+1, 2I+2.  Zero outside the grid.
-template <typename T> struct LinePts { T l, e, o, r; };
-template <typename T>
-__device__ __forceinline__ LinePts<T> load_line(const T* v, const SGeom& g, int j, int k, int e) {
-  LinePts<T> p;
-  p.l = p.e = p.o = p.r = T(0);
-  if ((unsigned)j < (unsigned)g.ny && (unsigned)k < (unsigned)g.nz) {
-    const T* ev = v + line_base(g, 0, j, k) + e;
-    const T* od = v + line_base(g, 1, j, k) + e;
-    if (e < g.we) p.e = ld_dep(ev);
-    if (e < g.wo) p.o = ld_dep(od);
-    if (e >= g.R && e - g.R < g.wo) p.l = ld_dep(od - g.R);
-    if (e + g.R < g.we) p.r = ld_dep(ev + g.R);
+// A thread takes V consecutive elements of an x-line, each standing for the
+// two points x = 2I and x = 2I + 1.  LinePts holds what they touch on one line:
+// x = 2I-1 (l), 2I (e), 2I+1 (o), 2I+2 (r), zero outside the grid.
+template <typename T, int V> struct LinePts { T l[V], e[V], o[V], r[V]; };
+
+// Which of a thread's elements exist (they depend on its position in x only).
+// VEC: the elements of a part come in whole, aligned groups of V.
+template <int R, int V, bool VEC> struct XMask {
+  bool e[V], o[V], l[V], r[V];
+  __device__ __forceinline__ XMask(const SGeom& g, int x) {
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      e[v] = VEC ? x < g.we : x + v < g.we;
+      o[v] = VEC ? x < g.wo : x + v < g.wo;
+      l[v] = x + v >= R && x + v - R < g.wo;
+      r[v] = x + v + R < g.we;
+    }
+  }
+};
+
+template <typename T, int V> struct VecOf { using type = T; };
+template <> struct VecOf<float, 2> { using type = float2; };
+__device__ __forceinline__ void unpack(float v, float (&o)[1]) { o[0] = v; }
+__device__ __forceinline__ void unpack(double v, double (&o)[1]) { o[0] = v; }
+__device__ __forceinline__ void unpack(float2 v, float (&o)[2]) { o[0] = v.x; o[1] = v.y; }
+
+// The line whose even and odd parts start (at the thread's element) at ev, od;
+// in: the line exists.
+template <typename T, int R, int V, bool VEC>
+__device__ __forceinline__ LinePts<T, V> load_line(const T* ev, const T* od, bool in,
+                                                   const XMask<R, V, VEC>& m) {
+  LinePts<T, V> p;
+#pragma unroll
+  for (int v = 0; v < V; ++v) p.l[v] = p.e[v] = p.o[v] = p.r[v] = T(0);
+  if (!in) return p;
+  if constexpr (VEC && V > 1) {
+    using P = typename VecOf<T, V>::type;
+    unpack(ld_dep(reinterpret_cast<const P*>(ev)), p.e);
+    if (m.o[0]) unpack(ld_dep(reinterpret_cast<const P*>(od)), p.o);
+    if constexpr (R % V == 0) {
+      if (m.l[0]) unpack(ld_dep(reinterpret_cast<const P*>(od - R)), p.l);
+      if (m.r[0]) unpack(ld_dep(reinterpret_cast<const P*>(ev + R)), p.r);
+    } else {   // R = 1
+      if (m.l[0]) p.l[0] = ld_dep(od - 1);
+      if (m.r[V - 1]) p.r[V - 1] = ld_dep(ev + V);
+#pragma unroll
+      for (int v = 1; v < V; ++v) {
+        p.l[v] = p.o[v - 1];
+        p.r[v - 1] = p.e[v];
+      }
+    }
+  } else {
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      if (m.e[v]) p.e[v] = ld_dep(ev + v);
+      if (m.o[v]) p.o[v] = ld_dep(od + v);
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      if (V > R && v >= R) p.l[v] = p.o[v - R];
+      else if (m.l[v]) p.l[v] = ld_dep(od + v - R);
+      if (V > R && v + R < V) p.r[v] = p.e[v + R];
+      else if (m.r[v]) p.r[v] = ld_dep(ev + v + R);
+    }
   }
   return p;
 }
 
-// acc + sum over the three points dx = -1..1 of a line at offset (dy, dz) of
-// a * x, for the even (px = 0) or odd point; sign: +1 adds, -1 subtracts the
-// products (fma of the negated coefficient, as the ELL kernels do).
-template <typename T, int SIGN>
-__device__ __forceinline__ T line_sum(const Coef<T>& c, int dyz, T l, T m, T r, T acc) {
-  const T a0 = c.a[dyz + 2], a1 = c.a[dyz + 3], a2 = c.a[dyz + 4];
-  acc = fma(SIGN > 0 ? a0 : -a0, l, acc);
-  acc = fma(SIGN > 0 ? a1 : -a1, m, acc);
-  return fma(SIGN > 0 ? a2 : -a2, r, acc);
+// Start of a plane's lines at element x: line j (parity p = j & 1) begins at
+// ev[p] + (j >> 1) * we and od[p] + (j >> 1) * wo.
+template <typename T> struct PlanePtr {
+  const T *ev[2], *od[2];
+  __device__ __forceinline__ PlanePtr(const T* v, const SGeom& g, int k, int x) {
+    const int K = k >> 1, cz = (k & 1) ? 0 : 4;
+    ev[0] = v + (g.off[cz | 3] + (unsigned)g.we * (unsigned)(g.he * K) + x);
+    od[0] = v + (g.off[cz | 2] + (unsigned)g.wo * (unsigned)(g.he * K) + x);
+    ev[1] = v + (g.off[cz | 1] + (unsigned)g.we * (unsigned)(g.ho * K) + x);
+    od[1] = v + (g.off[cz] + (unsigned)g.wo * (unsigned)(g.ho * K) + x);
+  }
+};
+
+// acc + the products of one line at dy + dz = dyz, for the even and odd points;
+// SIGN -1 subtracts them (fma of the negated coefficient, as the ELL kernels).
+template <typename T, int SIGN, int V>
+__device__ __forceinline__ void line_sum(const Coef<T>& c, int dyz, const LinePts<T, V>& p,
+                                         T (&ae)[V], T (&ao)[V]) {
+  const T a0 = SIGN > 0 ? c.a[dyz + 2] : -c.a[dyz + 2];
+  const T a1 = SIGN > 0 ? c.a[dyz + 3] : -c.a[dyz + 3];
+  const T a2 = SIGN > 0 ? c.a[dyz + 4] : -c.a[dyz + 4];
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    ae[v] = fma(a2, p.o[v], fma(a1, p.e[v], fma(a0, p.l[v], ae[v])));
+    ao[v] = fma(a2, p.r[v], fma(a1, p.o[v], fma(a0, p.e[v], ao[v])));
+  }
 }
 
-// Whether a point touches the grid's boundary.
-__device__ __forceinline__ bool on_boundary(const SGeom& g, int i, int j, int k) {
-  return i == 0 || i == g.nx - 1 || j == 0 || j == g.ny - 1 || k == 0 || k == g.nz - 1;
+// The same for one point of parity XO of element v.
+template <typename T, bool XO, int V>
+__device__ __forceinline__ T half_sum(const Coef<T>& c, int dyz, const LinePts<T, V>& p, int v,
+                                      T acc) {
+  const T l = XO ? p.e[v] : p.l[v], q = XO ? p.o[v] : p.e[v], r = XO ? p.r[v] : p.o[v];
+  return fma(-c.a[dyz + 4], r, fma(-c.a[dyz + 3], q, fma(-c.a[dyz + 2], l, acc)));
 }
 
-// acc + SIGN * A_ij x_j over all 27 slots in slot order, for the point pair at
-// element e of line (j, k); w[dz][dy] are the lines around it.  diag: the
-// diagonal entry of each point.
-template <typename T, int SIGN, bool ODD>
-__device__ __forceinline__ T point_sum(const Coef<T>& c, const LinePts<T> (&w)[3][3], T diag,
-                                       bool boundary, T acc) {
+// x / 26, correctly rounded: Markstein's division by a known divisor (IBM J.
+// Res. Dev. 34, 1990): with y = RN(1/26), q = RN(x y) and the exact remainder
+// x - 26 q, RN(q + remainder * y) is RN(x / 26) unless something under- or
+// overflows, which the range test leaves to the plain division.
+__device__ __forceinline__ float div_diag(float x) {
+  const float a = fabsf(x);
+  if (a >= 1e-30f && a <= 1e37f) {
+    constexpr float y = 1.0f / (float)kDiag;
+    const float q = x * y;
+    return fmaf(fmaf(-(float)kDiag, q, x), y, q);
+  }
+  return x / (float)kDiag;
+}
+__device__ __forceinline__ double div_diag(double x) {
+  const int e = __double2hiint(x) & 0x7ff00000;
+  if (e >= (200 << 20) && e <= (1900 << 20)) {   // 2^-823 .. 2^877
+    constexpr double y = 1.0 / kDiag;
+    const double q = x * y;
+    return fma(fma(-kDiag, q, x), y, q);
+  }
+  return x / kDiag;
+}
+
+// Whether element e of an x-line's even (px 0) or odd part is its first or
+// last grid point.
+__device__ __forceinline__ bool x_edge(const SGeom& g, int px, int e) {
+  return (px == 0 && e < g.R) || (px == ((g.nx - 1) & 1) && e >= (px ? g.wo : g.we) - g.R);
+}
+
+// f(slot, coefficient index, inside the grid, neighbour's row or else own row)
+// for the 27 slots of a storage row (geometry with R = 1) in slot order; false
+// for a padding row.  For kernels with one thread per storage row.
+template <typename F>
+__device__ __forceinline__ bool for_row_slots(const SGeom& g, unsigned row, F&& f) {
+  int colour = 0;
 #pragma unroll
-  for (int dz = -1; dz <= 1; ++dz)
+  for (int q = 1; q < kColours; ++q) colour += row >= g.off[q] ? 1 : 0;
+  const unsigned p = row - g.off[colour];
+  if (p >= g.cnt[colour]) return false;
+  const int px = colour_parity_x(colour), py = colour_parity_y(colour),
+            pz = colour_parity_z(colour);
+  const unsigned w = px ? g.wo : g.we, hl = py ? g.ho : g.he;
+  const int e = (int)(p % w), i = 2 * e + px;
+  const int j = 2 * (int)(p / w % hl) + py, k = 2 * (int)(p / w / hl) + pz;
 #pragma unroll
-    for (int dy = -1; dy <= 1; ++dy) {
-      const LinePts<T>& p = w[dz + 1][dy + 1];
-      const T l = ODD ? p.e : p.l, m = ODD ? p.o : p.e, r = ODD ? p.r : p.o;
-      if (dy == 0 && dz == 0) {
-        acc = fma(SIGN > 0 ? c.a[2] : -c.a[2], l, acc);
-        acc = fma(SIGN > 0 ? diag : -diag, m, acc);
-        acc = fma(SIGN > 0 ? c.a[4] : -c.a[4], r, acc);
-        if (boundary) acc = fma(T(0), m, acc);
-      } else {
-        acc = line_sum<T, SIGN>(c, dy + dz, l, m, r, acc);
-      }
-    }
-  return acc;
+  for (int s = 0; s < kSlots; ++s) {
+    const int dx = s % 3 - 1, dy = (s / 3) % 3 - 1, dz = s / 9 - 1;
+    const bool in = (unsigned)(i + dx) < (unsigned)g.nx && (unsigned)(j + dy) < (unsigned)g.ny &&
+                    (unsigned)(k + dz) < (unsigned)g.nz;
+    f(s, dx + dy + dz + 3, in,
+      in ? line_base(g, px ^ (dx & 1), j + dy, k + dz) + e + ((px + dx) >> 1) : row);
+  }
+  return true;
 }
 
 // Lines a thread of a whole-grid product takes (stencil_rows): 4 share their
-// neighbour lines in registers (72 loads for 8 rows instead of 144); 1 where
-// that would leave SMs without work.
+// neighbour lines in registers; 1 where that would leave SMs without work.
 constexpr int kRowLines = 4;
+// Elements of a line it takes: the loads of two FP32 elements are one load
+// each, and their addresses one computation; FP64 is bound by its FMAs.
+template <typename T> __host__ __device__ constexpr int row_elems() {
+  return sizeof(T) == 4 ? 2 : 1;
+}
+// Whether a vector's parts come in whole aligned groups of V elements.
+template <typename T, int V> inline bool whole_groups(const SGeom& g, const void* a, const void* b) {
+  return V == 1 || (g.we % V == 0 && g.wo % V == 0 &&
+                    (((uintptr_t)a | (uintptr_t)b) & (V * sizeof(T) - 1)) == 0);
+}
 
-// f(row element, sum, boundary) for every point of up to LINES consecutive
-// lines of plane k at element e, where sum = init(element) + SIGN * (A x).
-template <typename T, int SIGN, int LINES, typename Init, typename Out>
-__device__ __forceinline__ void stencil_rows(const SGeom& g, const Coef<T>& c, const T* x,
-                                             const T* diag, int e, int j0, int k, Init&& init,
+// out(first element, V sums, which exist) for the even and the odd points of up
+// to LINES lines of plane k from j0 on at element x, with sum = init(first
+// element) + SIGN * (A x) over all 27 slots in slot order.
+template <typename T, int SIGN, int R, int V, bool VEC, int LINES, typename Init, typename Out>
+__device__ __forceinline__ void stencil_rows(const SGeom& g, const Coef<T>& c, const T* xv,
+                                             const T* diag, int x, int j0, int k, Init&& init,
                                              Out&& out) {
-  LinePts<T> w[3][3];
+  const XMask<R, V, VEC> m(g, x);
+  const bool in_k[3] = {k > 0, true, k + 1 < g.nz};
+  const PlanePtr<T> pp[3] = {PlanePtr<T>(xv, g, in_k[0] ? k - 1 : k, x), PlanePtr<T>(xv, g, k, x),
+                             PlanePtr<T>(xv, g, in_k[2] ? k + 1 : k, x)};
+  LinePts<T, V> w[3][3];
+  auto fetch = [&](int dz, int j) {
+    const int p = j & 1, J = j >> 1;
+    return load_line<T, R, V, VEC>(pp[dz].ev[p] + J * g.we, pp[dz].od[p] + J * g.wo,
+                                   in_k[dz] && j >= 0 && j < g.ny, m);
+  };
 #pragma unroll
   for (int dz = 0; dz < 3; ++dz) {
-    w[dz][1] = load_line(x, g, j0 - 1, k + dz - 1, e);
-    w[dz][2] = load_line(x, g, j0, k + dz - 1, e);
+    w[dz][1] = fetch(dz, j0 - 1);
+    w[dz][2] = fetch(dz, j0);
+  }
+  bool be[V], bo[V], bx = false;   // points on the grid's x faces
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    be[v] = x_edge(g, 0, x + v);
+    bo[v] = x_edge(g, 1, x + v);
+    bx = bx || be[v] || bo[v];
   }
 #pragma unroll
   for (int q = 0; q < LINES; ++q) {
@@ -154,31 +275,78 @@ __device__ __forceinline__ void stencil_rows(const SGeom& g, const Coef<T>& c, c
     for (int dz = 0; dz < 3; ++dz) {
       w[dz][0] = w[dz][1];
       w[dz][1] = w[dz][2];
-      w[dz][2] = load_line(x, g, j + 1, k + dz - 1, e);
+      w[dz][2] = fetch(dz, j + 1);
     }
-    const int I2 = e / g.R * 2;
-    if (e < g.we) {
-      const unsigned p = line_base(g, 0, j, k) + e;
-      const T d = diag ? diag[p / (unsigned)g.R] : (T)kDiag;
-      out(p, point_sum<T, SIGN, false>(c, w, d, on_boundary(g, I2, j, k), init(p)));
-    }
-    if (e < g.wo) {
-      const unsigned p = line_base(g, 1, j, k) + e;
-      const T d = diag ? diag[p / (unsigned)g.R] : (T)kDiag;
-      out(p, point_sum<T, SIGN, true>(c, w, d, on_boundary(g, I2 + 1, j, k), init(p)));
-    }
+    const unsigned pe = line_base(g, 0, j, k) + x, po = line_base(g, 1, j, k) + x;
+    T ae[V], ao[V];
+    init(pe, m.e, ae);
+    init(po, m.o, ao);
+#pragma unroll
+    for (int dz = -1; dz <= 1; ++dz)
+#pragma unroll
+      for (int dy = -1; dy <= 1; ++dy) {
+        const LinePts<T, V>& p = w[dz + 1][dy + 1];
+        if (dy != 0 || dz != 0) {
+          line_sum<T, SIGN, V>(c, dy + dz, p, ae, ao);
+          continue;
+        }
+        const T a0 = SIGN > 0 ? c.a[2] : -c.a[2], a2 = SIGN > 0 ? c.a[4] : -c.a[4];
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+          T de = (T)kDiag, dd = (T)kDiag;
+          if (diag) {
+            if (m.e[v]) de = diag[(pe + v) / R];
+            if (m.o[v]) dd = diag[(po + v) / R];
+          }
+          if (SIGN < 0) de = -de, dd = -dd;
+          ae[v] = fma(a2, p.o[v], fma(de, p.e[v], fma(a0, p.l[v], ae[v])));
+          ao[v] = fma(a2, p.r[v], fma(dd, p.o[v], fma(a0, p.e[v], ao[v])));
+        }
+        if (bx || j == 0 || j == g.ny - 1 || k == 0 || k == g.nz - 1) {
+          const bool edge = j == 0 || j == g.ny - 1 || k == 0 || k == g.nz - 1;
+#pragma unroll
+          for (int v = 0; v < V; ++v) {
+            if (edge || be[v]) ae[v] = fma(T(0), p.e[v], ae[v]);
+            if (edge || bo[v]) ao[v] = fma(T(0), p.o[v], ao[v]);
+          }
+        }
+      }
+    out(pe, m.e, ae);
+    out(po, m.o, ao);
   }
 }
 
-// Threads of a whole-grid product with LINES lines each: (element, line group,
-// plane), plus one thread per padding row element at the end.
+// V elements of a vector at p (those in m), to and from registers.
+template <typename T, int V, bool VEC>
+__device__ __forceinline__ void load_elems(const T* p, const bool (&m)[V], T (&a)[V]) {
+  if constexpr (VEC && V > 1) {
+    if (m[0]) unpack(ld_dep(reinterpret_cast<const typename VecOf<T, V>::type*>(p)), a);
+  } else {
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+      if (m[v]) a[v] = ld_dep(p + v);
+  }
+}
+template <typename T, int V, bool VEC>
+__device__ __forceinline__ void store_elems(T* p, const bool (&m)[V], const T (&a)[V]) {
+  if constexpr (VEC && V == 2) {
+    if (m[0]) *reinterpret_cast<float2*>(p) = make_float2(a[0], a[1]);
+  } else {
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+      if (m[v]) p[v] = a[v];
+  }
+}
+
+// Threads of a whole-grid product: (element group, line group, plane), plus one
+// thread per padding row element at the end.
 struct RowPlan {
-  int lines;              // 1 or kRowLines
+  unsigned across;        // element groups of a line
   unsigned groups;        // line groups per plane
   unsigned threads;       // point threads
   unsigned pad;           // padding elements
 };
-RowPlan make_row_plan(const SGeom& g, int lines);
+RowPlan make_row_plan(const SGeom& g, int elems, int lines);
 
 // Padding element number q of an R-vector, or the first element past the end.
 __device__ __forceinline__ unsigned pad_element(const SGeom& g, unsigned q) {

@@ -18,7 +18,7 @@
 #include <cooperative_groups.h>
 #include <string.h>
 
-#include "stencil.cuh"
+#include "hpg_internal.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -70,13 +70,12 @@ struct ClusterRows {
   }
 };
 
-// One row's sum over NS slots from the S0-th on, in slot order or (GS) in
-// gs_order without the centre: the indices and values of the
+// One row's sum over slots [S0, S0 + NS): the indices and values of the
 // group are loaded together, then the gathers, then the FMAs, so a warp pays
 // two L2 round trips per group instead of two per slot (coarse phases have a
 // warp or two per SM, nothing else hides the latency).  Slots whose
 // neighbour is known to be zero are masked, not loaded.
-template <typename T, bool GS, int S0, int NS>
+template <typename T, int S0, int NS>
 __device__ __forceinline__ T row_group(const T* __restrict__ vals, const int* __restrict__ cols,
                                        const T* x, int ns, int row, int c, bool from_zero,
                                        int valid_end, T acc) {
@@ -85,8 +84,8 @@ __device__ __forceinline__ T row_group(const T* __restrict__ vals, const int* __
   bool use[NS];
 #pragma unroll
   for (int i = 0; i < NS; ++i) {
-    const int s = GS ? gs_order(S0 + i) : S0 + i;
-    use[i] = !(GS && s == kCentre) && !(from_zero && neighbour_colour(c, s) >= c);
+    const int s = S0 + i;
+    use[i] = !(from_zero && neighbour_colour(c, s) >= c);
     col[i] = use[i] ? __ldg(cols + s * ns + row) : 0;
     a[i] = use[i] ? __ldg(vals + s * ns + row) : T(0);
   }
@@ -114,8 +113,8 @@ __device__ void phase_gs(const VcParams& P, const VcPhase& ph, const ClusterRows
   for (int row = row0 + cr.first; row < row1; row += cr.step) {
     const T diag = __ldg(vals + kCentre * ns + row);
     T acc = __ldcg(r + row);
-    acc = row_group<T, true, 0, 13>(vals, cols, x, ns, row, c, from_zero, valid_end, acc);
-    acc = row_group<T, true, 13, 14>(vals, cols, x, ns, row, c, from_zero, valid_end, acc);
+    acc = row_group<T, 0, 13>(vals, cols, x, ns, row, c, from_zero, valid_end, acc);
+    acc = row_group<T, 14, 13>(vals, cols, x, ns, row, c, from_zero, valid_end, acc);
     x[row] = acc / diag;
   }
 }
@@ -137,8 +136,8 @@ __device__ void phase_restrict(const VcParams& P, const VcPhase& ph, const Clust
     const int row = row0 + p;
     T acc = __ldcg(r + row);
     // same slot order as the one-launch-per-phase restriction: 0..26
-    acc = row_group<T, false, 0, 14>(vals, cols, z, ns, row, 0, false, ns, acc);
-    acc = row_group<T, false, 14, 13>(vals, cols, z, ns, row, 0, false, ns, acc);
+    acc = row_group<T, 0, 14>(vals, cols, z, ns, row, 0, false, ns, acc);
+    acc = row_group<T, 14, 13>(vals, cols, z, ns, row, 0, false, ns, acc);
     const int I = p % cx;
     const int J = (p / cx) % cy;
     const int K = p / (cx * cy);
