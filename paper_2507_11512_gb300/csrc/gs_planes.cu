@@ -50,7 +50,7 @@ gs_colour_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T
     acc = fma(-c.a[dx + dy + dz + 3], v, acc);
   }
   if (!from_zero && (x_edge(g, px, e) || j == 0 || j == g.ny - 1 || k == 0 || k == g.nz - 1))
-    acc = fma(T(0), ld_dep(z + row), acc);
+    pad_slot(ld_dep(z + row), acc);
   z[row] = acc / (diag ? diag[row / (unsigned)g.R] : (T)kDiag);
 }
 
@@ -61,9 +61,9 @@ gs_colour_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T
 //   kOddFwd   colours 0 1 2 3          on the odd planes
 //   kEven     colours 4 5 6 7 6 5 4    on the even planes
 //   kOddBwd   colours 3 2 1 0          on the odd planes
-// is a whole symmetric sweep (15 phases) in 3 launches.  A CTA holds its part
-// of the plane in shared memory; the planes above and below, constant
-// meanwhile, are read where they are (L1 holds the lines two phases share).
+// is a whole symmetric sweep (15 phases) in 3 launches.  A CTA copies its
+// lines of the plane and of the two planes beside it (constant meanwhile) into
+// shared memory, all at once, and every phase runs from there.
 // The products of a row keep slot order -- plane below, own plane, plane above --
 // so values equal the one-launch-per-colour sweep's bit for bit.
 //
@@ -83,7 +83,8 @@ enum PlaneKind { kOddFwd = 0, kEven = 1, kOddBwd = 2 };
 struct PlanePlan {
   int lines;    // x-lines per CTA (even)
   int cs;       // CTAs per plane (cluster size)
-  int bx, by;   // threads along x, line groups in flight
+  int bx, by;   // threads along x, lines in flight (even)
+  int early;    // whether the next kernel may start while this one runs
   size_t smem;
 };
 
@@ -94,19 +95,15 @@ __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Asynchronous copy of one element global -> shared (L1-coherent like ld_dep),
-// completed by copy_wait().
-__device__ __forceinline__ void copy_async(float* dst, const float* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void copy_async(double* dst, const double* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void copy_async2(float* dst, const float* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(dst)), "l"(src)
-               : "memory");
+// Asynchronous copy of B bytes global -> shared, or zeros where !in (src is not
+// read then), completed by copy_wait().
+template <int B> __device__ __forceinline__ void copy_async(void* dst, const void* src, bool in) {
+  if constexpr (B == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src),
+                 "r"(in ? 16 : 0) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(smem_addr(dst)), "l"(src),
+                 "n"(B), "r"(in ? B : 0) : "memory");
 }
 __device__ __forceinline__ void copy_wait() {
   asm volatile("cp.async.wait_all;" ::: "memory");
@@ -114,8 +111,9 @@ __device__ __forceinline__ void copy_wait() {
 
 // Threads of a plane CTA, at most (a line's element groups must fit); two such
 // CTAs of the FP32 kernels fit an SM.
-constexpr int kPlaneThreads = 384;
-// Shared-memory layout of a CTA: z of the lines a-2 .. b+2, each as
+constexpr int kPlaneThreads = 768;
+// Shared-memory layout of a CTA: z of the lines a-2 .. b+2 of the planes k-1, k
+// and k+1, each line as
 //   [pad | even part | pad | odd part | pad]   (pads zero, parts rounded to V)
 template <int R, int V> struct PlaneLayout {
   int part, pitch, odd;
@@ -125,7 +123,9 @@ template <int R, int V> struct PlaneLayout {
     pitch = 2 * part + 3 * pad();
   }
   static __host__ __device__ constexpr int pad() { return R > V ? R : V; }
-  __host__ __device__ size_t elems(int lines) const { return (size_t)(lines + 5) * pitch; }
+  __host__ __device__ size_t elems(int lines) const {
+    return (size_t)(lines + 5) * pitch * 3;
+  }
 };
 
 template <typename T, int V>
@@ -154,16 +154,34 @@ __device__ __forceinline__ LinePts<T, V> smem_line(const T* ev, const T* od) {
   return p;
 }
 
-template <typename T, int R, bool VEC, int KIND, bool ZERO>
-__global__ void __launch_bounds__(kPlaneThreads, sizeof(T) == 4 ? 2 : 1)
+// u minus the products of one line in shared memory, for the points of x parity
+// XO (R a multiple of V).
+template <typename T, int R, int V, bool XO>
+__device__ __forceinline__ void half_line(const Coef<T>& c, int dyz, const T* ev, const T* od,
+                                          T (&u)[V]) {
+  T l[V], q[V], r[V];
+  lds<T, V>(XO ? ev : od - R, l);
+  lds<T, V>(XO ? od : ev, q);
+  lds<T, V>(XO ? ev + R : od, r);
+#pragma unroll
+  for (int v = 0; v < V; ++v)
+    u[v] = fma(-c.a[dyz + 4], r[v], fma(-c.a[dyz + 3], q[v], fma(-c.a[dyz + 2], l[v], u[v])));
+}
+
+template <typename T, int R, int V, bool VEC, int KIND, bool ZERO>
+__global__ void __launch_bounds__(kPlaneThreads)
 gs_plane_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T> c,
                 const __grid_constant__ PlanePlan pl, const T* r, const T* diag, T* z,
                 int c0_done) {
   extern __shared__ __align__(16) unsigned char plane_smem[];
-  constexpr int V = row_elems<T>();
   const PlaneLayout<R, V> lay(g);
   const int we = g.we, wo = g.wo;
-  T* sz = reinterpret_cast<T*>(plane_smem);
+  const int slab = (pl.lines + 5) * lay.pitch;
+  T* const sz = reinterpret_cast<T*>(plane_smem) + slab;   // plane k; k-1 before, k+1 after
+  constexpr bool outer = !(ZERO && KIND == kOddFwd);       // the planes beside are not zero
+  // the line and the plane after in registers for both x parities; four-element
+  // R-vector groups (64 registers of them) read them again instead
+  constexpr bool kHold = R % V != 0 || V < 4;
   const int rank = (int)(blockIdx.x % (unsigned)pl.cs);
   const int k = 2 * (int)(blockIdx.x / (unsigned)pl.cs) + (KIND == kEven ? 0 : 1);
   const int a = rank * pl.lines, b = min(a + pl.lines, g.ny);
@@ -172,107 +190,138 @@ gs_plane_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T>
   const int ty0 = (int)(threadIdx.x / (unsigned)pl.bx);
   const int ty = ty0 < pl.by ? ty0 : (1 << 24);      // threads past the last row idle
   const XMask<R, V, VEC> m(g, x);
-  pdl_trigger();
-  // zeros outside the parts
+  if (pl.early) pdl_trigger();
+  // zeros around the parts
   {
-    const int n = lay.pitch - we - wo;
-    for (int q = threadIdx.x; q < (pl.lines + 5) * n; q += blockDim.x) {
-      const int l = q / n;
-      int e = q - l * n;
-      if (e >= lay.pad()) e += we;
-      if (e >= lay.odd) e += wo;
-      sz[l * lay.pitch + e] = T(0);
+    constexpr int pad = PlaneLayout<R, V>::pad();
+    const int first = outer ? 0 : pl.lines + 5, last = (outer ? 3 : 2) * (pl.lines + 5);
+    for (int l = first + (int)threadIdx.x; l < last; l += blockDim.x) {
+      T* ln = sz + l * lay.pitch - slab;
+#pragma unroll
+      for (int e = 0; e < pad; ++e) ln[e] = ln[lay.odd - pad + e] = ln[lay.pitch - pad + e] = T(0);
+      if (!VEC)   // parts that are not whole groups
+        for (int e = 0; e < V; ++e) ln[lay.odd - pad - 1 - e] = ln[lay.pitch - pad - 1 - e] = T(0);
     }
+    if (!VEC) __syncthreads();   // the parts' ends are written below
   }
   pdl_wait();
 
-  // old values of the own plane (zero outside the grid, and before they are
-  // first computed in a sweep from zero): the lines zlo .. zhi
+  // The lines zlo .. zhi of the three planes (zero outside the grid; the own
+  // plane's also before they are first computed in a sweep from zero).  by is
+  // even, so a thread's lines have one parity and its pointers a fixed step.
   const int zlo = max(KIND == kOddBwd ? a - 1 : a - 2, 0);
   const int zhi = min(KIND == kOddFwd ? b : KIND == kEven ? b + 2 : b + 1, top);
-  const PlanePtr<T> pz(z, g, k, x);
-  for (int l = ty; l < pl.lines + 5; l += pl.by) {
-    const int j = a - 2 + l;
-    const bool in = j >= zlo && j <= zhi && (!ZERO || (KIND == kOddFwd && c0_done && (j & 1)));
-    T* le = sz + l * lay.pitch + lay.pad() + x;
-    T* lo = sz + l * lay.pitch + lay.odd + x;
-    if (in) {
-      const T* ev = pz.ev[j & 1] + (j >> 1) * we;
-      const T* od = pz.od[j & 1] + (j >> 1) * wo;
-      if constexpr (VEC && V == 2) {
-        if (!ZERO && m.e[0]) copy_async2(le, ev);
-        if (m.o[0]) copy_async2(lo, od);
-      } else {
+  if (ty < pl.by) {
+    const int p = ty & 1;   // a is even: the parity of a - 2 + ty
+    const bool in_lo = k > 0, in_up = k + 1 < g.nz;
+    const PlanePtr<T> p0(z, g, k, x), p1(z, g, in_lo ? k - 1 : k, x), p2(z, g, in_up ? k + 1 : k, x);
+    const bool own_o = !ZERO || (KIND == kOddFwd && c0_done && p);   // from zero: colour 0 at most
+    T* le = sz + ty * lay.pitch + lay.pad() + x;
+    T* lo = le - lay.pad() + lay.odd;
+    constexpr int B = VEC ? V * (int)sizeof(T) : (int)sizeof(T);
+    constexpr int N = VEC ? 1 : V;
+    for (int l = ty; l < pl.lines + 5; l += pl.by) {
+      const int j = a - 2 + l;
+      const bool in = j >= zlo && j <= zhi;
+      const int oe = in ? (j >> 1) * we : 0, oo = in ? (j >> 1) * wo : 0;
 #pragma unroll
-        for (int v = 0; v < V; ++v) {
-          if (!ZERO && m.e[v]) copy_async(le + v, ev + v);
-          if (m.o[v]) copy_async(lo + v, od + v);
+      for (int v = 0; v < N; ++v) {
+        if (m.e[v]) {
+          copy_async<B>(le + v, p0.ev[p] + oe + v, in && !ZERO);
+          if (outer) {
+            copy_async<B>(le + v - slab, p1.ev[p] + oe + v, in && in_lo);
+            copy_async<B>(le + v + slab, p2.ev[p] + oe + v, in && in_up);
+          }
+        }
+        if (VEC || m.o[v]) {   // whole groups: zeros past the end of an odd part
+          const bool has = in && m.o[v];
+          copy_async<B>(lo + v, p0.od[p] + oo + v, has && own_o);
+          if (outer) {
+            copy_async<B>(lo + v - slab, p1.od[p] + oo + v, has && in_lo);
+            copy_async<B>(lo + v + slab, p2.od[p] + oo + v, has && in_up);
+          }
         }
       }
-    }
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      if (m.e[v] && (ZERO || !in)) le[v] = T(0);
-      if (m.o[v] && !in) lo[v] = T(0);
+      le += pl.by * lay.pitch;
+      lo += pl.by * lay.pitch;
     }
   }
-  const PlanePtr<T> pr(r, g, k, x), pb(z, g, k > 0 ? k - 1 : k, x),
-      pa(z, g, k + 1 < g.nz ? k + 1 : k, x);
-  bool ready = false;   // whether the copies have been waited for
+  const PlanePtr<T> pz(z, g, k, x), pr(r, g, k, x);
+  // which of the thread's even / odd points lie on an x face of the grid
+  unsigned edge_e = 0, edge_o = 0;
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    edge_e |= x_edge(g, 0, x + v) ? 1u << v : 0u;
+    edge_o |= x_edge(g, 1, x + v) ? 1u << v : 0u;
+  }
+  const bool edge_k = k == 0 || k == g.nz - 1;
+  // r of the next pass's line, loaded a pass ahead
+  T re[V] = {}, ro[V] = {};
+  auto fetch_r = [&](int j, int hi) {
+    if (j <= hi) {
+      load_elems<T, V, VEC>(pr.ev[j & 1] + (j >> 1) * we, m.e, re);
+      load_elems<T, V, VEC>(pr.od[j & 1] + (j >> 1) * wo, m.o, ro);
+    }
+  };
+  const int olo = a > 0 && KIND != kOddBwd ? a - 1 : a + 1;   // first odd line of the first call
+  const int ohi = min(KIND == kEven ? b + 1 : b - 1, top);
+  if (KIND == kOddBwd || olo > ohi) fetch_r(a + 2 * ty, min(b, top));   // (no odd line)
+  else fetch_r(olo + 2 * ty, ohi);
+  copy_wait();
+  __syncwarp();
+  if (pl.cs > 1) cluster_arrive();
+  __syncthreads();
 
   // Colours of the lines lo, lo + 2, .. <= hi (one line parity), in the order
-  // x odd (ODD1), x even, x odd again (ODD2): the products up to the line before
-  // and the loads of the line and the plane after, once, then the updates.
-  auto colours = [&](auto odd1, auto odd2, bool skip, int lo, int hi) {
+  // x odd (ODD1), x even, x odd again (ODD2): the products up to the line before,
+  // once, then the updates.  nlo, nhi: the lines of the next call.
+  auto colours = [&](auto odd1, auto odd2, bool skip, int lo, int hi, int nlo, int nhi) {
     constexpr bool ODD1 = decltype(odd1)::value, ODD2 = decltype(odd2)::value;
-    constexpr bool outer = !(ZERO && KIND == kOddFwd);   // the other planes are not zero
     for (int jb = lo; jb <= hi; jb += 2 * pl.by) {
       const int j = jb + 2 * ty;
       const bool on = j <= hi;
-      const int p = jb & 1, J = j >> 1;
-      T ae[V] = {}, ao[V] = {};
-      LinePts<T, V> w[3];
-      if (on) {
-        load_elems<T, V, VEC>(pr.ev[p] + J * we, m.e, ae);
-        load_elems<T, V, VEC>(pr.od[p] + J * wo, m.o, ao);
-        if (outer) {
-          LinePts<T, V> w0[3];
+      T ae[V], ao[V];
 #pragma unroll
-          for (int u = 0; u < 3; ++u) {   // the lines j - 1, j, j + 1
-            const int pu = (p + u + 1) & 1, Ju = J + (p ? u >> 1 : (u + 1) / 2 - 1);
-            const bool in = j + u >= 1 && j + u <= top + 1;
-            w0[u] = load_line<T, R, V, VEC>(pb.ev[pu] + Ju * we, pb.od[pu] + Ju * wo,
-                                            in && k > 0, m);
-            w[u] = load_line<T, R, V, VEC>(pa.ev[pu] + Ju * we, pa.od[pu] + Ju * wo,
-                                           in && k + 1 < g.nz, m);
-          }
-#pragma unroll
-          for (int u = 0; u < 3; ++u) line_sum<T, -1, V>(c, u - 2, w0[u], ae, ao);
-        }
+      for (int v = 0; v < V; ++v) {
+        ae[v] = re[v];
+        ao[v] = ro[v];
       }
-      if (!ready) {   // the own plane's old values
-        copy_wait();
-        __syncwarp();
-        if (pl.cs > 1) cluster_arrive();
-        __syncthreads();
-        ready = true;
-      }
+      const bool more = jb + 2 * pl.by <= hi;
+      fetch_r(more ? j + 2 * pl.by : nlo + 2 * ty, more ? hi : nhi);
       T* le = sz + (on ? j - (a - 2) : 1) * lay.pitch + lay.pad() + x;
       T* lod = le - lay.pad() + lay.odd;
-      LinePts<T, V> after;
+      LinePts<T, V> after, w[3];
       T de[V], dd[V];
-      bool bnd = false;
+      unsigned be = 0, bo = 0;
       if (on) {
-        line_sum<T, -1, V>(c, -1, smem_line<T, R, V>(le - lay.pitch, lod - lay.pitch), ae, ao);
-        after = smem_line<T, R, V>(le + lay.pitch, lod + lay.pitch);
-        bnd = j == 0 || j == top || k == 0 || k == g.nz - 1 || x < R || x + V > wo - R;
         if (diag) {
 #pragma unroll
           for (int v = 0; v < V; ++v) {
-            de[v] = m.e[v] ? diag[(pr.ev[p] + J * we - r + v) / R] : T(1);
-            dd[v] = m.o[v] ? diag[(pr.od[p] + J * wo - r + v) / R] : T(1);
+            de[v] = m.e[v] ? diag[(pr.ev[j & 1] + (j >> 1) * we - r + v) / R] : T(1);
+            dd[v] = m.o[v] ? diag[(pr.od[j & 1] + (j >> 1) * wo - r + v) / R] : T(1);
           }
         }
+        if (outer) {
+#pragma unroll
+          for (int u = 0; u < 3; ++u) {   // the lines j - 1, j, j + 1 of plane k - 1
+            const int o = (u - 1) * lay.pitch - slab;
+            line_sum<T, -1, V>(c, u - 2, smem_line<T, R, V>(le + o, lod + o), ae, ao);
+          }
+        }
+        line_sum<T, -1, V>(c, -1, smem_line<T, R, V>(le - lay.pitch, lod - lay.pitch), ae, ao);
+        if (kHold) {
+          after = smem_line<T, R, V>(le + lay.pitch, lod + lay.pitch);
+          if (outer) {
+#pragma unroll
+            for (int u = 0; u < 3; ++u) {
+              const int o = (u - 1) * lay.pitch + slab;
+              w[u] = smem_line<T, R, V>(le + o, lod + o);
+            }
+          }
+        }
+        const bool all = edge_k || j == 0 || j == top;
+        be = all ? 15u : edge_e;
+        bo = all ? 15u : edge_o;
       }
       // x odd: neighbours even[x], even[x + R]; x even: odd[x - R], odd[x]
       auto update = [&](auto xodd) {
@@ -300,27 +349,40 @@ gs_plane_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T>
             }
           }
 #pragma unroll
-          for (int v = 0; v < V; ++v) {
+          for (int v = 0; v < V; ++v)
             u[v] = fma(-c.a[4], q[v], fma(-c.a[2], l[v], XO ? ao[v] : ae[v]));
-            u[v] = half_sum<T, XO>(c, 1, after, v, u[v]);
+          if (kHold) {
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+              u[v] = half_sum<T, XO>(c, 1, after, v, u[v]);
+              if (outer) {
+#pragma unroll
+                for (int d = 0; d < 3; ++d) u[v] = half_sum<T, XO>(c, d, w[d], v, u[v]);
+              }
+            }
+          } else {
+            half_line<T, R, V, XO>(c, 1, le + lay.pitch, lod + lay.pitch, u);
             if (outer) {
 #pragma unroll
-              for (int d = 0; d < 3; ++d) u[v] = half_sum<T, XO>(c, d, w[d], v, u[v]);
+              for (int d = 0; d < 3; ++d)
+                half_line<T, R, V, XO>(c, d, le + (d - 1) * lay.pitch + slab,
+                                       lod + (d - 1) * lay.pitch + slab, u);
             }
           }
-          if (bnd) {
+          if (XO ? bo : be) {
             T v0[V];
             lds<T, V>(own, v0);
-            const bool edge = j == 0 || j == top || k == 0 || k == g.nz - 1;
 #pragma unroll
             for (int v = 0; v < V; ++v)
-              if (edge || x_edge(g, XO ? 1 : 0, x + v)) u[v] = fma(T(0), v0[v], u[v]);
+              if (((XO ? bo : be) >> v) & 1u) pad_slot(v0[v], u[v]);
           }
+          if (diag) {
 #pragma unroll
-          for (int v = 0; v < V; ++v) {
-            u[v] = diag ? u[v] / (XO ? dd[v] : de[v]) : div_diag(u[v]);
-            if (XO ? m.o[v] : m.e[v]) own[v] = u[v];
+            for (int v = 0; v < V; ++v) u[v] = u[v] / (XO ? dd[v] : de[v]);
+          } else {
+            div_diag<T, V>(u);
           }
+          store_elems<T, V, VEC>(own, XO ? m.o : m.e, u);
         }
         __syncthreads();
       };
@@ -331,22 +393,17 @@ gs_plane_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T>
   };
   using Yes = std::true_type;
   using No = std::false_type;
+  const int eb = min(b, top), ob = min(b + 1, top);
   if (KIND == kOddFwd) {
-    colours(Yes(), No(), c0_done != 0, a > 0 ? a - 1 : 1, b - 1);   // odd lines a-1 ..
-    colours(Yes(), No(), false, a, b - 1);
+    colours(Yes(), No(), c0_done != 0, olo, b - 1, a, b - 1);   // odd lines a-1 .. b-1
+    colours(Yes(), No(), false, a, b - 1, 0, -1);
   } else if (KIND == kEven) {
-    colours(Yes(), No(), false, a > 0 ? a - 1 : 1, min(b + 1, top));
-    colours(Yes(), Yes(), false, a, min(b, top));
-    colours(No(), Yes(), false, a + 1, b - 1);
+    colours(Yes(), No(), false, olo, ob, a, eb);
+    colours(Yes(), Yes(), false, a, eb, a + 1, b - 1);
+    colours(No(), Yes(), false, a + 1, b - 1, 0, -1);
   } else {
-    colours(No(), Yes(), false, a, min(b, top));
-    colours(No(), Yes(), false, a + 1, b - 1);
-  }
-  if (!ready) {   // no line of this CTA has a phase
-    copy_wait();
-    __syncwarp();
-    if (pl.cs > 1) cluster_arrive();
-    __syncthreads();
+    colours(No(), Yes(), false, a, eb, a + 1, b - 1);
+    colours(No(), Yes(), false, a + 1, b - 1, 0, -1);
   }
   __syncwarp();
   if (pl.cs > 1) cluster_wait();
@@ -373,10 +430,9 @@ gs_plane_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T>
   }
 }
 
-// Shared memory of a plane CTA with `lines` own lines.
-template <typename T>
+// Shared memory of a plane CTA with `lines` own lines, V elements a thread.
+template <typename T, int V>
 static size_t plane_smem(const SGeom& g, int lines) {
-  constexpr int V = row_elems<T>();
   const size_t n = g.R == 1   ? PlaneLayout<1, V>(g).elems(lines)
                    : g.R == 2 ? PlaneLayout<2, V>(g).elems(lines)
                    : g.R == 4 ? PlaneLayout<4, V>(g).elems(lines)
@@ -385,43 +441,49 @@ static size_t plane_smem(const SGeom& g, int lines) {
 }
 
 constexpr size_t kMaxPlaneSmem = 227u << 10;
-constexpr size_t kPlaneSmemGoal = 50u << 10;   // four CTAs per SM
-constexpr int kMaxPlaneCtas = 8;               // portable cluster size
+constexpr size_t kPlaneSmemGoal = 112u << 10;   // two CTAs per SM
+constexpr int kMaxPlaneCtas = 8;                // portable cluster size
 
 // How a level's planes are split.  Up to 4 CTAs per plane while that makes at
 // most two CTAs per SM, with at least 8 lines each (a CTA recomputes up to 3
-// more); up to 8 where a CTA's lines would take more shared memory than four
-// CTAs per SM have (measured, 320^3 FP32 sweep: 775 us at one or two CTAs per SM,
-// 589 us at four; FP64 sweeps pay for the recomputed lines: 96^3 with 4 CTAs per
-// plane 197 us, with 8 213 us).  False: a line has more element groups than a
-// CTA threads, or its lines do not fit shared memory even so.
-template <typename T>
+// more); up to 8 where a CTA's lines would take more shared memory than two CTAs
+// per SM have.  (Measured, one sweep: 128^3 FP32 30 us with 4 CTAs per plane, 37
+// with 3 or 8; 96^3 FP64 177 us with 4, 226 with 3, 187 with 8.)  About 384
+// threads a CTA, twice that where only one fits an SM.  The next kernel may
+// start early only after grids that leave most SMs idle: otherwise its waiting
+// CTAs take the free places unevenly (96^3 FP64 V-cycle 595 us with an early start
+// everywhere, 493 us with this rule; 8^3 sweep 11.5 us without any, 9.5 us with).
+// False: a line has more element groups than a CTA threads, or its lines do not
+// fit shared memory even so.
+template <typename T, int V>
 static bool plane_plan(const SGeom& g, int num_sms, PlanePlan* out) {
-  constexpr int V = row_elems<T>();
   const int planes = std::max(g.de, 1);
   int cs = 1;
   auto lines_for = [&](int n) { return std::max(2, ((g.ny + n - 1) / n + 1) / 2 * 2); };
   while (cs < 4 && planes * (cs + 1) <= 2 * num_sms && lines_for(cs + 1) >= 8) ++cs;
-  while (cs < kMaxPlaneCtas && plane_smem<T>(g, lines_for(cs)) > kPlaneSmemGoal) ++cs;
-  if (plane_smem<T>(g, lines_for(cs)) > kMaxPlaneSmem) return false;
+  while (cs < kMaxPlaneCtas && plane_smem<T, V>(g, lines_for(cs)) > kPlaneSmemGoal) ++cs;
+  if (plane_smem<T, V>(g, lines_for(cs)) > kMaxPlaneSmem) return false;
   PlanePlan p;
   p.lines = lines_for(cs);
   p.cs = (g.ny + p.lines - 1) / p.lines;
   p.bx = (g.we + V - 1) / V;
-  if (p.bx > kPlaneThreads) return false;
+  if (2 * p.bx > kPlaneThreads) return false;
   // a phase has up to lines / 2 + 2 lines
-  const int rows = p.lines / 2 + 2, fit = std::max(1, kPlaneThreads / p.bx);
+  const int rows = p.lines / 2 + 2;
+  p.smem = plane_smem<T, V>(g, p.lines);
+  const int threads = p.smem > kPlaneSmemGoal ? kPlaneThreads : kPlaneThreads / 2;
+  const int fit = std::max(2, threads / p.bx & ~1);
   const int passes = (rows + fit - 1) / fit;
-  p.by = (rows + passes - 1) / passes;
-  p.smem = plane_smem<T>(g, p.lines);
+  p.by = ((rows + passes - 1) / passes + 1) & ~1;   // even (see the copies)
+  p.early = planes * p.cs <= num_sms / 4;
   *out = p;
   return true;
 }
 
-template <typename T, int R, bool VEC, int KIND, bool ZERO>
+template <typename T, int R, int V, bool VEC, int KIND, bool ZERO>
 static cudaError_t plane_launch_r(hpg_problem* h, const SGeom& g, const PlanePlan& pl, const T* r,
                                   const T* diag, T* z, int c0_done, cudaStream_t s) {
-  auto kern = gs_plane_kernel<T, R, VEC, KIND, ZERO>;
+  auto kern = gs_plane_kernel<T, R, V, VEC, KIND, ZERO>;
   if (pl.smem > (48u << 10)) {
     const cudaError_t e = cudaFuncSetAttribute(
         kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxPlaneSmem);
@@ -451,17 +513,39 @@ static cudaError_t plane_launch_r(hpg_problem* h, const SGeom& g, const PlanePla
   return cudaLaunchKernelEx(&cfg, kern, g, make_coef<T>(h->beta), pl, r, diag, z, c0_done);
 }
 
+// Elements a thread takes.  FP32 on large levels four where a line's parts and R
+// divide by it (they share each load, address and boundary test: 128^3 sweep 43
+// -> 32 us), else two (on small levels the longer code costs more than it saves:
+// 64^3 23 against 15 us); a line of odd width is read one by one.  FP64 one
+// (bound by its FMAs).
+template <typename T>
+static int plane_elems(const SGeom& g, const T* r, const T* z, bool* vec) {
+  *vec = true;
+  if (sizeof(T) == 8) return 1;
+  const bool large = (double)g.nx * g.ny * g.nz * g.R >= 600000.0;
+  if (large && (g.R == 1 || g.R >= 4) && whole_groups<T, 4>(g, r, z)) return 4;
+  *vec = whole_groups<T, 2>(g, r, z);
+  return 2;
+}
+
 template <typename T, int KIND, bool ZERO>
-static cudaError_t plane_launch(hpg_problem* h, const SGeom& g, const PlanePlan& pl, const T* r,
-                                const T* diag, T* z, int c0_done, cudaStream_t s) {
+static cudaError_t plane_launch(hpg_problem* h, const SGeom& g, int V, bool vec,
+                                const PlanePlan& pl, const T* r, const T* diag, T* z, int c0_done,
+                                cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {   // R-vectors are FP32
-    if (g.R == 8) return plane_launch_r<T, 8, true, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s);
-    if (g.R == 4) return plane_launch_r<T, 4, true, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s);
-    if (g.R == 2) return plane_launch_r<T, 2, true, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s);
-    if (!whole_groups<T, row_elems<T>()>(g, r, z))
-      return plane_launch_r<T, 1, false, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s);
+    if (g.R == 8)
+      return V == 4 ? plane_launch_r<T, 8, 4, true, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s)
+                    : plane_launch_r<T, 8, 2, true, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s);
+    if (g.R == 4)
+      return V == 4 ? plane_launch_r<T, 4, 4, true, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s)
+                    : plane_launch_r<T, 4, 2, true, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s);
+    if (g.R == 2) return plane_launch_r<T, 2, 2, true, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s);
+    if (V == 4) return plane_launch_r<T, 1, 4, true, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s);
+    if (!vec) return plane_launch_r<T, 1, 2, false, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s);
+    return plane_launch_r<T, 1, 2, true, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s);
+  } else {
+    return plane_launch_r<T, 1, 1, true, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s);
   }
-  return plane_launch_r<T, 1, true, KIND, ZERO>(h, g, pl, r, diag, z, c0_done, s);
 }
 
 template <typename T>
@@ -498,7 +582,12 @@ static int symgs_t(hpg_problem* h, int level, int R, const T* r, T* z, bool from
   const T* diag = level_diag<T>(L);
   int rc;
   PlanePlan pl;
-  if (!plane_plan<T>(g, h->num_sms, &pl)) {
+  bool vec = true;
+  const int V = plane_elems(g, r, z, &vec);
+  const bool fits = V == 4   ? plane_plan<T, 4>(g, h->num_sms, &pl)
+                    : V == 2 ? plane_plan<T, 2>(g, h->num_sms, &pl)
+                             : plane_plan<T, 1>(g, h->num_sms, &pl);
+  if (!fits || (R > 1 && !vec)) {
     for (int c = c0_done ? 1 : 0; c < kColours; ++c)
       if ((rc = stencil_colour_phase(h, level, R, c, from_zero, r, z, s))) return rc;
     for (int c = kColours - 2; c >= 0; --c)
@@ -518,19 +607,19 @@ static int symgs_t(hpg_problem* h, int level, int R, const T* r, T* z, bool from
     // r read, z written; not from zero: all of z read
     rc = launch(h, K_GS, level, prec, (half[0] * 2 + (from_zero ? 0.0 : all)) * sv, s,
                 "gs_plane_kernel", [&] {
-                  return from_zero ? plane_launch<T, kOddFwd, true>(h, g, pl, r, diag, z, c0_done, s)
-                                   : plane_launch<T, kOddFwd, false>(h, g, pl, r, diag, z, c0_done, s);
+                  return from_zero ? plane_launch<T, kOddFwd, true>(h, g, V, vec, pl, r, diag, z, c0_done, s)
+                                   : plane_launch<T, kOddFwd, false>(h, g, V, vec, pl, r, diag, z, c0_done, s);
                 }, phases(c0_done ? 1 : 0, 3));
     if (rc) return rc;
   }
   rc = launch(h, K_GS, level, prec, (half[1] * 2 + (from_zero ? half[0] : all)) * sv, s,
               "gs_plane_kernel", [&] {
-                return from_zero ? plane_launch<T, kEven, true>(h, g, pl, r, diag, z, 0, s)
-                                 : plane_launch<T, kEven, false>(h, g, pl, r, diag, z, 0, s);
+                return from_zero ? plane_launch<T, kEven, true>(h, g, V, vec, pl, r, diag, z, 0, s)
+                                 : plane_launch<T, kEven, false>(h, g, V, vec, pl, r, diag, z, 0, s);
               }, phases(4, 7) + phases(4, 6));
   if (rc || g.dO == 0) return rc;
   return launch(h, K_GS, level, prec, (half[0] * 2 + all) * sv, s, "gs_plane_kernel",
-                [&] { return plane_launch<T, kOddBwd, false>(h, g, pl, r, diag, z, 0, s); },
+                [&] { return plane_launch<T, kOddBwd, false>(h, g, V, vec, pl, r, diag, z, 0, s); },
                 phases(0, 3));
 }
 int stencil_symgs(hpg_problem* h, int level, int R, const float* r, float* z, bool from_zero,

@@ -60,6 +60,9 @@ static cudaError_t spmv_launch(hpg_problem* h, const SGeom& g, const T* x, const
   // four lines a thread once that leaves every SM several 256-thread blocks
   const bool big = (long long)g.we / V * g.ny * g.nz >= (long long)kRowLines * 2 * 256 * h->num_sms;
   const RowPlan pl = make_row_plan(g, V, big ? kRowLines : 1);
+  // small blocks spread few threads over all SMs, and FP64 work evenly (an SM
+  // has one FP64 unit, 16 cycles a warp instruction)
+  if (sizeof(T) == 8 || (long long)pl.threads <= 256LL * h->num_sms) block = 64;
   return kl(h, big ? stencil_spmv_kernel<T, R, VEC, kRowLines> : stencil_spmv_kernel<T, R, VEC, 1>,
             grid_for((long long)pl.threads + pl.pad, block), block, s, g, make_coef<T>(h->beta),
             pl, x, diag, y);
@@ -140,7 +143,7 @@ stencil_restrict_kernel(const __grid_constant__ SGeom gf, const __grid_constant_
       acc = fma(-d, m[u], acc);
       acc = fma(-c.a[4], rr[u], acc);
       if (x_edge(gf, 0, (int)e) || j == 0 || j == gf.ny - 1 || k == 0 || k == gf.nz - 1)
-        acc = fma(T(0), m[u], acc);
+        pad_slot(m[u], acc);
     } else {
       acc = sub_line(c, dyz, l[u], m[u], rr[u], acc);
     }

@@ -11,14 +11,11 @@
 //
 // An R-vector ([n_store][R], R right-hand sides of one problem) is the same
 // thing with every line R times as wide and a step in x of R elements, so all
-// kernels here take R at run time and serve one right-hand side with R = 1;
-// the arithmetic of a column does not depend on R.
+// kernels here serve one right-hand side with R = 1; the arithmetic of a column
+// does not depend on R.
 //
 // Values equal those of the ELL kernels bit for bit: same coefficients, same
-// order of the products.  A neighbour outside the grid is an ELL padding slot
-// there (column = own row, value 0); here it contributes nothing, and one
-// product 0 * (own entry) on boundary rows keeps the effect such a slot has
-// when the own entry is infinite or NaN.
+// order of the products (pad_slot covers neighbours outside the grid).
 #pragma once
 
 #include "hpg_internal.cuh"
@@ -87,9 +84,13 @@ template <int R, int V, bool VEC> struct XMask {
 
 template <typename T, int V> struct VecOf { using type = T; };
 template <> struct VecOf<float, 2> { using type = float2; };
+template <> struct VecOf<float, 4> { using type = float4; };
 __device__ __forceinline__ void unpack(float v, float (&o)[1]) { o[0] = v; }
 __device__ __forceinline__ void unpack(double v, double (&o)[1]) { o[0] = v; }
 __device__ __forceinline__ void unpack(float2 v, float (&o)[2]) { o[0] = v.x; o[1] = v.y; }
+__device__ __forceinline__ void unpack(float4 v, float (&o)[4]) {
+  o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
+}
 
 // The line whose even and odd parts start (at the thread's element) at ev, od;
 // in: the line exists.
@@ -173,23 +174,50 @@ __device__ __forceinline__ T half_sum(const Coef<T>& c, int dyz, const LinePts<T
 // Res. Dev. 34, 1990): with y = RN(1/26), q = RN(x y) and the exact remainder
 // x - 26 q, RN(q + remainder * y) is RN(x / 26) unless something under- or
 // overflows, which the range test leaves to the plain division.
-__device__ __forceinline__ float div_diag(float x) {
-  const float a = fabsf(x);
-  if (a >= 1e-30f && a <= 1e37f) {
-    constexpr float y = 1.0f / (float)kDiag;
-    const float q = x * y;
-    return fmaf(fmaf(-(float)kDiag, q, x), y, q);
-  }
-  return x / (float)kDiag;
+__device__ __forceinline__ bool div_safe(float x) {   // 2^-95 <= |x| < 2^123
+  return (__float_as_uint(x) & 0x7fffffffu) - 0x10000000u < 0x7d000000u - 0x10000000u;
 }
-__device__ __forceinline__ double div_diag(double x) {
-  const int e = __double2hiint(x) & 0x7ff00000;
-  if (e >= (200 << 20) && e <= (1900 << 20)) {   // 2^-823 .. 2^877
-    constexpr double y = 1.0 / kDiag;
-    const double q = x * y;
-    return fma(fma(-kDiag, q, x), y, q);
+__device__ __forceinline__ bool div_safe(double x) {  // 2^-823 <= |x| < 2^877
+  return ((unsigned)__double2hiint(x) & 0x7fffffffu) - (200u << 20) < (1700u << 20);
+}
+__device__ __forceinline__ float div_known(float x) {
+  constexpr float y = 1.0f / (float)kDiag;
+  const float q = x * y;
+  return fmaf(fmaf(-(float)kDiag, q, x), y, q);
+}
+__device__ __forceinline__ double div_known(double x) {
+  constexpr double y = 1.0 / kDiag;
+  const double q = x * y;
+  return fma(fma(-kDiag, q, x), y, q);
+}
+// Out of line: inlined, part of the division runs on the safe path as well
+// (FP64 sweeps 20 % slower).
+static __device__ __noinline__ float div_plain(float x) { return x / (float)kDiag; }
+static __device__ __noinline__ double div_plain(double x) { return x / kDiag; }
+template <typename T, int V> __device__ __forceinline__ void div_diag(T (&x)[V]) {
+  bool safe = true;
+  T q[V];
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    safe = safe && div_safe(x[v]);
+    q[v] = div_known(x[v]);
   }
-  return x / kDiag;
+  if (!safe) {
+#pragma unroll
+    for (int v = 0; v < V; ++v) q[v] = div_plain(x[v]);
+  }
+#pragma unroll
+  for (int v = 0; v < V; ++v) x[v] = q[v];
+}
+
+// What an ELL padding slot (own column, value 0) adds on boundary rows: nothing,
+// unless the own entry is infinite or NaN.  The test is on its exponent, so that
+// FP64 rows do not pay for a product.
+__device__ __forceinline__ void pad_slot(float own, float& acc) {
+  if ((__float_as_uint(own) & 0x7f800000u) == 0x7f800000u) acc = fmaf(0.0f, own, acc);
+}
+__device__ __forceinline__ void pad_slot(double own, double& acc) {
+  if ((__double2hiint(own) & 0x7ff00000) == 0x7ff00000) acc = fma(0.0, own, acc);
 }
 
 // Whether element e of an x-line's even (px 0) or odd part is its first or
@@ -306,8 +334,8 @@ __device__ __forceinline__ void stencil_rows(const SGeom& g, const Coef<T>& c, c
           const bool edge = j == 0 || j == g.ny - 1 || k == 0 || k == g.nz - 1;
 #pragma unroll
           for (int v = 0; v < V; ++v) {
-            if (edge || be[v]) ae[v] = fma(T(0), p.e[v], ae[v]);
-            if (edge || bo[v]) ao[v] = fma(T(0), p.o[v], ao[v]);
+            if (edge || be[v]) pad_slot(p.e[v], ae[v]);
+            if (edge || bo[v]) pad_slot(p.o[v], ao[v]);
           }
         }
       }
@@ -331,6 +359,8 @@ template <typename T, int V, bool VEC>
 __device__ __forceinline__ void store_elems(T* p, const bool (&m)[V], const T (&a)[V]) {
   if constexpr (VEC && V == 2) {
     if (m[0]) *reinterpret_cast<float2*>(p) = make_float2(a[0], a[1]);
+  } else if constexpr (VEC && V == 4) {
+    if (m[0]) *reinterpret_cast<float4*>(p) = make_float4(a[0], a[1], a[2], a[3]);
   } else {
 #pragma unroll
     for (int v = 0; v < V; ++v)
