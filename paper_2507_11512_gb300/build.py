@@ -20,7 +20,8 @@ LIB_NAME = "libhpgmxp.so"
 LIB_PATH = os.path.join(PKG_DIR, LIB_NAME)
 
 SOURCES = ["problem.cu", "sparse.cu", "stencil.cu", "gs_planes.cu",
-           "krylov.cu", "profile.cu", "vcycle_cluster.cu", "batch.cu"]
+           "krylov.cu", "profile.cu", "vcycle_cluster.cu", "vcycle_tail.cu",
+           "batch.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CFLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-fvisibility=hidden",
           "-I" + INCLUDE, "-I" + CSRC]

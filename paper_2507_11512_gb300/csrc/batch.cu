@@ -248,7 +248,8 @@ template <int R>
 static int mvcycle_t(hpg_problem* h, int l, const float* rhs, float* z, cudaStream_t s) {
   const Level& L = h->lev[l];
   BatchSpace* bs = h->batch;
-  int rc;
+  int rc = launch_vcycle_tail(h, l, R, rhs, z, false, s);
+  if (rc != HPG_ERR_UNSUPPORTED) return rc;
   if (l == h->nlev - 1) return stencil_symgs(h, l, R, rhs, z, true, false, s);
   if (h->pre == 0) {
     HPG_CK(cudaMemsetAsync(z, 0, sizeof(float) * L.g.n_store * R, s));

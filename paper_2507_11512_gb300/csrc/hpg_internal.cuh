@@ -300,6 +300,8 @@ namespace hpg {
 int prof_begin(hpg_problem* h, cudaStream_t s);
 void prof_end(hpg_problem* h, int slot, int cls, int level, int prec, double bytes,
               cudaStream_t s, int phases);
+// Counts work of a class that ran inside a launch recorded under another one.
+void prof_note(hpg_problem* h, int cls, int level, int prec, int phases);
 void destroy_profiler(hpg_problem* h);
 
 // Enqueues kernel<<<grid, block, 0, s>>>(args...), with the programmatic
@@ -357,6 +359,12 @@ int run_vcycle(hpg_problem* h, int level, hpg_prec prec, const void* r, void* z,
 // one kernel per phase).
 int launch_vcycle_cluster(hpg_problem* h, int level, hpg_prec prec, const void* r, void* z,
                           cudaStream_t s);
+// V-cycle from `level` down with every vector in one cluster's shared memory
+// (R right-hand sides); HPG_ERR_UNSUPPORTED where the level is too large for it.
+int launch_vcycle_tail(hpg_problem* h, int level, int R, const float* r, float* z, bool c0_done,
+                       cudaStream_t s);
+int launch_vcycle_tail(hpg_problem* h, int level, int R, const double* r, double* z, bool c0_done,
+                       cudaStream_t s);
 int launch_permute(hpg_problem* h, int level, int direction, hpg_prec in_prec,
                    const void* in, hpg_prec out_prec, void* out, cudaStream_t s);
 void destroy_workspace(hpg_problem* h);

@@ -18,7 +18,7 @@ struct ProfRec {
   int cls, level, prec;
   double bytes;
   int phases;
-  int ev;   // index of the start event; ev + 1 is the stop event
+  int ev;   // index of the start event; ev + 1 is the stop event (-1: only counted)
 };
 
 struct Profiler {
@@ -60,6 +60,11 @@ void prof_end(hpg_problem* h, int slot, int cls, int level, int prec, double byt
   p->recs.push_back(ProfRec{cls, level, prec, bytes, phases, slot});
 }
 
+void prof_note(hpg_problem* h, int cls, int level, int prec, int phases) {
+  if (!h->prof || !h->prof->on) return;
+  h->prof->recs.push_back(ProfRec{cls, level, prec, 0.0, phases, -1});
+}
+
 void destroy_profiler(hpg_problem* h) {
   if (!h->prof) return;
   for (cudaEvent_t e : h->prof->events) cudaEventDestroy(e);
@@ -97,9 +102,11 @@ HPG_API int hpg_profile_report(hpg_problem_t* h, hpg_kernel_stat* out, int capac
   Profiler* p = h->prof;
   std::map<std::tuple<int, int, int>, hpg_kernel_stat> agg;
   for (const ProfRec& r : p->recs) {
-    HPG_CK(cudaEventSynchronize(p->events[r.ev + 1]));
     float ms = 0.f;
-    HPG_CK(cudaEventElapsedTime(&ms, p->events[r.ev], p->events[r.ev + 1]));
+    if (r.ev >= 0) {
+      HPG_CK(cudaEventSynchronize(p->events[r.ev + 1]));
+      HPG_CK(cudaEventElapsedTime(&ms, p->events[r.ev], p->events[r.ev + 1]));
+    }
     hpg_kernel_stat& st = agg[std::make_tuple(r.cls, r.level, r.prec)];
     st.name = kernel_class_name(r.cls);
     st.level = r.level;

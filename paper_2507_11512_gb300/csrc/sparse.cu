@@ -705,6 +705,15 @@ static int coarsest_sweep(hpg_problem* h, int l, const T* r, T* z, bool c0_done,
   return symgs<T>(h, l, r, z, true, st, s);
 }
 
+// The rest of the V-cycle in one kernel where level l is small, unless an
+// option asks for a sweep of its own there.
+template <typename T>
+static int vcycle_tail(hpg_problem* h, int l, const T* r, T* z, bool c0_done, cudaStream_t s) {
+  if (h->coarse_cluster || h->coarse_cta || h->gs_halo || h->gs_pipeline > 1)
+    return HPG_ERR_UNSUPPORTED;
+  return launch_vcycle_tail(h, l, 1, r, z, c0_done, s);
+}
+
 // Whether the restriction from level l also runs the first phase (colour 0)
 // of level l+1's first sweep from zero: true when that sweep goes through the
 // launched phases (not the cluster kernel) and starts from zero (the
@@ -721,6 +730,8 @@ static int vcycle_t(hpg_problem* h, int l, const T* r, T* z, cudaStream_t s,
   if (c0_done) st.last = 0;   // colour 0 of the first sweep came with the restriction
   int rc = launch_vcycle_cluster(h, l, Prec<T>::idx == 0 ? HPG_FP64 : HPG_FP32, r, z, s);
   if (rc != HPG_ERR_UNSUPPORTED) return rc;   // small level: the rest runs in one cluster
+  rc = vcycle_tail<T>(h, l, r, z, c0_done, s);
+  if (rc != HPG_ERR_UNSUPPORTED) return rc;
   if (l == h->nlev - 1) return coarsest_sweep<T>(h, l, r, z, c0_done, s);
   if (h->pre == 0) {
     HPG_CK(cudaMemsetAsync(z, 0, sizeof(T) * L.g.n_store, s));
@@ -878,7 +889,8 @@ static int vcycle_noalloc_t(hpg_problem* h, int l, const T* r, T* z, T* const* c
   const Level& L = h->lev[l];
   SweepState st;
   if (c0_done) st.last = 0;   // colour 0 of the first sweep came with the restriction
-  int rc;
+  int rc = vcycle_tail<T>(h, l, r, z, c0_done, s);
+  if (rc != HPG_ERR_UNSUPPORTED) return rc;
   if (l == h->nlev - 1) return coarsest_sweep<T>(h, l, r, z, c0_done, s);
   if (h->pre == 0) {
     HPG_CK(cudaMemsetAsync(z, 0, sizeof(T) * L.g.n_store, s));
