@@ -47,6 +47,10 @@ def _ptr(a):
 def _stream(stream):
     if stream is None:
         torch = _torch()
+        if torch.cuda.is_initialized():
+            # the handle alone: asking for availability and building a Stream object
+            # took half of a small product's 20 us call
+            return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
         if torch.cuda.is_available():
             return torch.cuda.current_stream().cuda_stream
         return None
