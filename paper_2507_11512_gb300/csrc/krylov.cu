@@ -168,16 +168,11 @@ __device__ __forceinline__ A warp_max(A v) {
 
 // ------------------------------------------------------------ vector access
 // Four consecutive rows of a vector (16-byte aligned: storage rows come in
-// multiples of 32).  Streaming variants for data read once, L2 variants for
-// data read twice in one pass.
+// multiples of 32), streaming.
 template <typename T> struct Vec4;
 template <> struct Vec4<float> {
   static __device__ __forceinline__ void ld_cs(const float* p, float (&v)[4]) {
     const float4 t = __ldcs(reinterpret_cast<const float4*>(p));
-    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
-  }
-  static __device__ __forceinline__ void ld_cg(const float* p, float (&v)[4]) {
-    const float4 t = __ldcg(reinterpret_cast<const float4*>(p));
     v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
   }
   static __device__ __forceinline__ void st(float* p, const float (&v)[4]) {
@@ -188,11 +183,6 @@ template <> struct Vec4<double> {
   static __device__ __forceinline__ void ld_cs(const double* p, double (&v)[4]) {
     const double2 a = __ldcs(reinterpret_cast<const double2*>(p));
     const double2 b = __ldcs(reinterpret_cast<const double2*>(p) + 1);
-    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
-  }
-  static __device__ __forceinline__ void ld_cg(const double* p, double (&v)[4]) {
-    const double2 a = __ldcg(reinterpret_cast<const double2*>(p));
-    const double2 b = __ldcg(reinterpret_cast<const double2*>(p) + 1);
     v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
   }
   static __device__ __forceinline__ void st(double* p, const double (&v)[4]) {
@@ -255,67 +245,68 @@ __host__ __device__ constexpr int pass_min_blocks() {
 }
 
 // V consecutive elements (V * sizeof(E) bytes, aligned to that size up to 16:
-// storage rows come in multiples of 32), streaming loads / plain stores.
-// FP32 and FP64 elements move as float/double vector types (moving them
-// through integer vectors measured up to 2x slower for FP64 passes); 2-byte
-// elements move as packed integers.
-// Load policy: KEEP leaves the lines in L2 (a later pass reads them again),
-// otherwise they stream (evict-first).
-template <bool KEEP, typename P>
-__device__ __forceinline__ P ld_policy(const P* p) {
-  if constexpr (KEEP) return __ldcg(p);
-  else return __ldcs(p);
+// storage rows come in multiples of 32) past L1 with an L2 policy chosen at run
+// time: evict-first where nothing reads the lines again soon, normal where a
+// later pass does.  FP32 and FP64 elements move as float / double vectors
+// (through integer vectors FP64 passes measured up to 2x slower); 2-byte elements
+// as packed integers.
+__device__ __forceinline__ unsigned long long l2_policy(bool keep) {
+  unsigned long long first, normal;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(first));
+  asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(normal));
+  return keep ? normal : first;
 }
-
-template <typename E, int V, bool KEEP = false>
-__device__ __forceinline__ void ld_group(const E* p, E (&v)[V]) {
+#define HPG_LD "ld.global.L1::no_allocate.L2::cache_hint"
+template <typename E, int V>
+__device__ __forceinline__ void ld_group(const E* p, E (&v)[V], unsigned long long pol) {
   if constexpr (sizeof(E) == 8 && V == 1) {
-    v[0] = ld_policy<KEEP>(p);
+    asm volatile(HPG_LD ".f64 %0, [%1], %2;" : "=d"(v[0]) : "l"(p), "l"(pol));
   } else if constexpr (sizeof(E) == 8) {
     static_assert(V % 2 == 0, "FP64 row groups of 1 or 2k elements");
 #pragma unroll
-    for (int i = 0; i < V / 2; ++i) {
-      const double2 t = ld_policy<KEEP>(reinterpret_cast<const double2*>(p) + i);
-      v[2 * i] = t.x;
-      v[2 * i + 1] = t.y;
-    }
+    for (int i = 0; i < V / 2; ++i)
+      asm volatile(HPG_LD ".v2.f64 {%0, %1}, [%2], %3;"
+                   : "=d"(v[2 * i]), "=d"(v[2 * i + 1]) : "l"(p + 2 * i), "l"(pol));
   } else if constexpr (sizeof(E) == 4 && V % 4 == 0) {
 #pragma unroll
-    for (int i = 0; i < V / 4; ++i) {
-      const float4 t = ld_policy<KEEP>(reinterpret_cast<const float4*>(p) + i);
-      v[4 * i] = t.x;
-      v[4 * i + 1] = t.y;
-      v[4 * i + 2] = t.z;
-      v[4 * i + 3] = t.w;
-    }
+    for (int i = 0; i < V / 4; ++i)
+      asm volatile(HPG_LD ".v4.f32 {%0, %1, %2, %3}, [%4], %5;"
+                   : "=f"(v[4 * i]), "=f"(v[4 * i + 1]), "=f"(v[4 * i + 2]), "=f"(v[4 * i + 3])
+                   : "l"(p + 4 * i), "l"(pol));
   } else if constexpr (sizeof(E) == 4 && V == 2) {
-    const float2 t = ld_policy<KEEP>(reinterpret_cast<const float2*>(p));
-    v[0] = t.x;
-    v[1] = t.y;
+    asm volatile(HPG_LD ".v2.f32 {%0, %1}, [%2], %3;"
+                 : "=f"(v[0]), "=f"(v[1]) : "l"(p), "l"(pol));
   } else if constexpr (sizeof(E) == 4) {
     static_assert(V == 1, "FP32 row groups of 1, 2 or 4k elements");
-    v[0] = ld_policy<KEEP>(p);
+    asm volatile(HPG_LD ".f32 %0, [%1], %2;" : "=f"(v[0]) : "l"(p), "l"(pol));
   } else {
     static_assert(sizeof(E) == 2, "2-, 4- or 8-byte elements");
     constexpr int bytes = 2 * V;
     if constexpr (bytes % 16 == 0) {
 #pragma unroll
       for (int i = 0; i < bytes / 16; ++i) {
-        const uint4 t = ld_policy<KEEP>(reinterpret_cast<const uint4*>(p) + i);
+        uint4 t;
+        asm volatile(HPG_LD ".v4.u32 {%0, %1, %2, %3}, [%4], %5;"
+                     : "=r"(t.x), "=r"(t.y), "=r"(t.z), "=r"(t.w)
+                     : "l"(reinterpret_cast<const uint4*>(p) + i), "l"(pol));
         memcpy(reinterpret_cast<char*>(v) + 16 * i, &t, 16);
       }
     } else if constexpr (bytes == 8) {
-      const uint2 t = ld_policy<KEEP>(reinterpret_cast<const uint2*>(p));
+      uint2 t;
+      asm volatile(HPG_LD ".v2.u32 {%0, %1}, [%2], %3;"
+                   : "=r"(t.x), "=r"(t.y) : "l"(p), "l"(pol));
       memcpy(v, &t, 8);
-    } else if constexpr (bytes == 4) {
-      const unsigned t = ld_policy<KEEP>(reinterpret_cast<const unsigned*>(p));
-      memcpy(v, &t, 4);
     } else {
-      static_assert(bytes == 2, "2-byte row groups of 1, 2, 4 or 8k elements");
-      const unsigned short t = ld_policy<KEEP>(reinterpret_cast<const unsigned short*>(p));
-      memcpy(v, &t, 2);
+      static_assert(bytes == 4, "2-byte row groups of 2, 4 or 8k elements");
+      unsigned t;
+      asm volatile(HPG_LD ".u32 %0, [%1], %2;" : "=r"(t) : "l"(p), "l"(pol));
+      memcpy(v, &t, 4);
     }
   }
+}
+#undef HPG_LD
+template <typename E, int V> __device__ __forceinline__ void ld_group(const E* p, E (&v)[V]) {
+  ld_group<E, V>(p, v, l2_policy(false));
 }
 template <typename E, int V>
 __device__ __forceinline__ void st_group(E* p, const E (&v)[V]) {
@@ -473,6 +464,10 @@ __device__ void arnoldi_givens_warp(double beta, int k, double* __restrict__ H, 
                                     unsigned long long next) {
   if ((threadIdx.x & 31) != 0) return;
   double* hc = H + (long long)k * ldh;
+  // the loads first: none depends on beta or on a store below
+  const double a = __ldcg(hc + k);   // H[k,k] after the old rotations
+  const double tk = t[k], rho0 = st->rho0, tol = st->tol;
+  const int iters = st->iters + 1, maxit = st->maxit, m = st->m;
   st->beta = beta;
   bool go = false;
   if (!isfinite(beta)) {
@@ -480,7 +475,6 @@ __device__ void arnoldi_givens_warp(double beta, int k, double* __restrict__ H, 
     st->active = 0;
     hc[k + 1] = beta;
   } else {
-    const double a = __ldcg(hc + k);   // H[k,k] after the old rotations
     const double mu = hypot(a, beta);
     if (!(mu > 0.0) || !isfinite(mu)) {
       st->status = isfinite(mu) ? HPG_ERR_BREAKDOWN : HPG_ERR_NAN;
@@ -492,14 +486,13 @@ __device__ void arnoldi_givens_warp(double beta, int k, double* __restrict__ H, 
       sn[k] = sv;
       hc[k] = mu;
       hc[k + 1] = 0.0;
-      const double tk = t[k];
       t[k + 1] = -sv * tk;
       t[k] = c * tk;
       const double rho = fabs(-sv * tk);
       st->rho = rho;
       st->k = k + 1;
-      st->iters += 1;
-      go = !(rho / st->rho0 < st->tol || st->iters >= st->maxit || k + 1 >= st->m);
+      st->iters = iters;
+      go = !(rho / rho0 < tol || iters >= maxit || k + 1 >= m);
       st->active = go ? 1 : 0;
     }
   }
@@ -532,21 +525,6 @@ cgs2_pass_kernel(const B* __restrict__ Q, long long ns, int ncol, const T* w,
   constexpr bool MAXLAST = S && KIND == kFinal;
   __shared__ T shc[KMAX];   // h1 (reorth) or h2 (final), scaled for a 2-byte basis
   __shared__ double sums[KMAX];
-  pdl_trigger();
-  pdl_wait();   // w, Q and h come from earlier kernels
-  if (KIND != kGemvT) {
-    const double* hc = KIND == kReorth ? h1 : h2;
-    for (int j = threadIdx.x; j < ncol; j += kRedThreads)
-      shc[j] = (T)(S ? ld_dep(hc + j) * (double)ld_dep(qscale + j) : ld_dep(hc + j));
-    __syncthreads();
-  }
-  // the rotations that do not need beta, by one warp while the pass streams;
-  // block 0 takes its ticket (and the last block reads H) only afterwards
-  if (KIND == kFinal && blockIdx.x == 0 && threadIdx.x < 32)
-    arnoldi_rotate_warp<KMAX>(ncol - 1, h1, h2, H, ldh, cs, sn);
-  T acc[KMAX];
-#pragma unroll
-  for (int j = 0; j < KMAX; ++j) acc[j] = T(0);
   // Zig-zag over the passes (zigzag != 0, basis vectors much smaller than
   // L2): the reorth pass walks the rows backwards, so it starts on the rows
   // the GEMVT pass read last (still in L2), and the final pass forwards again;
@@ -554,58 +532,87 @@ cgs2_pass_kernel(const B* __restrict__ Q, long long ns, int ncol, const T* w,
   // faster 128^3 GMRES(30) solves; with 131 MB vectors (320^3) the backward
   // pass streamed at half the rate of a forward one.
   const bool rev = zigzag && KIND == kReorth;
-  const bool keep = zigzag && KIND != kFinal;
+  const unsigned long long pol = l2_policy(zigzag && KIND != kFinal);
   const long long ng = ns / V;
   const long long stride = (long long)gridDim.x * kRedThreads;
-  auto load = [&](long long g, T (&wr)[V], B (&q)[KMAX][V]) {
-    if (keep) {
-      ld_group<T, V, true>(w + g * V, wr);
-#pragma unroll
-      for (int j = 0; j < KMAX; ++j)
-        if (j < ncol) ld_group<B, V, true>(Q + j * ns + g * V, q[j]);
-    } else {
-      ld_group<T, V, false>(w + g * V, wr);
-#pragma unroll
-      for (int j = 0; j < KMAX; ++j)
-        if (j < ncol) ld_group<B, V, false>(Q + j * ns + g * V, q[j]);
-    }
+  T wr[V];
+  B q[KMAX][V];
+  auto load_w = [&](long long gi, T (&o)[V]) {
+    ld_group<T, V>(w + (rev ? ng - 1 - gi : gi) * V, o, pol);
   };
-  for (long long gi = blockIdx.x * (long long)kRedThreads + threadIdx.x; gi < ng; gi += stride) {
-    const long long g = rev ? ng - 1 - gi : gi;
-    T wr[V];
-    B q[KMAX][V];
-    load(g, wr, q);
-    const long long r0 = g * V;
+  auto load_q = [&](long long gi, int j) {
+    ld_group<B, V>(Q + j * ns + (rev ? ng - 1 - gi : gi) * V, q[j], pol);
+  };
+  long long gi = blockIdx.x * (long long)kRedThreads + threadIdx.x;
+  // A pass lets the next one start only after its own wait, so when the reorth
+  // or the final pass runs, every kernel before its predecessor has finished: Q
+  // (and for the reorth pass w) is final, and its first row group is loaded while
+  // the predecessor's last block still adds the partial sums.
+  constexpr bool kEarly = KIND != kGemvT;
+  if (kEarly && gi < ng) {
+    if (KIND == kReorth) load_w(gi, wr);
+#pragma unroll
+    for (int j = 0; j < KMAX; ++j)
+      if (j < ncol) load_q(gi, j);
+  }
+  pdl_wait();   // h (and w, Q) come from earlier kernels
+  pdl_trigger();
+  if (KIND != kGemvT) {
+    const double* hc = KIND == kReorth ? h1 : h2;
+    for (int j = threadIdx.x; j < ncol; j += kRedThreads)
+      shc[j] = (T)(S ? ld_dep(hc + j) * (double)ld_dep(qscale + j) : ld_dep(hc + j));
+    __syncthreads();
+  }
+  // the rotations that do not need beta, by one warp of the last block (the one
+  // with the fewest rows) while the pass streams; it takes its ticket (and the
+  // last block to do so reads H) only afterwards
+  if (KIND == kFinal && blockIdx.x == gridDim.x - 1 && threadIdx.x < 32)
+    arnoldi_rotate_warp<KMAX>(ncol - 1, h1, h2, H, ldh, cs, sn);
+  T acc[KMAX];
+#pragma unroll
+  for (int j = 0; j < KMAX; ++j) acc[j] = T(0);
+  if (gi < ng) {
+    if (KIND != kReorth) load_w(gi, wr);
+    if (!kEarly) {
+#pragma unroll
+      for (int j = 0; j < KMAX; ++j)
+        if (j < ncol) load_q(gi, j);
+    }
+  }
+  // In the GEMVT and final passes a column's registers are refilled with the next
+  // row group's values as soon as they have been used, so the loads of a thread
+  // never pause (128^3, 17 columns: GEMVT 41.1 -> 38.2 us, final 40.5 -> 34.1); the
+  // reorth pass, which uses them twice, was slower that way (28.5 -> 30.4 us at 16
+  // columns).
+  for (; gi < ng; gi += stride) {
+    const long long gn = gi + stride;
+    const bool more = gn < ng;
+    const long long r0 = (rev ? ng - 1 - gi : gi) * V;
+    T wn[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) wn[v] = T(0);
+    if (more) load_w(gn, wn);
     if (KIND == kGemvT) {
 #pragma unroll
       for (int j = 0; j < KMAX; ++j)
         if (j < ncol) {
 #pragma unroll
           for (int v = 0; v < V; ++v) acc[j] = fma((T)basis_to(q[j][v]), wr[v], acc[j]);
+          if (more) load_q(gn, j);
         }
     } else {
-      // s = (Q c)_row, c = h1 or h2.  Rows always sum over j in ascending
-      // order; for a 2-byte basis (8 rows per thread) the column-outer order
-      // reads each coefficient from shared memory once per row group
-      // (measured faster there, slower for FP32/FP64 rows).
+      // s = (Q c)_row, c = h1 or h2; rows sum over j in ascending order
       T sc[V];
 #pragma unroll
       for (int v = 0; v < V; ++v) sc[v] = T(0);
-      if constexpr (S) {
 #pragma unroll
-        for (int j = 0; j < KMAX; ++j)
-          if (j < ncol) {
-            const T c = shc[j];
+      for (int j = 0; j < KMAX; ++j)
+        if (j < ncol) {
+          const T c = shc[j];
 #pragma unroll
-            for (int v = 0; v < V; ++v) sc[v] = fma((T)basis_to(q[j][v]), c, sc[v]);
-          }
-      } else {
-#pragma unroll
-        for (int v = 0; v < V; ++v)
-#pragma unroll
-          for (int j = 0; j < KMAX; ++j)
-            if (j < ncol) sc[v] = fma((T)basis_to(q[j][v]), shc[j], sc[v]);
-      }
+          for (int v = 0; v < V; ++v) sc[v] = fma((T)basis_to(q[j][v]), c, sc[v]);
+          if (KIND == kFinal && more) load_q(gn, j);
+        }
 #pragma unroll
       for (int v = 0; v < V; ++v) wr[v] = wr[v] - sc[v];   // w' = w - Q h1 / w'' = w' - Q h2
       st_group<T, V>(wout + r0, wr);
@@ -616,6 +623,11 @@ cgs2_pass_kernel(const B* __restrict__ Q, long long ns, int ncol, const T* w,
 #pragma unroll
             for (int v = 0; v < V; ++v) acc[j] = fma((T)basis_to(q[j][v]), wr[v], acc[j]);
           }
+        if (more) {
+#pragma unroll
+          for (int j = 0; j < KMAX; ++j)
+            if (j < ncol) load_q(gn, j);
+        }
       } else {
 #pragma unroll
         for (int v = 0; v < V; ++v) {
@@ -624,6 +636,8 @@ cgs2_pass_kernel(const B* __restrict__ Q, long long ns, int ncol, const T* w,
         }
       }
     }
+#pragma unroll
+    for (int v = 0; v < V; ++v) wr[v] = wn[v];
   }
   const int nred = KIND == kFinal ? (MAXLAST ? 2 : 1) : ncol;
   if (!block_partials_last<T, KMAX, MAXLAST>(acc, nred, partials, counter, sums)) return;
@@ -929,19 +943,13 @@ template <typename T> constexpr int prec_of() { return sizeof(T) == 8 ? HPG_FP64
 // Basis vectors up to this size take the zig-zag pass order (cgs2_pass_kernel).
 constexpr long long kZigZagVectorBytes = 32LL << 20;
 
-// Grid of a CGS2 pass: every resident block of the instantiation (one wave
-// of grid-stride blocks), at most the G blocks the partials are sized for.
+// Grid of a CGS2 pass: one wave of grid-stride blocks, at most the G blocks the
+// partials are sized for.  The grid fixes which rows a partial sum covers, and so
+// the rounding of every solve: these are constants, not an occupancy query.
 template <typename T, typename B, int KMAX, int KIND>
 static int pass_grid(hpg_problem* h) {
-  static int per_sm = 0;
-  if (per_sm == 0) {
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per_sm, cgs2_pass_kernel<T, B, KMAX, KIND>, kRedThreads, 0) != cudaSuccess ||
-        per_sm < 1) {
-      cudaGetLastError();
-      per_sm = 1;
-    }
-  }
+  constexpr int per_sm = sizeof(B) == 2 && KMAX == 64 && KIND == kFinal
+                             ? 2 : pass_min_blocks<T, KMAX>();
   const int g = per_sm * h->num_sms;
   return g < h->ws->G ? g : h->ws->G;
 }
