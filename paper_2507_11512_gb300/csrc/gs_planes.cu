@@ -444,11 +444,12 @@ constexpr size_t kMaxPlaneSmem = 227u << 10;
 constexpr size_t kPlaneSmemGoal = 112u << 10;   // two CTAs per SM
 constexpr int kMaxPlaneCtas = 8;                // portable cluster size
 
-// How a level's planes are split.  Up to 4 CTAs per plane while that makes at
-// most two CTAs per SM, with at least 8 lines each (a CTA recomputes up to 3
-// more); up to 8 where a CTA's lines would take more shared memory than two CTAs
-// per SM have.  (Measured, one sweep: 128^3 FP32 30 us with 4 CTAs per plane, 37
-// with 3 or 8; 96^3 FP64 177 us with 4, 226 with 3, 187 with 8.)  About 384
+// How a level's planes are split.  FP32: up to 4 CTAs per plane while that makes
+// at most two CTAs per SM; FP64, whose time is the busiest SM's FP64 work, up to 5
+// and three per SM; with at least 8 lines each (a CTA recomputes up to 3 more).
+// Up to 8 where a CTA's lines would take more shared memory than two CTAs per SM
+// have.  (Measured, one sweep: 128^3 FP32 30 us with 4 CTAs per plane, 37 with 3 or
+// 8; 96^3 FP64 150 us with 5, 177 with 4, 226 with 3, 187 with 8.)  About 384
 // threads a CTA, twice that where only one fits an SM.  The next kernel may
 // start early only after grids that leave most SMs idle: otherwise its waiting
 // CTAs take the free places unevenly (96^3 FP64 V-cycle 595 us with an early start
@@ -460,7 +461,8 @@ static bool plane_plan(const SGeom& g, int num_sms, PlanePlan* out) {
   const int planes = std::max(g.de, 1);
   int cs = 1;
   auto lines_for = [&](int n) { return std::max(2, ((g.ny + n - 1) / n + 1) / 2 * 2); };
-  while (cs < 4 && planes * (cs + 1) <= 2 * num_sms && lines_for(cs + 1) >= 8) ++cs;
+  constexpr int most = sizeof(T) == 8 ? 5 : 4, per_sm = sizeof(T) == 8 ? 3 : 2;
+  while (cs < most && planes * (cs + 1) <= per_sm * num_sms && lines_for(cs + 1) >= 8) ++cs;
   while (cs < kMaxPlaneCtas && plane_smem<T, V>(g, lines_for(cs)) > kPlaneSmemGoal) ++cs;
   if (plane_smem<T, V>(g, lines_for(cs)) > kMaxPlaneSmem) return false;
   PlanePlan p;

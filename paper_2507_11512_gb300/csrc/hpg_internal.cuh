@@ -72,15 +72,8 @@ __device__ inline int colour_of_row(const Geom& g, long long row) {
 }
 
 // ------------------------------------------------------------- cached loads
-// Matrix entries are read once per sweep: stream them past L1 and mark them
-// evict-first in L2 so that the vectors stay resident.
-__device__ __forceinline__ float ld_stream(const float* p) { return __ldcs(p); }
-__device__ __forceinline__ double ld_stream(const double* p) { return __ldcs(p); }
-__device__ __forceinline__ int ld_stream(const int* p) { return __ldcs(p); }
-
-// Matrix load of the bandwidth-variant kernels: streamed (evict-first), or
-// cached normally where the slice is read again soon (a streamed level's
-// kept colour phases, levels below the streaming size).
+// Matrix load of the pipelined sweep: streamed (evict-first), or cached normally
+// on levels below the streaming size.
 template <bool STREAM, typename V>
 __device__ __forceinline__ V ld_matrix(const V* p) {
   if (STREAM) return __ldcs(p);
@@ -284,8 +277,7 @@ struct hpg_problem {
   bool coarse_cluster = false;    // coarse levels of a V-cycle in one cluster kernel
   bool gs_halo = false;           // streamed GS phases stage z's neighbourhood in shared memory
   bool coarse_cta = false;        // coarsest level's sweep in one CTA when it fits
-  long long pdl_rows = 16384;     // latency-variant GS phases launched programmatically up
-                                  // to this many rows
+  long long pdl_rows = 16384;     // HPG_OPT_PDL_ROWS (accepted, without effect)
   int gs_pipeline = 1;            // pipelined sweep kernel: 0 never; on streamed levels
                                   // 1 FP64 sweeps after hpg_inject_stall, 2 always;
                                   // 3 every level
@@ -365,6 +357,12 @@ int launch_vcycle_tail(hpg_problem* h, int level, int R, const float* r, float* 
                        cudaStream_t s);
 int launch_vcycle_tail(hpg_problem* h, int level, int R, const double* r, double* z, bool c0_done,
                        cudaStream_t s);
+// `sweeps` symmetric sweeps of a small level in the same kernel (one launch);
+// HPG_ERR_UNSUPPORTED likewise.
+int launch_small_sweeps(hpg_problem* h, int level, const float* r, float* z, int sweeps,
+                        bool from_zero, cudaStream_t s);
+int launch_small_sweeps(hpg_problem* h, int level, const double* r, double* z, int sweeps,
+                        bool from_zero, cudaStream_t s);
 int launch_permute(hpg_problem* h, int level, int direction, hpg_prec in_prec,
                    const void* in, hpg_prec out_prec, void* out, cudaStream_t s);
 void destroy_workspace(hpg_problem* h);

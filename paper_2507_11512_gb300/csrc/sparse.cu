@@ -1,14 +1,8 @@
-// Stencil-matrix kernels: ELLPACK SpMV, the FP64 outer residual, one colour
-// phase of multicolour Gauss-Seidel, the fused residual-restriction and the
-// injection prolongation, plus the V-cycle that strings them together.
-//
-// Kernels read the slot-major ELL arrays by level size: streaming
-// (evict-first) where the matrix is larger than L2, normally cached on
-// mid-size levels, and marked evict-last on the small coarse levels (read by
-// every V-cycle; measured on GB300 at 128^3, this cut a V-cycle from 570 to
-// 494 us).  x is gathered through the read-only path; rows of one colour block
-// are contiguous, so a warp reads each slot of 32 consecutive rows as one
-// 128-byte (FP32) or 256-byte (FP64) transaction.
+// The V-cycle and the smoother: which kernels run on a level, the prolongation,
+// and the kernels on the stored (slot-major ELL) matrix that the implementation
+// options select -- the pipelined sweep, TMA-tiled colour phases and the coarsest
+// level in one CTA.  Without options every operator is evaluated straight from
+// the grid (stencil.cuh); results are the same.
 
 #include <limits.h>
 #include <string.h>
@@ -705,13 +699,15 @@ static int coarsest_sweep(hpg_problem* h, int l, const T* r, T* z, bool c0_done,
   return symgs<T>(h, l, r, z, true, st, s);
 }
 
-// The rest of the V-cycle in one kernel where level l is small, unless an
-// option asks for a sweep of its own there.
+// Whether no option asks for sweeps of a kind of their own.
+static bool own_kernels(const hpg_problem* h) {
+  return !h->coarse_cluster && !h->coarse_cta && !h->gs_halo && h->gs_pipeline <= 1;
+}
+
+// The rest of the V-cycle in one kernel where level l is small.
 template <typename T>
 static int vcycle_tail(hpg_problem* h, int l, const T* r, T* z, bool c0_done, cudaStream_t s) {
-  if (h->coarse_cluster || h->coarse_cta || h->gs_halo || h->gs_pipeline > 1)
-    return HPG_ERR_UNSUPPORTED;
-  return launch_vcycle_tail(h, l, 1, r, z, c0_done, s);
+  return own_kernels(h) ? launch_vcycle_tail(h, l, 1, r, z, c0_done, s) : HPG_ERR_UNSUPPORTED;
 }
 
 // Whether the restriction from level l also runs the first phase (colour 0)
@@ -773,8 +769,12 @@ static int smooth_t(hpg_problem* h, int level, const T* r, T* z, int sweeps, boo
     }
     return HPG_OK;
   }
-  SweepState st;
   int rc;
+  if (own_kernels(h)) {
+    rc = launch_small_sweeps(h, level, r, z, sweeps, from_zero, s);
+    if (rc != HPG_ERR_UNSUPPORTED) return rc;
+  }
+  SweepState st;
   for (int it = 0; it < sweeps; ++it)
     if ((rc = symgs<T>(h, level, r, z, from_zero && it == 0, st, s))) return rc;
   return HPG_OK;

@@ -32,6 +32,9 @@ constexpr size_t kTailSmem = 227u << 10;
 // cluster made its V-cycle 125 instead of 80 us, a 24^3 FP64 level 180 instead of
 // 158 (eight SMs' FP64 units against all).
 constexpr long long kTailPoints32 = 33000, kTailPoints64 = 5000;
+// A sweep alone pays for one launch instead of three (15.3 -> 10.9 us of host time)
+// but loads and stores the level (16^3 13.5 us against 11.1, 32^3 19 against 11).
+constexpr long long kTailSweepPoints32 = 16384;
 
 // Quotients by a fixed divisor (below 2^16, dividends likewise).
 struct FastDiv {
@@ -63,6 +66,7 @@ template <typename T> struct TailLevel {
 template <typename T> struct TailParams {
   int nlev, nops, ctas, threads;
   int ppc;                     // planes per CTA on the first level
+  int given;                   // z enters as given (sweeps), not as 0
   int sp, elems;               // offset of the sums up to the plane below; elements in all
   Coef<T> c;
   const T* r;
@@ -98,7 +102,8 @@ vcycle_tail_kernel(const __grid_constant__ TailParams<T> P) {
   unsigned rank;
   asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
   pdl_trigger();
-  for (int i = tid; i < P.elems; i += blockDim.x) sm[i] = T(0);
+  for (int i = tid; i < (P.elems * (int)sizeof(T) + 15) / 16; i += blockDim.x)
+    reinterpret_cast<float4*>(tail_smem)[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   __syncthreads();
   // first plane of this CTA on level l, and of the next CTA
   auto first_plane = [&](int l, int c) { return ((c * P.ppc) + (1 << l) - 1) >> l; };
@@ -117,6 +122,11 @@ vcycle_tail_kernel(const __grid_constant__ TailParams<T> P) {
       if (l == 0) {
         sm[L.r + q * row + x] = ld_dep(P.r + pe);
         if (has_o) sm[L.r + q * row + L.g.we + x] = ld_dep(P.r + po);
+        if (P.given) {
+          T* ln = sm + L.z + ip * L.plane + (j + 1) * L.pitch + x;
+          ln[L.g.R] = ld_dep(P.z + pe);
+          if (has_o) ln[L.odd] = ld_dep(P.z + po);
+        }
       }
       if (L.diag) {
         sm[L.d + q * row + x] = L.diag[pe / (unsigned)L.g.R];
@@ -332,13 +342,16 @@ vcycle_tail_kernel(const __grid_constant__ TailParams<T> P) {
   if (rank == 0)   // padding rows (identity)
     for (int c = 0; c < kColours; ++c)
       for (unsigned p = L.g.off[c] + L.g.cnt[c] + tid; p < L.g.end[c]; p += blockDim.x)
-        P.z[p] = ld_dep(P.r + p);
+        P.z[p] = P.given ? fma(T(-0.0), ld_dep(P.z + p), ld_dep(P.r + p)) : ld_dep(P.r + p);
 }
 
-// Fills P for the V-cycle from `level` down; false if it does not fit.
+// Fills P for the V-cycle from `level` down, or for `sweeps` > 0 sweeps on it;
+// false if it does not fit.
 template <typename T>
-static bool tail_plan(const hpg_problem* h, int level, int R, TailParams<T>& P) {
-  P.nlev = h->nlev - level;
+static bool tail_plan(const hpg_problem* h, int level, int R, int sweeps, bool from_zero,
+                      TailParams<T>& P) {
+  P.nlev = sweeps ? 1 : h->nlev - level;
+  P.given = sweeps && !from_zero;
   const Geom& top = h->lev[level].g;
   P.ppc = std::max(2, ((top.nz + kTailCtas - 1) / kTailCtas + 1) / 2 * 2);
   P.ctas = (top.nz + P.ppc - 1) / P.ppc;
@@ -389,11 +402,12 @@ static bool tail_plan(const hpg_problem* h, int level, int R, TailParams<T>& P) 
     push({kTailStage, lv, 0, zero && !odd, 0x391B, 7, 1});
     if (odd) push({kTailStage, lv, 1, 0, 0xE4, 4, 1});
   };
+  for (int i = 0; i < sweeps; ++i) sweep(0, from_zero && i == 0);
   for (int l = 0; l + 1 < P.nlev; ++l) {
     for (int i = 0; i < h->pre; ++i) sweep(l, i == 0);
     push({kTailRestrict, (unsigned char)l, 0, 0, 0, 0, 0});
   }
-  sweep(P.nlev - 1, true);
+  if (!sweeps) sweep(P.nlev - 1, true);
   for (int l = P.nlev - 2; l >= 0; --l) {
     P.op[P.nops - 1].cluster = 0;
     push({kTailProlong, (unsigned char)l, 0, 0, 0, 0, 1});
@@ -404,32 +418,34 @@ static bool tail_plan(const hpg_problem* h, int level, int R, TailParams<T>& P) 
 }
 
 template <typename T>
-static int tail_t(hpg_problem* h, int level, int R, const T* r, T* z, bool c0_done,
-                  cudaStream_t s) {
+static int tail_t(hpg_problem* h, int level, int R, const T* r, T* z, int sweeps,
+                  bool from_zero, bool c0_done, cudaStream_t s) {
   const Level& top = h->lev[level];
-  if (top.n * R > (sizeof(T) == 4 ? kTailPoints32 : kTailPoints64)) return HPG_ERR_UNSUPPORTED;
+  const long long most = sizeof(T) == 8 ? kTailPoints64 : sweeps ? kTailSweepPoints32 : kTailPoints32;
+  if (top.n * R > most) return HPG_ERR_UNSUPPORTED;
   TailParams<T> P;
-  if (!tail_plan(h, level, R, P)) return HPG_ERR_UNSUPPORTED;
+  if (!tail_plan(h, level, R, sweeps, from_zero, P)) return HPG_ERR_UNSUPPORTED;
   P.r = r;
   P.z = z;
   auto kern = vcycle_tail_kernel<T>;
-  HPG_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)kTailSmem));
+  if ((size_t)P.elems * sizeof(T) > (48u << 10) - 16)
+    HPG_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)kTailSmem));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)P.ctas);
   cfg.blockDim = dim3((unsigned)P.threads);
-  cfg.dynamicSmemBytes = (size_t)P.elems * sizeof(T);
+  cfg.dynamicSmemBytes = ((size_t)P.elems * sizeof(T) + 15) / 16 * 16;
   cfg.stream = s;
   const int prec = sizeof(T) == 8 ? HPG_FP64 : HPG_FP32;
   // colour phases of the first level (what the profile counts); the lower
   // levels' operations are noted without a time of their own
-  auto phases = [&](int l, int sweeps) {
+  auto phases = [&](int l, int count) {
     int n = 0, m = 0;
     for (int c = 0; c < kColours; ++c) {
       n += h->lev[l].cnt[c] > 0;
       m += c < kColours - 1 && h->lev[l].cnt[c] > 0;
     }
-    return sweeps * (n + m);
+    return count * (n + m);
   };
   const int last = h->nlev - 1;
   const int rc = launch(h, K_GS, level, prec, 2.0 * top.n * R * sizeof(T), s,
@@ -449,8 +465,8 @@ static int tail_t(hpg_problem* h, int level, int R, const T* r, T* z, bool c0_do
     cfg.attrs = attr;
     cfg.numAttrs = na;
     return cudaLaunchKernelEx(&cfg, kern, P);
-  }, phases(level, level == last ? 1 : h->pre + h->post) - (c0_done ? 1 : 0));
-  if (rc) return rc;
+  }, phases(level, sweeps ? sweeps : level == last ? 1 : h->pre + h->post) - (c0_done ? 1 : 0));
+  if (rc || sweeps) return rc;
   for (int l = level; l < last; ++l) {
     prof_note(h, K_RESTRICT, l, prec, 1);
     prof_note(h, K_PROLONG, l, prec, 1);
@@ -460,11 +476,20 @@ static int tail_t(hpg_problem* h, int level, int R, const T* r, T* z, bool c0_do
 }
 int launch_vcycle_tail(hpg_problem* h, int level, int R, const float* r, float* z, bool c0_done,
                        cudaStream_t s) {
-  return tail_t<float>(h, level, R, r, z, c0_done, s);
+  return tail_t<float>(h, level, R, r, z, 0, true, c0_done, s);
 }
 int launch_vcycle_tail(hpg_problem* h, int level, int R, const double* r, double* z, bool c0_done,
                        cudaStream_t s) {
-  return tail_t<double>(h, level, R, r, z, c0_done, s);
+  return tail_t<double>(h, level, R, r, z, 0, true, c0_done, s);
+}
+
+int launch_small_sweeps(hpg_problem* h, int level, const float* r, float* z, int sweeps,
+                        bool from_zero, cudaStream_t s) {
+  return tail_t<float>(h, level, 1, r, z, sweeps, from_zero, false, s);
+}
+int launch_small_sweeps(hpg_problem* h, int level, const double* r, double* z, int sweeps,
+                        bool from_zero, cudaStream_t s) {
+  return tail_t<double>(h, level, 1, r, z, sweeps, from_zero, false, s);
 }
 
 }  // namespace hpg
