@@ -356,13 +356,12 @@ def run_gpu(args):
     prof.sort(key=lambda p: -p["total_ms"])
     peak, peak_src = measured_peaks()
 
-    # ---- dominant kernel (level-0 FP32 Gauss-Seidel phase) timed with CUDA
-    # events on the launching stream, launched exactly as the V-cycle launches
-    # it: hpg_mg_smooth = 15 colour phases per sweep (colours 0..7, 6..0).
-    # Between sweeps the level-0 FP32 SpMV streams the whole matrix (453 MB,
-    # evict-first) as it does after every V-cycle of the solve, so that no
-    # phase finds the slice the previous sweep left in L2; only the sweeps
-    # are timed.
+    # ---- dominant kernel (level-0 FP32 Gauss-Seidel plane kernel) timed with
+    # CUDA events on the launching stream, launched exactly as the V-cycle
+    # launches it: hpg_mg_smooth = three launches per symmetric sweep.  A
+    # level-0 FP32 SpMV runs between sweeps, as after every V-cycle of the
+    # solve; the vectors of a 128^3 level (25 MB) stay in L2 there as in the
+    # solve, so the figure is the kernel's rate, not a DRAM rate.
     gs_reps = 20
     info0 = prob.info[0]
     r_gs = prob.to_storage(torch.randn(n, dtype=torch.float64, device=dev,
@@ -482,8 +481,11 @@ def run_gpu(args):
                        "smoother": "1+1 symmetric multicolour Gauss-Seidel",
                        "rhs": "A*1 + N(0, %g^2), seed %d" % (w.noise_std, w.seed),
                        "inner": "fp32", "basis": args.basis, "outer": "fp64",
-                       "l2": "inputs larger than L2 (FP32 ELL matrix %.0f MB)" % (
-                           prob.n_store() * 27 * 8 / 1e6),
+                       "l2": "working set larger than L2 (Krylov basis of %d vectors, %.0f MB)" % (
+                           w.restart + 1, (w.restart + 1) * prob.n_store() *
+                           {"fp32": 4}.get(args.basis, 2) / 1e6),
+                       "operator": "evaluated from the grid, beta and theta (the stored ELL "
+                                   "matrix is not read)",
                        "parallelism": "replicas" if world > 1 else "single"},
             "gpu_launches": launches, "clocks": clocks,
             "cpu_baseline": cpu,

@@ -104,7 +104,9 @@ typedef struct {
 
 /* Creates a problem on the current CUDA device: the fine-level 27-point
  * ELLPACK matrix (Sec. 3.2.2; slot-major column-index array shared by an FP64
- * and an FP32 value array), generated on the device in storage order.
+ * and an FP32 value array), generated on the device in storage order.  It is what
+ * the implementation options below run on; without them the operator is
+ * evaluated straight from the grid, beta and theta, with equal results.
  * Padding slots (neighbours outside the grid, Dirichlet truncation, Sec. 2)
  * hold column = own row and value 0.
  * nx, ny, nz >= 1 and nx*ny*nz*27 < 2^31.  p may be NULL (beta = 0).
@@ -181,9 +183,8 @@ HPG_API int hpg_mg_smooth(hpg_problem_t* h, int level, hpg_prec prec,
  * code running inside a CUDA stream capture (cudaMalloc is not allowed there),
  * real-time loops that must not stall on the allocator, or memory-pool owners
  * that forbid allocations outside their pool.  It computes what hpg_mg_vcycle
- * computes with one kernel launch per colour phase and transfer (the same
- * kernels, order and results as hpg_mg_vcycle with the default options; it
- * ignores HPG_OPT_COARSE_CLUSTER and always launches the phases), but the
+ * computes (the same kernels, order and results as hpg_mg_vcycle with the
+ * default options; it ignores HPG_OPT_COARSE_CLUSTER), but the
  * coarse levels' work vectors (restricted residuals and corrections of levels
  * level+1 .. last) live in one static device array of
  * HPG_NOALLOC_SCRATCH_BYTES bytes that the library declares at file scope:
@@ -295,15 +296,15 @@ HPG_API int hpg_gmres_ir_solve_batch(hpg_problem_t* h, int nrhs, const double* B
 /* Launch shape of the multi-right-hand-side kernels of `level`: kind 0 the
  * Gauss-Seidel phases, kind 1 the SpMV; lpr lanes per row (1, 2 or nrhs; 0 =
  * default 1) and block threads (64, 128, 256; 0 = default).  Every shape
- * gives the same results.  hpg_batch_tune sets them by timing. */
+ * gives the same results.  The SpMV uses the block size; the other values are
+ * stored and returned, but the kernels choose their own shapes. */
 HPG_API int hpg_batch_set_shape(hpg_problem_t* h, int level, int kind, int nrhs, int lpr,
                                 int block);
 HPG_API int hpg_batch_get_shape(const hpg_problem_t* h, int level, int kind, int nrhs,
                                 int* lpr, int* block);
 
-/* Times every launch shape of the multi-right-hand-side Gauss-Seidel sweep
- * on each level and of the level-0 SpMV for nrhs right-hand sides and keeps
- * the fastest (the autotuner; a few milliseconds per level).  Synchronises
+/* Times the block sizes of the level-0 SpMV for nrhs right-hand sides and keeps
+ * the fastest (the autotuner; well under a millisecond).  Synchronises
  * `stream`. */
 HPG_API int hpg_batch_tune(hpg_problem_t* h, int nrhs, void* stream);
 
@@ -343,8 +344,12 @@ HPG_API int hpg_batch_tune_solve(hpg_batch_t* b, const double* const* B, double*
  * every kernel the handle launches is bracketed by two CUDA events on its
  * own stream; the report aggregates per (kernel class, level, precision)
  * the launches, the summed event durations and the summed algorithmic DRAM
- * bytes of the library's byte model (matrix slots, vectors read and written
- * once).  Enabling adds two event records per launch. */
+ * bytes of the library's byte model (what a launch must move: its vectors read and
+ * written once, and matrix slots where a kernel reads the stored matrix).  A
+ * launch that runs several Gauss-Seidel colour phases counts each of them; one
+ * that runs a whole V-cycle on small levels is timed under its first level's
+ * phases, the other levels' operations being counted without a time of their own.
+ * Enabling adds two event records per launch. */
 typedef struct {
   const char* name;      /* kernel class (static string)                 */
   int level;             /* multigrid level (0 for vector kernels)       */
@@ -384,8 +389,9 @@ HPG_API int hpg_set_execution(hpg_problem_t* h, int mode);
  * kernel in which a tile of a colour phase starts as soon as the tiles of the
  * previous phase within one grid plane of it are done (bounded waits; a wait
  * that runs out makes the solve return HPG_ERR_TIMEOUT) instead of one launch
- * per colour phase; same results.  0: never; 1 (default): FP64 sweeps only
- * (measured faster on GB300 for FP64, slower for FP32); 2: always.  Setting
+ * per colour phase; same results.  It runs on the stored matrix and is slower than
+ * the default sweeps.  0: never; 1 (default): FP64 sweeps of a level after
+ * hpg_inject_stall; 2: always; 3: on every level.  Setting
  * an option drops captured solve graphs (single- and many-right-hand-side).
  * HPG_ERR_INVALID for an unknown option; HPG_ERR_STATE while a multi-system
  * batch uses the problem (its graph keeps the options it was captured
@@ -407,22 +413,17 @@ HPG_API int hpg_set_execution(hpg_problem_t* h, int mode);
  * fits in 64 KB; 0: one launch per colour phase there too.  Same results
  * (measured slower than the default on GB300).  Ignored while
  * HPG_OPT_GS_PIPELINE is 3.
- * HPG_OPT_PDL_ROWS (default 16384): Gauss-Seidel phases of levels whose
- * matrix does not stream from memory, up to this many rows per phase, let
- * the next kernel launch as soon as they start (their own matrix loads then
- * overlap the previous phase); larger phases let it launch only as their
- * blocks exit.  Multi-right-hand-side phases (the *_batch calls and batched
- * solves) up to this many rows are launched programmatically and let the
- * next kernel launch as soon as they start; larger ones start after the
- * previous kernel has completed.  Same results: kernels read the vectors an
- * earlier kernel wrote only after the grid-dependency wait, through coherent
- * loads. */
+ * HPG_OPT_PDL_ROWS (default 16384): accepted for values >= 0; it governed the
+ * programmatic launch of single colour phases on the stored matrix and has no
+ * effect on the sweeps by planes. */
 #define HPG_OPT_COARSE_CTA 5
 #define HPG_OPT_PDL_ROWS 6
 HPG_API int hpg_set_option(hpg_problem_t* h, int option, int value);
 
-/* Failure-detection test support (not a step of the method): the next
- * pipelined sweep on `level` starts its tile queue at `tiles`, so the tiles
+/* Failure-detection test support (not a step of the method): from here on FP64
+ * sweeps of `level`, where its matrix streams, run pipelined (unless
+ * HPG_OPT_GS_PIPELINE is 0), and the next pipelined
+ * sweep on `level` starts its tile queue at `tiles`, so the tiles
  * below never run and the waits of the tiles after them on those run out
  * (each wait is bounded, under a second); that sweep then abandons its
  * remaining tiles and records the error, and the solve that contains it (or

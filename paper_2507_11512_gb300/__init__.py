@@ -168,7 +168,7 @@ def set_execution(h, mode):
 
 def set_option(h, option, value):
     """hpg_set_option: HPG_OPT_COARSE_CLUSTER, HPG_OPT_PDL (0 / 1) or
-    HPG_OPT_GS_PIPELINE (0 never, 1 FP64 sweeps, 2 always)."""
+    HPG_OPT_GS_PIPELINE (0 never, 1 default, 2 streamed levels, 3 every level)."""
     check(load().hpg_set_option(h, option, int(value)), "hpg_set_option")
 
 

@@ -1,16 +1,13 @@
 // Multi-right-hand-side path: R right-hand sides of one system advance
-// together through the same kernels, so every matrix slot loaded from HBM
-// serves R rows of work instead of one.
+// together through the same kernels, so a launch and its latencies serve R
+// columns of work instead of one.
 //
 // Layout: an R-vector of a level is [n_store][R] (the R values of one storage
 // row are contiguous), in FP32 for the inner solve and FP64 for the outer
-// refinement; R is 1, 2, 4 or 8.  A row is handled by LPR lanes (1, 2 or R),
-// each lane owning RL = R / LPR consecutive right-hand sides, so a gather of
-// neighbour j reads RL contiguous values.  Which LPR and block size a level
-// uses is picked by timing (hpg_batch_tune); every choice computes the same
-// values in the same order as the single-right-hand-side kernels of
-// sparse.cu, so a column of a multi-right-hand-side SpMV or V-cycle is bitwise
-// the single-vector result.
+// refinement; R is 1, 2, 4 or 8.  The operator's kernels are the single-vector
+// ones (stencil.cuh: an R-vector is a grid with lines R times as wide), so a
+// column of a multi-right-hand-side SpMV or V-cycle is bitwise the single-vector
+// result.
 //
 // The Krylov part (batched GMRES-IR, Algorithm 3 per right-hand side) keeps a
 // separate basis, Hessenberg matrix, rotations and state per right-hand side;
@@ -131,10 +128,11 @@ mto_natural_kernel(const __grid_constant__ Geom g, int R, const Tin* __restrict_
 
 // ----------------------------------------------------------- batch space
 constexpr int kMaxR = 8;
-constexpr int kShapeGs = 0, kShapeSpmv = 1;
+constexpr int kShapeSpmv = 1;   // shape kinds: 0 sweeps, 1 SpMV
 
-// Launch shape of a multi-RHS stencil kernel on one level: lanes per row and
-// block size (0 = default).
+// Launch shape of a level (0 = default): block is the SpMV's threads per block;
+// lanes per row and the sweeps' block are kept for their callers (the plane
+// kernels choose their own).
 struct Shape {
   int lpr = 0;
   int block = 0;
@@ -1225,10 +1223,8 @@ static int msolve_t(hpg_problem* h, const double* B, double* X, double tol, int 
 }
 
 // --------------------------------------------------- host: launch tuning
-// Times every launch shape of the multi-RHS Gauss-Seidel sweep on each level
-// and of the level-0 SpMV, on zero data (the work does not depend on the
-// values), and keeps the fastest.  Shapes: lanes per row 1, 2 or R, blocks of
-// 64, 128 or 256 threads.
+// Times the block sizes of the level-0 SpMV, on zero data (the work does not
+// depend on the values), and keeps the fastest; the other kernels have one shape.
 template <int R>
 static int tune_t(hpg_problem* h, int reps, cudaStream_t s) {
   int rc = ensure_vcycle_buffers(h);
@@ -1241,42 +1237,31 @@ static int tune_t(hpg_problem* h, int reps, cudaStream_t s) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (rc == HPG_OK && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess))
     rc = cuda_fail(cudaGetLastError(), "cudaEventCreate", __FILE__, __LINE__);
-  std::vector<int> lprs = {1};
-  if (R >= 2) lprs.push_back(2);
-  if (R > 2) lprs.push_back(R);
-  const int blocks[3] = {64, 128, 256};
-  for (int l = 0; l < h->nlev && rc == HPG_OK; ++l) {
-    for (int kind = 0; kind < 2 && rc == HPG_OK; ++kind) {
-      if (kind == kShapeSpmv && l > 0) continue;
-      float* a = l == 0 ? x0 : bs->rc[l];
-      float* b = l == 0 ? y0 : bs->zc[l];
-      float best = 1e30f;
-      Shape best_shape;
-      for (int lpr : lprs)
-        for (int blk : blocks) {
-          bs->shape[l][kind][R].lpr = lpr;
-          bs->shape[l][kind][R].block = blk;
-          float ms = 0.0f;
-          for (int it = 0; it <= reps && rc == HPG_OK; ++it) {
-            if (it == 1 && cudaEventRecord(e0, s) != cudaSuccess) rc = HPG_ERR_CUDA;
-            h->pdl_next = false;
-            rc = kind == kShapeGs ? stencil_symgs(h, l, R, a, b, false, false, s)
-                                  : run_mspmv(h, R, l, a, b, s);
-          }
-          if (rc) break;
-          if (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
-              cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
-            rc = cuda_fail(cudaGetLastError(), "tuning events", __FILE__, __LINE__);
-            break;
-          }
-          if (ms < best) {
-            best = ms;
-            best_shape = bs->shape[l][kind][R];
-          }
-        }
-      bs->shape[l][kind][R] = best_shape;
+  for (int l = 0; l < h->nlev && rc == HPG_OK; ++l)
+    for (int kind = 0; kind < 2; ++kind) bs->shape[l][kind][R] = Shape();
+  float best = 1e30f;
+  Shape best_shape;
+  for (int blk : {64, 128, 256}) {
+    if (rc) break;
+    bs->shape[0][kShapeSpmv][R].block = blk;
+    float ms = 0.0f;
+    for (int it = 0; it <= reps && rc == HPG_OK; ++it) {
+      if (it == 1 && cudaEventRecord(e0, s) != cudaSuccess) rc = HPG_ERR_CUDA;
+      h->pdl_next = false;
+      if (rc == HPG_OK) rc = run_mspmv(h, R, 0, x0, y0, s);
+    }
+    if (rc) break;
+    if (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
+        cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
+      rc = cuda_fail(cudaGetLastError(), "tuning events", __FILE__, __LINE__);
+      break;
+    }
+    if (ms < best) {
+      best = ms;
+      best_shape = bs->shape[0][kShapeSpmv][R];
     }
   }
+  if (rc == HPG_OK) bs->shape[0][kShapeSpmv][R] = best_shape;
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   dev_free(x0);
