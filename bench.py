@@ -484,8 +484,8 @@ def run_gpu(args):
                        "l2": "working set larger than L2 (Krylov basis of %d vectors, %.0f MB)" % (
                            w.restart + 1, (w.restart + 1) * prob.n_store() *
                            {"fp32": 4}.get(args.basis, 2) / 1e6),
-                       "operator": "evaluated from the grid, beta and theta (the stored ELL "
-                                   "matrix is not read)",
+                       "operator": "evaluated from the grid, beta and theta (FP64 sweeps of a "
+                                   "given iterate read the stored ELL matrix)",
                        "parallelism": "replicas" if world > 1 else "single"},
             "gpu_launches": launches, "clocks": clocks,
             "cpu_baseline": cpu,

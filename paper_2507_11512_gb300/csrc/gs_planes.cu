@@ -12,46 +12,74 @@
 
 namespace hpg {
 
-// One colour phase (Sec. 3.2.1), one point per thread, in place: what a sweep
-// falls back to where an x-line is too long for gs_plane_kernel's shared
-// memory, and beside the TMA-tiled phases (HPG_OPT_GS_HALO).  from_zero: only
-// neighbours of a lower colour count (first forward sweep from z = 0).
-template <typename T>
+// One colour phase (Sec. 3.2.1), one point per thread, in place: FP64 sweeps of
+// larger levels (see symgs_t), sweeps whose x-lines are too long for
+// gs_plane_kernel, and phases beside the TMA-tiled ones (HPG_OPT_GS_HALO).  FP64:
+// bound by the FP64 unit (29 operations a point, 16 cycles a warp instruction and
+// SM), which small blocks spread evenly.  MC = -1: all neighbours; MC = 0..7: the
+// phase of colour MC in the first forward sweep from z = 0, where only neighbours
+// of a lower colour count (the set is fixed at compile time).
+template <typename T, int MC>
 __global__ void __launch_bounds__(256)
-gs_colour_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T> c, int colour,
-                 int from_zero, const T* r, const T* diag, T* z) {
+gs_colour_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T> c, int colour_,
+                 const T* r, const T* diag, T* z) {
+  constexpr unsigned kMask = MC < 0 ? (1u << kSlots) - 1u : gs_slot_mask(MC, true);
+  const int colour = MC < 0 ? colour_ : MC;
   pdl_trigger();
-  pdl_wait();
   const unsigned p = blockIdx.x * blockDim.x + threadIdx.x;
   const unsigned row = g.off[colour] + p;
   if (row >= g.end[colour]) return;
   if (p >= g.cnt[colour]) {   // padding row: identity
+    pdl_wait();
     const T v = ld_dep(r + row);
-    z[row] = from_zero ? v : fma(T(-0.0), ld_dep(z + row), v);
+    z[row] = MC >= 0 ? v : fma(T(-0.0), ld_dep(z + row), v);
     return;
   }
   const int px = colour_parity_x(colour), py = colour_parity_y(colour),
             pz = colour_parity_z(colour);
   const unsigned w = px ? g.wo : g.we, hl = py ? g.ho : g.he;
-  const int e = (int)(p % w);
-  const int j = 2 * (int)(p / w % hl) + py, k = 2 * (int)(p / w / hl) + pz;
+  const unsigned q = p / w, q2 = q / hl;
+  const int e = (int)(p - q * w);
+  const int j = 2 * (int)(q - q2 * hl) + py, k = 2 * (int)q2 + pz;
   const int i = 2 * (e / g.R) + px;
-  T acc = ld_dep(r + row);
+  pdl_wait();
+  T v[kSlots];
 #pragma unroll
   for (int s = 0; s < kSlots; ++s) {
     const int dx = s % 3 - 1, dy = (s / 3) % 3 - 1, dz = s / 9 - 1;
-    if (s == kCentre) continue;
-    const int nc = colour ^ ((dx & 1) | ((dy & 1) << 1) | ((dz & 1) << 2));
+    v[s] = T(0);
+    if (s == kCentre || !((kMask >> s) & 1u)) continue;
     const bool in = (unsigned)(i + dx) < (unsigned)g.nx && (unsigned)(j + dy) < (unsigned)g.ny &&
-                    (unsigned)(k + dz) < (unsigned)g.nz && !(from_zero && nc > colour);
-    T v = T(0);
-    if (in) v = ld_dep(z + line_base(g, px ^ (dx & 1), j + dy, k + dz) + e +
-                       ((px + dx) >> 1) * g.R);
-    acc = fma(-c.a[dx + dy + dz + 3], v, acc);
+                    (unsigned)(k + dz) < (unsigned)g.nz;
+    if (in) v[s] = ld_dep(z + line_base(g, px ^ (dx & 1), j + dy, k + dz) + e +
+                          ((px + dx) >> 1) * g.R);
   }
-  if (!from_zero && (x_edge(g, px, e) || j == 0 || j == g.ny - 1 || k == 0 || k == g.nz - 1))
-    pad_slot(ld_dep(z + row), acc);
-  z[row] = acc / (diag ? diag[row / (unsigned)g.R] : (T)kDiag);
+  T u[1] = {ld_dep(r + row)};
+#pragma unroll
+  for (int s = 0; s < kSlots; ++s)
+    if (s != kCentre && ((kMask >> s) & 1u))
+      u[0] = fma(-c.a[s % 3 - 1 + (s / 3) % 3 - 1 + s / 9 - 1 + 3], v[s], u[0]);
+  if (MC < 0 && (x_edge(g, px, e) || j == 0 || j == g.ny - 1 || k == 0 || k == g.nz - 1))
+    pad_slot(ld_dep(z + row), u[0]);
+  if (diag) u[0] = u[0] / diag[row / (unsigned)g.R];
+  else div_diag<T, 1>(u);
+  z[row] = u[0];
+}
+
+template <typename T>
+using ColourFn = void (*)(const SGeom, const Coef<T>, int, const T*, const T*, T*);
+template <typename T> static ColourFn<T> colour_fn(int colour, bool from_zero) {
+  if (!from_zero) return gs_colour_kernel<T, -1>;
+  switch (colour) {
+    case 0: return gs_colour_kernel<T, 0>;
+    case 1: return gs_colour_kernel<T, 1>;
+    case 2: return gs_colour_kernel<T, 2>;
+    case 3: return gs_colour_kernel<T, 3>;
+    case 4: return gs_colour_kernel<T, 4>;
+    case 5: return gs_colour_kernel<T, 5>;
+    case 6: return gs_colour_kernel<T, 6>;
+    default: return gs_colour_kernel<T, 7>;
+  }
 }
 
 // The symmetric sweep by planes.  Points of one z parity form whole planes,
@@ -75,9 +103,12 @@ gs_colour_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T
 // loads are done and waits only before it stores, after its last phase.
 //
 // Large grids are bound by the vectors' traffic and by instruction issue (R
-// and the loads' offsets are compile-time, two FP32 elements share loads and
+// and the loads' offsets are compile-time, two or four FP32 elements share loads and
 // addresses for that reason), FP64 by the FP64 rate; small ones by the chain of
 // load, phases and store.
+// One sweep on GB300, stored matrix with a launch per colour -> this: FP32 64^3 39
+// -> 13 us, 128^3 139 -> 30 us, 320^3 2.1 ms -> 495 us; FP64 64^3 66 -> 48 us, 96^3 229
+// -> 150 us.
 enum PlaneKind { kOddFwd = 0, kEven = 1, kOddBwd = 2 };
 
 struct PlanePlan {
@@ -445,11 +476,14 @@ constexpr size_t kPlaneSmemGoal = 112u << 10;   // two CTAs per SM
 constexpr int kMaxPlaneCtas = 8;                // portable cluster size
 
 // How a level's planes are split.  FP32: up to 4 CTAs per plane while that makes
-// at most two CTAs per SM; FP64, whose time is the busiest SM's FP64 work, up to 5
-// and three per SM; with at least 8 lines each (a CTA recomputes up to 3 more).
+// at most two CTAs per SM, with at least 8 lines each (a CTA recomputes up to 3
+// more).  FP64, whose time is the busiest SM's FP64 work: the split of up to 5 CTAs
+// with the fewest lines on that SM -- one CTA per SM up to 85 % of the SMs (clusters
+// do not reach all of them), else whole rounds of two (64^3 sweep 76 -> 48 us, 80^3
+// 112 -> 92, against 5 CTAs throughout).
 // Up to 8 where a CTA's lines would take more shared memory than two CTAs per SM
 // have.  (Measured, one sweep: 128^3 FP32 30 us with 4 CTAs per plane, 37 with 3 or
-// 8; 96^3 FP64 150 us with 5, 177 with 4, 226 with 3, 187 with 8.)  About 384
+// 8; 96^3 FP64 150 us with 5, 177 with 4, 187 with 8.)  About 384
 // threads a CTA, twice that where only one fits an SM.  The next kernel may
 // start early only after grids that leave most SMs idle: otherwise its waiting
 // CTAs take the free places unevenly (96^3 FP64 V-cycle 595 us with an early start
@@ -461,8 +495,20 @@ static bool plane_plan(const SGeom& g, int num_sms, PlanePlan* out) {
   const int planes = std::max(g.de, 1);
   int cs = 1;
   auto lines_for = [&](int n) { return std::max(2, ((g.ny + n - 1) / n + 1) / 2 * 2); };
-  constexpr int most = sizeof(T) == 8 ? 5 : 4, per_sm = sizeof(T) == 8 ? 3 : 2;
-  while (cs < most && planes * (cs + 1) <= per_sm * num_sms && lines_for(cs + 1) >= 8) ++cs;
+  if (sizeof(T) == 8) {
+    double best = 1e30;
+    for (int n = 1; n <= 5 && (n == 1 || lines_for(n) >= 8); ++n) {
+      const int ctas = planes * n;
+      const int rounds = ctas <= num_sms * 0.85 ? 1 : (ctas + 2 * num_sms - 1) / (2 * num_sms) * 2;
+      const double cost = rounds * (lines_for(n) + 1.5);
+      if (cost < best) {
+        best = cost;
+        cs = n;
+      }
+    }
+  } else {
+    while (cs < 4 && planes * (cs + 1) <= 2 * num_sms && lines_for(cs + 1) >= 8) ++cs;
+  }
   while (cs < kMaxPlaneCtas && plane_smem<T, V>(g, lines_for(cs)) > kPlaneSmemGoal) ++cs;
   if (plane_smem<T, V>(g, lines_for(cs)) > kMaxPlaneSmem) return false;
   PlanePlan p;
@@ -561,9 +607,9 @@ static int colour_phase_t(hpg_problem* h, int level, int R, int colour, bool fro
   return launch(h, K_GS, level, sizeof(T) == 8 ? HPG_FP64 : HPG_FP32,
                 L.cnt[colour] * (2.0 + nslots / 26.0) * R * sizeof(T), s, "gs_colour_kernel",
                 [&] {
-                  return kl(h, gs_colour_kernel<T>, grid_for(n, 256), 256, s, g,
-                            make_coef<T>(h->beta), colour, (int)from_zero, r, level_diag<T>(L),
-                            z);
+                  const int block = sizeof(T) == 8 ? 64 : 256;
+                  return kl(h, colour_fn<T>(colour, from_zero), grid_for(n, block), block, s, g,
+                            make_coef<T>(h->beta), colour, r, level_diag<T>(L), z);
                 });
 }
 int stencil_colour_phase(hpg_problem* h, int level, int R, int colour, bool from_zero,
@@ -574,6 +620,12 @@ int stencil_colour_phase(hpg_problem* h, int level, int R, int colour, bool from
                          const double* r, double* z, cudaStream_t s) {
   return colour_phase_t<double>(h, level, R, colour, from_zero, r, z, s);
 }
+
+// FP64 sweeps from this many points on run one launch per colour: there a launch
+// costs little beside its FP64 work, and small blocks use every SM's FP64 unit,
+// which whole planes cannot (one sweep, planes against colours: 96^3 150 / 153 us,
+// 112^3 213 / 219, 128^3 440 / 287, 200^3 1444 / 945).
+constexpr long long kColourPoints64 = 1000000;
 
 // One symmetric sweep; c0_done: z already holds colour 0's first phase.
 template <typename T>
@@ -589,7 +641,7 @@ static int symgs_t(hpg_problem* h, int level, int R, const T* r, T* z, bool from
   const bool fits = V == 4   ? plane_plan<T, 4>(g, h->num_sms, &pl)
                     : V == 2 ? plane_plan<T, 2>(g, h->num_sms, &pl)
                              : plane_plan<T, 1>(g, h->num_sms, &pl);
-  if (!fits || (R > 1 && !vec)) {
+  if (!fits || (R > 1 && !vec) || (sizeof(T) == 8 && L.n >= kColourPoints64)) {
     for (int c = c0_done ? 1 : 0; c < kColours; ++c)
       if ((rc = stencil_colour_phase(h, level, R, c, from_zero, r, z, s))) return rc;
     for (int c = kColours - 2; c >= 0; --c)

@@ -39,7 +39,7 @@ def theta_of(dims, seed):
 # whole groups of 4, of 2 and ragged parts, small and large (four elements a thread from
 # 600,000 points), one and several CTAs per plane, lines longer than a CTA takes (1538 FP32),
 # single planes, lines and columns
-GRIDS = [(128, 96, 72), (100, 92, 80), (130, 82, 78), (34, 18, 10), (40, 37, 3), (5, 3, 7),
+GRIDS = [(128, 96, 72), (130, 100, 80), (100, 92, 80), (130, 82, 78), (34, 18, 10), (40, 37, 3), (5, 3, 7),
          (1538, 3, 2), (3100, 2, 3), (1, 9, 4), (6, 1, 5), (7, 6, 1), (2, 2, 2)]
 
 
