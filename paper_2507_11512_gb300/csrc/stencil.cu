@@ -17,7 +17,7 @@ namespace hpg {
 // an element group of LINES consecutive x-lines, so that a warp's loads run
 // along x, neighbour lines are reused in registers and two FP32 elements share
 // loads and addresses.  GB300, stored matrix -> this: FP32 128^3 74 -> 9.1 us, 320^3
-// 1.2 ms -> 115 us; FP64 82x78x84 41 -> 32 us, 128^3 131 -> 103 us.
+// 1.2 ms -> 117 us; FP64 96^3 57 -> 45 us, 128^3 128 -> 99 us.
 template <typename T, int R, bool VEC, int LINES>
 __global__ void __launch_bounds__(256)
 stencil_spmv_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T> c,
@@ -44,6 +44,26 @@ stencil_spmv_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coe
   }
 }
 
+// The same with one thread per storage row, for FP64 levels between these sizes,
+// whose FP64 work single rows spread most evenly over the SMs (rows against pairs
+// of lines: 40^3 6.2 / 7.0 us, 72^3 20.9 / 23.9, 96^3 44.7 / 45.5; 128^3 101 / 99, 16^3
+// 5.0 / 4.2).
+constexpr long long kRowPoints64 = 60000, kRowPointsMax64 = 1500000;
+__global__ void __launch_bounds__(64)
+stencil_spmv_row_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<double> c,
+                        unsigned ns, const double* x, const double* diag, double* y) {
+  pdl_trigger();
+  const unsigned row = blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_wait();
+  if (row >= ns) return;
+  double v = 0.0;
+  const bool point = for_row_slots(g, row, [&](int s, int ci, bool in, unsigned q) {
+    const double a = s == kCentre ? (diag ? diag[row] : kDiag) : in ? c.a[ci] : 0.0;
+    v = fma(a, ld_dep(x + q), v);
+  });
+  y[row] = point ? v : ld_dep(x + row);   // padding row: identity
+}
+
 RowPlan make_row_plan(const SGeom& g, int elems, int lines) {
   RowPlan p;
   p.across = (unsigned)((g.we + elems - 1) / elems);
@@ -58,13 +78,18 @@ template <typename T, int R, bool VEC>
 static cudaError_t spmv_launch(hpg_problem* h, const SGeom& g, const T* x, const T* diag, T* y,
                                int block, cudaStream_t s) {
   constexpr int V = row_elems<T>();
-  // four lines a thread once that leaves every SM several 256-thread blocks
-  const bool big = (long long)g.we / V * g.ny * g.nz >= (long long)kRowLines * 2 * 256 * h->num_sms;
-  const RowPlan pl = make_row_plan(g, V, big ? kRowLines : 1);
+  // lines a thread takes: as many as leave every SM enough threads (FP32 64^3 4.6 us
+  // with one, 3.3 with two; 96^3 9.9 / 5.8 / 5.4 with one, two, four)
+  const long long groups = (long long)((g.we + V - 1) / V) * g.ny * g.nz;
+  const int lines = groups < 25000 || (sizeof(T) == 8 && groups < 50000) ? 1
+                    : sizeof(T) == 8 || groups < 150000                  ? 2 : kRowLines;
+  const RowPlan pl = make_row_plan(g, V, lines);
   // small blocks spread few threads over all SMs, and FP64 work evenly (an SM
   // has one FP64 unit, 16 cycles a warp instruction)
   if (sizeof(T) == 8 || (long long)pl.threads <= 256LL * h->num_sms) block = 64;
-  return kl(h, big ? stencil_spmv_kernel<T, R, VEC, kRowLines> : stencil_spmv_kernel<T, R, VEC, 1>,
+  return kl(h, lines == 1   ? stencil_spmv_kernel<T, R, VEC, 1>
+               : lines == 2 ? stencil_spmv_kernel<T, R, VEC, 2>
+                            : stencil_spmv_kernel<T, R, VEC, kRowLines>,
             grid_for((long long)pl.threads + pl.pad, block), block, s, g, make_coef<T>(h->beta),
             pl, x, diag, y);
 }
@@ -78,6 +103,10 @@ static int spmv_t(hpg_problem* h, int level, int R, const T* x, T* y, cudaStream
   return launch(h, K_SPMV, level, sizeof(T) == 8 ? HPG_FP64 : HPG_FP32,
                 (double)L.n * R * 2.0 * sizeof(T) + (diag ? L.n * (double)sizeof(T) : 0.0), s,
                 "stencil_spmv_kernel", [&] {
+                  if constexpr (sizeof(T) == 8)
+                    if (L.n >= kRowPoints64 && L.n < kRowPointsMax64)
+                      return kl(h, stencil_spmv_row_kernel, grid_for(L.g.n_store, 64), 64, s, g,
+                                make_coef<double>(h->beta), (unsigned)L.g.n_store, x, diag, y);
                   const bool vec = whole_groups<T, row_elems<T>()>(g, x, y);
                   if constexpr (sizeof(T) == 4) {   // R-vectors are FP32
                     if (R == 8) return spmv_launch<T, 8, true>(h, g, x, diag, y, block, s);

@@ -252,8 +252,8 @@ __device__ __forceinline__ bool for_row_slots(const SGeom& g, unsigned row, F&& 
   return true;
 }
 
-// Lines a thread of a whole-grid product takes (stencil_rows): 4 share their
-// neighbour lines in registers; 1 where that would leave SMs without work.
+// Lines a thread of a whole-grid product takes (stencil_rows), at most: they
+// share their neighbour lines in registers.
 constexpr int kRowLines = 4;
 // Elements of a line it takes: the loads of two FP32 elements are one load
 // each, and their addresses one computation; FP64 is bound by its FMAs.
