@@ -128,11 +128,13 @@ constexpr long long kResidentMatrixBytes = 16LL << 20;
 // ---------------------------------------------- programmatic dependent launch
 // Kernels of the solve chain are launched with programmatic stream
 // serialization: the next kernel may start while its predecessor drains.
-// Every kernel calls pdl_trigger() on entry, may touch data that no earlier
-// kernel of the chain writes (the matrix) before pdl_wait(), and reads or
-// writes everything else only after pdl_wait(), which returns once all
-// prerequisite grids have completed and their writes are visible.  Without a
-// programmatic launch both are no-ops.
+// A kernel calls pdl_trigger() on entry, or not at all (the next one then starts
+// as its blocks exit).  Before pdl_wait() it touches only data that no kernel of
+// the chain writes (the matrix, diagonals).  Everything else it reads or writes
+// after pdl_wait(), which returns once all prerequisite grids have completed and
+// made their writes visible to this grid: that an earlier kernel must have
+// finished by then does not make its writes visible to a grid that has not
+// waited.  Without a programmatic launch both are no-ops.
 __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

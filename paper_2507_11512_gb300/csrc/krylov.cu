@@ -525,6 +525,8 @@ cgs2_pass_kernel(const B* __restrict__ Q, long long ns, int ncol, const T* w,
   constexpr bool MAXLAST = S && KIND == kFinal;
   __shared__ T shc[KMAX];   // h1 (reorth) or h2 (final), scaled for a 2-byte basis
   __shared__ double sums[KMAX];
+  pdl_trigger();
+  pdl_wait();   // w, Q and h come from earlier kernels
   // Zig-zag over the passes (zigzag != 0, basis vectors much smaller than
   // L2): the reorth pass walks the rows backwards, so it starts on the rows
   // the GEMVT pass read last (still in L2), and the final pass forwards again;
@@ -544,19 +546,12 @@ cgs2_pass_kernel(const B* __restrict__ Q, long long ns, int ncol, const T* w,
     ld_group<B, V>(Q + j * ns + (rev ? ng - 1 - gi : gi) * V, q[j], pol);
   };
   long long gi = blockIdx.x * (long long)kRedThreads + threadIdx.x;
-  // A pass lets the next one start only after its own wait, so when the reorth
-  // or the final pass runs, every kernel before its predecessor has finished: Q
-  // (and for the reorth pass w) is final, and its first row group is loaded while
-  // the predecessor's last block still adds the partial sums.
-  constexpr bool kEarly = KIND != kGemvT;
-  if (kEarly && gi < ng) {
-    if (KIND == kReorth) load_w(gi, wr);
+  if (gi < ng) {   // the first row group, while the coefficients arrive
+    load_w(gi, wr);
 #pragma unroll
     for (int j = 0; j < KMAX; ++j)
       if (j < ncol) load_q(gi, j);
   }
-  pdl_wait();   // h (and w, Q) come from earlier kernels
-  pdl_trigger();
   if (KIND != kGemvT) {
     const double* hc = KIND == kReorth ? h1 : h2;
     for (int j = threadIdx.x; j < ncol; j += kRedThreads)
@@ -571,14 +566,6 @@ cgs2_pass_kernel(const B* __restrict__ Q, long long ns, int ncol, const T* w,
   T acc[KMAX];
 #pragma unroll
   for (int j = 0; j < KMAX; ++j) acc[j] = T(0);
-  if (gi < ng) {
-    if (KIND != kReorth) load_w(gi, wr);
-    if (!kEarly) {
-#pragma unroll
-      for (int j = 0; j < KMAX; ++j)
-        if (j < ncol) load_q(gi, j);
-    }
-  }
   // In the GEMVT and final passes a column's registers are refilled with the next
   // row group's values as soon as they have been used, so the loads of a thread
   // never pause (128^3, 17 columns: GEMVT 41.1 -> 38.2 us, final 40.5 -> 34.1); the
