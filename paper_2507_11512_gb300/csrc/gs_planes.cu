@@ -12,73 +12,155 @@
 
 namespace hpg {
 
-// One colour phase (Sec. 3.2.1), one point per thread, in place: FP64 sweeps of
-// larger levels (see symgs_t), sweeps whose x-lines are too long for
-// gs_plane_kernel, and phases beside the TMA-tiled ones (HPG_OPT_GS_HALO).  FP64:
-// bound by the FP64 unit (29 operations a point, 16 cycles a warp instruction and
-// SM), which small blocks spread evenly.  MC = -1: all neighbours; MC = 0..7: the
-// phase of colour MC in the first forward sweep from z = 0, where only neighbours
-// of a lower colour count (the set is fixed at compile time).
-template <typename T, int MC>
-__global__ void __launch_bounds__(256)
-gs_colour_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<T> c, int colour_,
-                 const T* r, const T* diag, T* z) {
-  constexpr unsigned kMask = MC < 0 ? (1u << kSlots) - 1u : gs_slot_mask(MC, true);
-  const int colour = MC < 0 ? colour_ : MC;
-  pdl_trigger();
-  const unsigned p = blockIdx.x * blockDim.x + threadIdx.x;
-  const unsigned row = g.off[colour] + p;
-  if (row >= g.end[colour]) return;
-  if (p >= g.cnt[colour]) {   // padding row: identity
-    pdl_wait();
-    const T v = ld_dep(r + row);
-    z[row] = MC >= 0 ? v : fma(T(-0.0), ld_dep(z + row), v);
-    return;
+// Quotients by a fixed divisor below 2^31 of dividends below 2^31 (Granlund and
+// Montgomery, PLDI 1994: the multiplier for 31-bit operands fits 32 bits).
+struct Div31 {
+  unsigned d, m, sh;
+  explicit Div31(unsigned n) : d(n), m(0), sh(0) {
+    if (n <= 1) return;
+    unsigned s = 1;
+    while ((1ULL << s) < n) ++s;
+    m = (unsigned)((1ULL << (31 + s)) / n + 1);
+    sh = s - 1;
   }
+  __device__ __forceinline__ unsigned div(unsigned t) const { return m ? __umulhi(t, m) >> sh : t; }
+};
+
+// What a colour phase needs of its level, in elements of an R-vector.  A
+// neighbour's line part is told by which of its parities differ from the colour's:
+// flip f (bit 0 x, 1 y, 2 z) starts at o[f] and steps w[f] a line, wh[f] a plane; slot
+// s adds d[s].
+struct ColourPlan {
+  unsigned off, cnt, end;     // the colour's block (end: with padding rows)
+  Div31 across, lines;        // a line's element groups, a plane's lines
+  int px, py, pz, ny, nz, R, rshift;
+  int early;                  // whether the next kernel may start while this one runs
+  unsigned o[8], w[8], wh[8];
+  int d[kSlots];
+};
+static ColourPlan make_colour_plan(const SGeom& g, int colour, int V) {
   const int px = colour_parity_x(colour), py = colour_parity_y(colour),
             pz = colour_parity_z(colour);
-  const unsigned w = px ? g.wo : g.we, hl = py ? g.ho : g.he;
-  const unsigned q = p / w, q2 = q / hl;
-  const int e = (int)(p - q * w);
-  const int j = 2 * (int)(q - q2 * hl) + py, k = 2 * (int)q2 + pz;
-  const int i = 2 * (e / g.R) + px;
+  ColourPlan q{g.off[colour], g.cnt[colour], g.end[colour],
+               Div31((unsigned)((px ? g.wo : g.we) / V)), Div31((unsigned)(py ? g.ho : g.he))};
+  q.px = px; q.py = py; q.pz = pz; q.ny = g.ny; q.nz = g.nz; q.R = g.R;
+  q.rshift = g.R == 8 ? 3 : g.R >> 1;
+  q.early = 1;
+  for (int f = 0; f < 8; ++f) {
+    const int x = px ^ (f & 1), y = py ^ (f >> 1 & 1), z = pz ^ (f >> 2);
+    q.o[f] = g.off[(x ^ 1) | (y ^ 1) << 1 | (z ^ 1) << 2];
+    q.w[f] = (unsigned)(x ? g.wo : g.we);
+    q.wh[f] = q.w[f] * (unsigned)(y ? g.ho : g.he);
+  }
+  for (int s = 0; s < kSlots; ++s) {
+    const int dx = s % 3 - 1, dy = (s / 3) % 3 - 1, dz = s / 9 - 1;
+    const int f = (dx & 1) | (dy & 1) << 1 | (dz & 1) << 2;
+    q.d[s] = ((px + dx) >> 1) * g.R + ((py + dy) >> 1) * (int)q.w[f] + ((pz + dz) >> 1) * (int)q.wh[f];
+  }
+  return q;
+}
+
+// One colour phase (Sec. 3.2.1), V consecutive elements of a line per thread (V
+// divides R, so that neighbour groups are aligned), in place: FP64 sweeps of larger
+// levels and levels whose planes do not fit (see symgs_t), and phases beside the
+// TMA-tiled ones (HPG_OPT_GS_HALO).  Small phases are bound by the chain of wait, loads,
+// products and division, so positions and line addresses are formed before the wait,
+// from eight bases and fixed steps, and no load waits for another; large FP32 ones by
+// instruction issue; FP64 by the FP64 unit (29 operations a point, 16 cycles a warp
+// instruction and SM), which small blocks spread evenly.  One sweep, against a
+// kernel that found each neighbour's line by itself after the wait and read the own entry
+// of boundary points last: FP32 2000 x 4 x 4 47 -> 25 us, 400 x 400 x 40 373 -> 165; FP64
+// 2000 x 4 x 4 54 -> 38, 112^3 218 -> 195, 160^3 511 -> 478; 256 x 256 x 8 with eight
+// right-hand sides, V-cycle 634 -> 254 (two elements a thread; four held too few loads in
+// flight, 309).  MC = -1: all
+// neighbours; MC = 0..7: the phase of colour MC in the first forward sweep from
+// z = 0, where only neighbours of a lower colour count (the set is fixed at compile
+// time).
+template <typename T, int V, int MC>
+__global__ void __launch_bounds__(256)
+gs_colour_kernel(const __grid_constant__ ColourPlan g, const __grid_constant__ Coef<T> c,
+                 const T* r, const T* diag, T* z) {
+  constexpr unsigned kMask = MC < 0 ? (1u << kSlots) - 1u : gs_slot_mask(MC, true);
+  using P = typename VecOf<T, V>::type;
+  if (g.early) pdl_trigger();
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned p = t * V, row = g.off + p;
+  if (row >= g.end) return;
+  if (p >= g.cnt) {   // padding row: identity
+    pdl_wait();
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      const T rv = ld_dep(r + row + v);
+      z[row + v] = MC >= 0 ? rv : fma(T(-0.0), ld_dep(z + row + v), rv);
+    }
+    return;
+  }
+  const unsigned q = g.across.div(t), e = (t - q * g.across.d) * V;
+  const unsigned K = g.lines.div(q), J = q - K * g.lines.d;
+  const int j = 2 * (int)J + g.py, k = 2 * (int)K + g.pz;
+  // whether the points before and after exist along x, y and z
+  const bool lo[3] = {g.px || e >= (unsigned)g.R, j > 0, k > 0};
+  const bool up[3] = {e + (unsigned)(g.px * g.R) < g.w[1], j + 1 < g.ny, k + 1 < g.nz};
+  const bool edge = !(lo[0] && up[0] && lo[1] && up[1] && lo[2] && up[2]);
+  unsigned base[8];
+#pragma unroll
+  for (int f = 0; f < 8; ++f) {
+    base[f] = g.o[f] + g.w[f] * J + g.wh[f] * K + e;
+    asm volatile("" : "+r"(base[f]));   // formed here, not after the wait
+  }
+  const T dg = diag ? diag[row >> g.rshift] : T(0);
   pdl_wait();
-  T v[kSlots];
+  T x[kSlots][V], u[V];
 #pragma unroll
   for (int s = 0; s < kSlots; ++s) {
     const int dx = s % 3 - 1, dy = (s / 3) % 3 - 1, dz = s / 9 - 1;
-    v[s] = T(0);
-    if (s == kCentre || !((kMask >> s) & 1u)) continue;
-    const bool in = (unsigned)(i + dx) < (unsigned)g.nx && (unsigned)(j + dy) < (unsigned)g.ny &&
-                    (unsigned)(k + dz) < (unsigned)g.nz;
-    if (in) v[s] = ld_dep(z + line_base(g, px ^ (dx & 1), j + dy, k + dz) + e +
-                          ((px + dx) >> 1) * g.R);
+#pragma unroll
+    for (int v = 0; v < V; ++v) x[s][v] = T(0);
+    if (s == kCentre ? MC >= 0 : !((kMask >> s) & 1u)) continue;
+    bool in = s != kCentre || edge;
+    if (dx) in = in && (dx < 0 ? lo[0] : up[0]);
+    if (dy) in = in && (dy < 0 ? lo[1] : up[1]);
+    if (dz) in = in && (dz < 0 ? lo[2] : up[2]);
+    const unsigned f = (dx & 1) | (dy & 1) << 1 | (dz & 1) << 2;
+    if (in) unpack(ld_dep(reinterpret_cast<const P*>(z + (base[f] + (unsigned)g.d[s]))), x[s]);
   }
-  T u[1] = {ld_dep(r + row)};
+  unpack(ld_dep(reinterpret_cast<const P*>(r + row)), u);
 #pragma unroll
   for (int s = 0; s < kSlots; ++s)
-    if (s != kCentre && ((kMask >> s) & 1u))
-      u[0] = fma(-c.a[s % 3 - 1 + (s / 3) % 3 - 1 + s / 9 - 1 + 3], v[s], u[0]);
-  if (MC < 0 && (x_edge(g, px, e) || j == 0 || j == g.ny - 1 || k == 0 || k == g.nz - 1))
-    pad_slot(ld_dep(z + row), u[0]);
-  if (diag) u[0] = u[0] / diag[row / (unsigned)g.R];
-  else div_diag<T, 1>(u);
-  z[row] = u[0];
+    if (s != kCentre && ((kMask >> s) & 1u)) {
+#pragma unroll
+      for (int v = 0; v < V; ++v)
+        u[v] = fma(-c.a[s % 3 - 1 + (s / 3) % 3 - 1 + s / 9 - 1 + 3], x[s][v], u[v]);
+    }
+  if (MC < 0 && edge) {
+#pragma unroll
+    for (int v = 0; v < V; ++v) pad_slot(x[kCentre][v], u[v]);
+  }
+  if (diag) {
+#pragma unroll
+    for (int v = 0; v < V; ++v) u[v] = u[v] / dg;
+  } else {
+    div_diag<T, V>(u);
+  }
+  bool all[V];
+#pragma unroll
+  for (int v = 0; v < V; ++v) all[v] = true;
+  store_elems<T, V, true>(z + row, all, u);
 }
 
 template <typename T>
-using ColourFn = void (*)(const SGeom, const Coef<T>, int, const T*, const T*, T*);
-template <typename T> static ColourFn<T> colour_fn(int colour, bool from_zero) {
-  if (!from_zero) return gs_colour_kernel<T, -1>;
+using ColourFn = void (*)(const ColourPlan, const Coef<T>, const T*, const T*, T*);
+template <typename T, int V> static ColourFn<T> colour_fn(int colour, bool from_zero) {
+  if (!from_zero) return gs_colour_kernel<T, V, -1>;
   switch (colour) {
-    case 0: return gs_colour_kernel<T, 0>;
-    case 1: return gs_colour_kernel<T, 1>;
-    case 2: return gs_colour_kernel<T, 2>;
-    case 3: return gs_colour_kernel<T, 3>;
-    case 4: return gs_colour_kernel<T, 4>;
-    case 5: return gs_colour_kernel<T, 5>;
-    case 6: return gs_colour_kernel<T, 6>;
-    default: return gs_colour_kernel<T, 7>;
+    case 0: return gs_colour_kernel<T, V, 0>;
+    case 1: return gs_colour_kernel<T, V, 1>;
+    case 2: return gs_colour_kernel<T, V, 2>;
+    case 3: return gs_colour_kernel<T, V, 3>;
+    case 4: return gs_colour_kernel<T, V, 4>;
+    case 5: return gs_colour_kernel<T, V, 5>;
+    case 6: return gs_colour_kernel<T, V, 6>;
+    default: return gs_colour_kernel<T, V, 7>;
   }
 }
 
@@ -596,6 +678,17 @@ static cudaError_t plane_launch(hpg_problem* h, const SGeom& g, int V, bool vec,
   }
 }
 
+// Whether the next phase may start while one of `threads` threads runs.  Its blocks
+// then wait in the places that are left, and spread unevenly over the SMs, unless
+// the phase is so small that it does not matter or takes every place itself (1024
+// FP64 threads an SM at these kernels' registers, 1536 FP32).  One sweep, early /
+// not: FP64 40^3 40.6 / 40.9 us, 48^3 43.8 / 43.0, 80^3 135 / 87, 104^3 161 / 157, 112^3
+// 195 / 197; FP32 64^3 28.6 / 28.2, 88^3 46 / 39, 112^3 54.7 / 53.8, 120^3 56 / 61.
+template <typename T> static int colour_early(long long threads, int num_sms) {
+  const long long few = sizeof(T) == 8 ? 80 : 260, full = sizeof(T) == 8 ? 980 : 1350;
+  return threads <= few * num_sms || threads >= full * num_sms;
+}
+
 template <typename T>
 static int colour_phase_t(hpg_problem* h, int level, int R, int colour, bool from_zero,
                           const T* r, T* z, cudaStream_t s) {
@@ -604,12 +697,20 @@ static int colour_phase_t(hpg_problem* h, int level, int R, int colour, bool fro
   const unsigned n = g.end[colour] - g.off[colour];
   if (n == 0) return HPG_OK;
   const int nslots = __builtin_popcount(gs_slot_mask(colour, from_zero)) - 1;
+  // two elements of an aligned R-vector share loads, addresses and tests
+  const int V = R > 1 && (((uintptr_t)r | (uintptr_t)z) & 7u) == 0 ? 2 : 1;
+  ColourPlan q = make_colour_plan(g, colour, V);
+  q.early = colour_early<T>(n / V, h->num_sms);
   return launch(h, K_GS, level, sizeof(T) == 8 ? HPG_FP64 : HPG_FP32,
                 L.cnt[colour] * (2.0 + nslots / 26.0) * R * sizeof(T), s, "gs_colour_kernel",
                 [&] {
                   const int block = sizeof(T) == 8 ? 64 : 256;
-                  return kl(h, colour_fn<T>(colour, from_zero), grid_for(n, block), block, s, g,
-                            make_coef<T>(h->beta), colour, r, level_diag<T>(L), z);
+                  ColourFn<T> fn = colour_fn<T, 1>(colour, from_zero);
+                  if constexpr (sizeof(T) == 4) {
+                    if (V == 2) fn = colour_fn<T, 2>(colour, from_zero);
+                  }
+                  return kl(h, fn, grid_for(n / V, block), block, s, q, make_coef<T>(h->beta), r,
+                            level_diag<T>(L), z);
                 });
 }
 int stencil_colour_phase(hpg_problem* h, int level, int R, int colour, bool from_zero,

@@ -1,0 +1,111 @@
+"""Grids far from a cube -- long lines, few planes, single planes -- and vectors of
+several right-hand sides on them: values bit for bit those of the stored-matrix or
+the single-vector kernels, and times near those of a compact grid of about the
+same number of points (each ratio stood at 1.6 or more where a rule looked at the
+number of points alone, or a kernel was slow on such a grid)."""
+
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import paper_2507_11512_gb300 as hpg  # noqa: E402
+from paper_2507_11512_gb300 import batch  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda"
+STORED = 3   # HPG_OPT_GS_PIPELINE: every sweep on the stored matrix
+DTYPE = {"fp32": torch.float32, "fp64": torch.float64}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+    __graft_entry__.build()
+    assert torch.cuda.is_available()
+
+
+def vec(p, dtype, seed):
+    g = torch.Generator(device="cpu").manual_seed(seed)
+    nat = torch.randn(p.info[0]["n"], generator=g, dtype=torch.float64).to(DEV)
+    return p.to_storage(nat, dtype=dtype)
+
+
+def graph_us(call):
+    """Device time of a call: eight of them in a CUDA graph, the fastest of ten replays."""
+    call()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        for _ in range(8):
+            call()
+    best = float("inf")
+    for _ in range(11):
+        e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        e0.record()
+        g.replay()
+        e1.record()
+        torch.cuda.synchronize()
+        best = min(best, e0.elapsed_time(e1) * 1e3 / 8)
+    return best
+
+
+def case_us(op, prec, dims):
+    with hpg.Problem(*dims, beta=0.4, levels=1 if op == "smooth" else 4) as p:
+        r = vec(p, DTYPE[prec], 1)
+        z = torch.zeros_like(r)
+        if op == "smooth":
+            return graph_us(lambda: hpg.mg_smooth(p.h, 0, r, z, 1, False))
+        return graph_us(lambda: hpg.mg_vcycle(p.h, 0, r, z))
+
+
+# (what, precision, grid, compact grid, bound on the ratio of their times)
+TIMES = [
+    # lines that no plane takes: colour phases whose addresses are formed before the wait
+    # (47 us; 25 now) against 26 us by planes
+    ("smooth", "fp32", (2000, 4, 4), (1000, 8, 8), 1.4),
+]
+
+
+@pytest.mark.parametrize("op,prec,dims,compact,bound", TIMES)
+def test_time_against_a_compact_grid(op, prec, dims, compact, bound):
+    t, ref = case_us(op, prec, dims), case_us(op, prec, compact)
+    assert t <= bound * ref, (t, ref)
+
+
+LONG_LINES = [(2000, 4, 4), (3100, 3, 2), (1700, 5, 7)]
+
+
+@pytest.mark.parametrize("dims", LONG_LINES)
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("theta", [False, True])
+def test_sweeps_equal_stored_matrix(dims, prec, theta):
+    n = dims[0] * dims[1] * dims[2]
+    g = torch.Generator(device="cpu").manual_seed(3)
+    th = (0.9 + 0.2 * torch.rand(n, generator=g, dtype=torch.float64)).numpy() if theta else None
+    with hpg.Problem(*dims, beta=-0.4, levels=1, theta=th) as p:
+        r, z0 = vec(p, DTYPE[prec], 1), vec(p, DTYPE[prec], 2)
+        out = []
+        for pipe in (1, STORED):
+            hpg.set_option(p.h, hpg.HPG_OPT_GS_PIPELINE, pipe)
+            for zero in (True, False):
+                z = z0.clone()
+                hpg.mg_smooth(p.h, 0, r, z, 1, zero)
+                out.append(z)
+        assert torch.equal(out[0], out[2]) and torch.equal(out[1], out[3])
+
+
+# lines longer than a plane's CTA takes, even and odd edges
+@pytest.mark.parametrize("dims", [(1600, 3, 4), (801, 5, 3)])
+@pytest.mark.parametrize("R", [2, 4, 8])
+@pytest.mark.parametrize("theta", [False, True])
+def test_rvector_colour_phases_equal_single_vector(dims, R, theta):
+    n = dims[0] * dims[1] * dims[2]
+    g = torch.Generator(device="cpu").manual_seed(3)
+    th = (0.9 + 0.2 * torch.rand(n, generator=g, dtype=torch.float64)).numpy() if theta else None
+    with hpg.Problem(*dims, beta=0.5, levels=1, theta=th) as p:
+        X = torch.stack([vec(p, torch.float32, 20 + q) for q in range(R)], dim=1).contiguous()
+        Y = torch.empty_like(X)
+        batch.vcycle_batch(p.h, 0, X, Y)
+        for q in range(R):
+            assert torch.equal(Y[:, q], p.vcycle(X[:, q].contiguous())), q
