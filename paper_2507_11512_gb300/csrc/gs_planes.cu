@@ -6,6 +6,7 @@
 // kernels' bit for bit.
 
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "stencil.cuh"
@@ -722,11 +723,45 @@ int stencil_colour_phase(hpg_problem* h, int level, int R, int colour, bool from
   return colour_phase_t<double>(h, level, R, colour, from_zero, r, z, s);
 }
 
-// FP64 sweeps from this many points on run one launch per colour: there a launch
-// costs little beside its FP64 work, and small blocks use every SM's FP64 unit,
-// which whole planes cannot (one sweep, planes against colours: 96^3 150 / 153 us,
-// 112^3 213 / 219, 128^3 440 / 287, 200^3 1444 / 945).
-constexpr long long kColourPoints64 = 1000000;
+// Whether a sweep takes one launch per colour although its planes fit: where whole
+// planes leave SMs without work (few planes, or FP64, whose time is the busiest SM's),
+// or lines are so short that a thread's elements are padding.  Both times are
+// estimated, in us, from linear fits to 550 sweeps (GB300, 1 to 8 right-hand sides,
+// cubes of 12 to 208 and flat, long and thin grids): planes by the busiest SM's elements
+// (of the lines a CTA computes, in thousands) and its rounds of lines, colours by
+// phases and elements per SM, to 15 % and 6 %.  `least` counts what the host needs to
+// launch a phase where that is more.  Planes against colours, one sweep:
+// FP64 64^3 48 / 60 us, 72^3 77 / 69, 96^3 150 / 132, 128^3 434 / 263, 200 x 200 x 1 92 / 19,
+// 128 x 128 x 8 136 / 43, 64 x 64 x 16 43 / 40, 8 x 1000 x 8 73 / 40; FP32 128^3 31 / 68, 128 x
+// 128 x 8 22 / 27, 300 x 300 x 4 47 / 32, 16 x 2000 x 4 44 / 27, 1 x 1000 x 1000 82 / 29.
+struct SweepCost { double launch, work, round, phase, element, least; };
+template <typename T>
+static bool by_colours(const SGeom& g, const Level& L, const PlanePlan& pl, int V, bool vec,
+                       int num_sms) {
+  const SweepCost c = sizeof(T) == 8 ? SweepCost{4.0, 11.0, 1.0, 2.3, 8.4, 3.3}
+                      : g.R == 1     ? SweepCost{3.3, 1.0, 0.25, 1.9, 1.66, 1.9}
+                                     : SweepCost{2.6, 0.75, 0.75, 1.7, 0.8, 1.7};
+  // clusters do not reach every SM; CTAs beyond one an SM come two at a time where two fit
+  const double ctas = (double)g.de * pl.cs, sms = num_sms, reach = pl.cs > 1 ? 0.85 * sms : sms;
+  const bool two = pl.smem <= kPlaneSmemGoal;
+  const double busiest = ctas <= reach ? 1.0 : std::max(2.0, std::ceil(ctas / (two ? sms : reach)));
+  const double waves =
+      std::ceil(ctas / ((two && pl.bx * pl.by <= kPlaneThreads / 2 ? 2.0 : 1.0) * reach));
+  const double lines = std::min(pl.lines, g.ny) + (pl.cs > 1 ? 1.5 : 0.0);   // with the halo
+  const double elements = lines * 2.0 * pl.bx * V / 1000.0 * (vec ? 1.0 : 1.5);
+  const double rounds = (pl.lines / 2 + 2 + pl.by - 1) / pl.by;
+  const double body = c.work * busiest * elements + c.round * waves * rounds;
+  // without odd planes one launch runs seven phases, otherwise three run fifteen
+  const double planes = g.dO > 0 ? 3.0 * (c.launch + body) : c.launch + 5.0 / 3.0 * body;
+  double phases = 0.0, points = 0.0;
+  for (int q = 0; q < kColours; ++q) {
+    const double times = q < kColours - 1 ? 2.0 : 1.0;
+    if (L.cnt[q] > 0) phases += times;
+    points += times * (double)L.cnt[q];
+  }
+  return std::max(c.least * phases, c.phase * phases + c.element * points * g.R / sms / 1000.0) <
+         planes;
+}
 
 // One symmetric sweep; c0_done: z already holds colour 0's first phase.
 template <typename T>
@@ -742,7 +777,7 @@ static int symgs_t(hpg_problem* h, int level, int R, const T* r, T* z, bool from
   const bool fits = V == 4   ? plane_plan<T, 4>(g, h->num_sms, &pl)
                     : V == 2 ? plane_plan<T, 2>(g, h->num_sms, &pl)
                              : plane_plan<T, 1>(g, h->num_sms, &pl);
-  if (!fits || (R > 1 && !vec) || (sizeof(T) == 8 && L.n >= kColourPoints64)) {
+  if (!fits || (R > 1 && !vec) || by_colours<T>(g, L, pl, V, vec, h->num_sms)) {
     for (int c = c0_done ? 1 : 0; c < kColours; ++c)
       if ((rc = stencil_colour_phase(h, level, R, c, from_zero, r, z, s))) return rc;
     for (int c = kColours - 2; c >= 0; --c)

@@ -64,6 +64,13 @@ TIMES = [
     # lines that no plane takes: colour phases whose addresses are formed before the wait
     # (47 us; 25 now) against 26 us by planes
     ("smooth", "fp32", (2000, 4, 4), (1000, 8, 8), 1.4),
+    # few planes, in FP64 few busy SMs: colours instead (136, 92 and 47 us; 43, 19 and 32
+    # now, against 42, 26 and 15 by planes)
+    ("smooth", "fp64", (128, 128, 8), (64, 64, 32), 1.6),
+    ("smooth", "fp64", (200, 200, 1), (40, 40, 40), 1.6),
+    ("smooth", "fp32", (300, 300, 4), (72, 72, 72), 2.6),
+    # lines of one point (82 us; 29 now, against 28)
+    ("smooth", "fp32", (1, 1000, 1000), (104, 104, 104), 1.6),
 ]
 
 
@@ -73,10 +80,10 @@ def test_time_against_a_compact_grid(op, prec, dims, compact, bound):
     assert t <= bound * ref, (t, ref)
 
 
-LONG_LINES = [(2000, 4, 4), (3100, 3, 2), (1700, 5, 7)]
-
-
-@pytest.mark.parametrize("dims", LONG_LINES)
+# lines that no plane takes; grids on both sides of the choice between planes and colours
+@pytest.mark.parametrize("dims", [(2000, 4, 4), (3100, 3, 2), (1700, 5, 7),
+                                  (200, 200, 1), (128, 128, 8), (150, 150, 2), (1, 300, 300),
+                                  (2, 300, 300), (72, 71, 72), (64, 64, 64), (16, 2000, 4)])
 @pytest.mark.parametrize("prec", ["fp32", "fp64"])
 @pytest.mark.parametrize("theta", [False, True])
 def test_sweeps_equal_stored_matrix(dims, prec, theta):
