@@ -29,14 +29,19 @@ constexpr int kTailThreads = 512;
 constexpr int kTailCtas = 16, kTailPortableCtas = 8;
 constexpr int kTailOps = 160;
 constexpr size_t kTailSmem = 227u << 10;
-// Largest first level (points times right-hand sides).  Measured: with the 32^3
-// FP32 level the 128^3 V-cycle takes 138 us, without it 144; a 40^3 level in the
-// cluster made its V-cycle 125 instead of 80 us, a 24^3 FP64 level 180 instead of
-// 158 (eight SMs' FP64 units against all).
-constexpr long long kTailPoints32 = 33000, kTailPoints64 = 5000;
-// A sweep alone pays for one launch instead of three (15.3 -> 10.9 us of host time)
-// but loads and stores the level (16^3 13.5 us against 11.1, 32^3 19 against 11).
-constexpr long long kTailSweepPoints32 = 16384;
+// Largest first level, by the points (times right-hand sides) of a CTA: a level of few
+// planes has few CTAs, so its total says nothing.  Measured, V-cycles, with the
+// level in the cluster / launched by itself: FP32 32^3 (2048 points a CTA) 66 / 71 us,
+// 28^3 x 2 (3136) 58 / 62, 40 x 40 x 8 (3200) 70 / 66, 32^3 x 2 (4096) 78 / 72, 64 x 64 x 8
+// (8192) 105 / 70, 90 x 88 x 4 (15840) 120 / 64; FP64 16^3 (512) 133 / 146, 20^3 (800)
+// 109 / 118, 16 x 16 x 64 (1024) 147 / 145, 24^3 (1152) 158 / 152 (a few SMs' FP64 units
+// against all).
+constexpr long long kTailPoints32 = 3200, kTailPoints64 = 900;
+// A sweep alone pays for one launch instead of three, but loads and stores the level.
+// Host and device time of a call, here / by planes: FP32 12^3 (288 points a CTA) 16 /
+// 14 us, 16^3 (512) 14 / 14, 33 x 17 x 24 (1122) 17 / 18, 24^3 (1152) 16 / 14, 64 x 64 x 4
+// (8192) 35 / 14; FP64 16^3 25 / 27, 24 x 16 x 12 (768) 27 / 27, 24 x 24 x 8 (1152) 34 / 27.
+constexpr long long kTailSweepPoints32 = 1140, kTailSweepPoints64 = 600;
 
 // Quotients by a fixed divisor (below 2^16, dividends likewise).
 struct FastDiv {
@@ -347,6 +352,9 @@ vcycle_tail_kernel(const __grid_constant__ TailParams<T> P) {
         P.z[p] = P.given ? fma(T(-0.0), ld_dep(P.z + p), ld_dep(P.r + p)) : ld_dep(P.r + p);
 }
 
+static int tail_planes(int nz, int ctas) {   // planes per CTA of the first level
+  return std::max(2, ((nz + ctas - 1) / ctas + 1) / 2 * 2);
+}
 // Fills P for the V-cycle from `level` down, or for `sweeps` > 0 sweeps on it;
 // false if it does not fit.
 template <typename T>
@@ -355,7 +363,7 @@ static bool tail_plan(const hpg_problem* h, int level, int R, int sweeps, bool f
   P.nlev = sweeps ? 1 : h->nlev - level;
   P.given = sweeps && !from_zero;
   const Geom& top = h->lev[level].g;
-  P.ppc = std::max(2, ((top.nz + ctas - 1) / ctas + 1) / 2 * 2);
+  P.ppc = tail_planes(top.nz, ctas);
   P.ctas = (top.nz + P.ppc - 1) / P.ppc;
   P.c = make_coef<T>(h->beta);
   long long off = 0;
@@ -454,12 +462,14 @@ template <typename T>
 static int tail_t(hpg_problem* h, int level, int R, const T* r, T* z, int sweeps,
                   bool from_zero, bool c0_done, cudaStream_t s) {
   const Level& top = h->lev[level];
-  const long long most = sizeof(T) == 8 ? kTailPoints64 : sweeps ? kTailSweepPoints32 : kTailPoints32;
-  if (top.n * R > most) return HPG_ERR_UNSUPPORTED;
   TailParams<T> P;
   int most_ctas = 0;
   const int prc = tail_ctas<T>(h, &most_ctas);
   if (prc) return prc;
+  const long long most = sizeof(T) == 8 ? (sweeps ? kTailSweepPoints64 : kTailPoints64)
+                                        : (sweeps ? kTailSweepPoints32 : kTailPoints32);
+  if ((long long)tail_planes(top.g.nz, most_ctas) * top.g.nx * top.g.ny * R > most)
+    return HPG_ERR_UNSUPPORTED;
   if (!tail_plan(h, level, R, sweeps, from_zero, most_ctas, P)) return HPG_ERR_UNSUPPORTED;
   P.r = r;
   P.z = z;

@@ -71,6 +71,10 @@ TIMES = [
     ("smooth", "fp32", (300, 300, 4), (72, 72, 72), 2.6),
     # lines of one point (82 us; 29 now, against 28)
     ("smooth", "fp32", (1, 1000, 1000), (104, 104, 104), 1.6),
+    # few planes are few CTAs of the small levels' cluster (120 and 34 us; 65 and 12 now,
+    # against 66 and 13)
+    ("vcycle", "fp32", (90, 88, 4), (32, 32, 32), 1.4),
+    ("smooth", "fp32", (64, 64, 4), (32, 32, 32), 1.6),
 ]
 
 
@@ -116,3 +120,23 @@ def test_rvector_colour_phases_equal_single_vector(dims, R, theta):
         batch.vcycle_batch(p.h, 0, X, Y)
         for q in range(R):
             assert torch.equal(Y[:, q], p.vcycle(X[:, q].contiguous())), q
+
+
+# V-cycles that leave the small levels' cluster: planes and colours with a diagonal per
+# cell, two and four elements a thread (600,000 elements), odd edges
+@pytest.mark.parametrize("dims", [(45, 37, 41), (64, 64, 8), (64, 64, 2), (46, 44, 40),
+                                  (45, 44, 40)])
+@pytest.mark.parametrize("R", [2, 4, 8])
+def test_rvector_vcycle_with_cell_diagonals_equals_single_vector(dims, R):
+    n = dims[0] * dims[1] * dims[2]
+    g = torch.Generator(device="cpu").manual_seed(3)
+    th = (0.9 + 0.2 * torch.rand(n, generator=g, dtype=torch.float64)).numpy()
+    with hpg.Problem(*dims, beta=0.5, theta=th) as p:
+        X = torch.stack([vec(p, torch.float32, 20 + q) for q in range(R)], dim=1).contiguous()
+        Y = torch.empty_like(X)
+        batch.vcycle_batch(p.h, 0, X, Y)
+        for q in range(R):
+            assert torch.equal(Y[:, q], p.vcycle(X[:, q].contiguous())), q
+        batch.spmv_batch(p.h, 0, X, Y)
+        for q in range(R):
+            assert torch.equal(Y[:, q], p.spmv(X[:, q].contiguous())), q
