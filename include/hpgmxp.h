@@ -390,9 +390,8 @@ HPG_API int hpg_set_execution(hpg_problem_t* h, int mode);
  * previous phase within one grid plane of it are done (bounded waits; a wait
  * that runs out makes the solve return HPG_ERR_TIMEOUT) instead of one launch
  * per colour phase; same results.  It runs on the stored matrix and is mostly
- * slower than the default sweeps.  0: never; 1 (default): FP64 sweeps, from a given
- * iterate on levels of 1.9 to 6 million points, where it is the faster one, and of
- * a level after hpg_inject_stall; 2: always; 3: on every level.  Setting
+ * slower than the default sweeps.  0: never; 1 (default): FP64 sweeps of a level after
+ * hpg_inject_stall; 2: always; 3: on every level.  Setting
  * an option drops captured solve graphs (single- and many-right-hand-side).
  * HPG_ERR_INVALID for an unknown option; HPG_ERR_STATE while a multi-system
  * batch uses the problem (its graph keeps the options it was captured

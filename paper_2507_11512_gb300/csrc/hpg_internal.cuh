@@ -281,7 +281,7 @@ struct hpg_problem {
   bool coarse_cta = false;        // coarsest level's sweep in one CTA when it fits
   long long pdl_rows = 16384;     // HPG_OPT_PDL_ROWS (accepted, without effect)
   int gs_pipeline = 1;            // pipelined sweep kernel: 0 never; on streamed levels
-                                  // 1 some FP64 sweeps (symgs), 2 always;
+                                  // 1 FP64 sweeps of a stalled level, 2 always;
                                   // 3 every level
   unsigned* pipe_err = nullptr;   // device word: a pipelined sweep's wait ran out
   int tail_ctas[2] = {0, 0};      // vcycle_tail.cu: cluster size per precision (0: not asked)

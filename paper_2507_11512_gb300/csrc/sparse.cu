@@ -523,21 +523,15 @@ static int symgs_pipelined(hpg_problem* h, int level, const T* r, T* z, bool fro
                 });
 }
 
-constexpr long long kStoredPoints64 = 1900000, kStoredPointsMax64 = 6000000;
-
 // One symmetric Gauss-Seidel sweep (eqs. (1)-(2)): colours 0..7 then 7..0.
 template <typename T>
 static int symgs(hpg_problem* h, int level, const T* r, T* z, bool from_zero, SweepState& st,
                  cudaStream_t s) {
   const Level& L = h->lev[level];
   const bool streamed_level = L.g.n_store * 27LL * 8 > kStreamMatrixBytes;
-  // FP64 sweeps of a given iterate between these sizes are still fastest on the
-  // stored matrix (128^3 280 us against 287 by colours, 160^3 494 / 510; 200^3 1011
-  // / 945)
-  const bool stored64 = sizeof(T) == 8 && (L.stalled || (!from_zero && L.n >= kStoredPoints64 &&
-                                                         L.n <= kStoredPointsMax64));
   const bool pipe = h->gs_pipeline == 3 ||
-                    (streamed_level && (h->gs_pipeline == 2 || (h->gs_pipeline == 1 && stored64)));
+                    (streamed_level && (h->gs_pipeline == 2 ||
+                                        (h->gs_pipeline == 1 && sizeof(T) == 8 && L.stalled)));
   if (pipe && L.pipe_flags && h->pipe_err)
     return symgs_pipelined<T>(h, level, r, z, from_zero, st, s);
   int rc;

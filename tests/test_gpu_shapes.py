@@ -122,6 +122,19 @@ def test_rvector_colour_phases_equal_single_vector(dims, R, theta):
             assert torch.equal(Y[:, q], p.vcycle(X[:, q].contiguous())), q
 
 
+@pytest.mark.parametrize("dims", [(128, 128, 128), (160, 128, 104), (96, 96, 96)])
+def test_default_sweeps_read_no_stored_matrix(dims):
+    """By the profile's byte model: vectors alone, at every size (the pipelined sweep on
+    the stored matrix, 15/8 x 27 x 12 bytes a point, was the default in a band of sizes)."""
+    with hpg.Problem(*dims, beta=0.4, levels=1) as p:
+        r, z = vec(p, torch.float64, 1), vec(p, torch.float64, 2)
+        hpg.set_profiling(p.h, True)
+        hpg.mg_smooth(p.h, 0, r, z, 1, False)
+        torch.cuda.synchronize()
+        total = sum(k["bytes"] for k in hpg.profile_report(p.h))
+    assert 0 < total < 100.0 * p.info[0]["n"]
+
+
 # V-cycles that leave the small levels' cluster: planes and colours with a diagonal per
 # cell, two and four elements a thread (600,000 elements), odd edges
 @pytest.mark.parametrize("dims", [(45, 37, 41), (64, 64, 8), (64, 64, 2), (46, 44, 40),
