@@ -59,8 +59,9 @@ __device__ __forceinline__ void st_n(float* p, const float (&v)[N]) {
 }
 
 // ------------------------------------------------- multi-RHS stencil kernels
-// Prolongation and correction z_{f_c(I)} += zc_I (eq. (3) transposed).
-template <int R>
+// Prolongation and correction z_{f_c(I)} += zc_I (eq. (3) transposed).  ALIGNED: the R
+// values of a row of z are aligned for vector loads (a caller's z need not be).
+template <int R, bool ALIGNED>
 __global__ void __launch_bounds__(256)
 mprolong_kernel(const __grid_constant__ Geom gf, const __grid_constant__ Geom gc,
                 const float* __restrict__ zc, float* __restrict__ z) {
@@ -75,11 +76,18 @@ mprolong_kernel(const __grid_constant__ Geom gf, const __grid_constant__ Geom gc
   const int K = (int)(p / ((long long)cx * cy));
   const long long row = gf.off[kCoarseColour] + p;
   float a[R], b[R];
-  ld_n<R>(z + row * R, a);
   ld_n<R>(zc + store_index(gc, I, J, K) * R, b);
+  if (ALIGNED) {
+    ld_n<R>(z + row * R, a);
 #pragma unroll
-  for (int r = 0; r < R; ++r) a[r] += b[r];
-  st_n<R>(z + row * R, a);
+    for (int r = 0; r < R; ++r) a[r] += b[r];
+    st_n<R>(z + row * R, a);
+  } else {
+#pragma unroll
+    for (int r = 0; r < R; ++r) a[r] = ld_dep(z + row * R + r);
+#pragma unroll
+    for (int r = 0; r < R; ++r) z[row * R + r] = a[r] + b[r];
+  }
 }
 
 // Natural order (R vectors of n values, vector r at in[r * n]) <-> storage
@@ -264,7 +272,9 @@ static int mvcycle_t(hpg_problem* h, int l, const float* rhs, float* z, cudaStre
   if (rc) return rc;
   if ((rc = mvcycle_t<R>(h, l + 1, rcv, zcv, s))) return rc;
   rc = launch(h, K_PROLONG, l, HPG_FP32, cnt * 3.0 * 4 * R, s, "mprolong_kernel", [&] {
-    return kl(h, mprolong_kernel<R>, grid_for(cnt, 256), 256, s, L.g, C.g, (const float*)zcv, z);
+    const bool aligned = ((uintptr_t)z & (sizeof(float) * std::min(R, 4) - 1)) == 0;
+    return kl(h, aligned ? mprolong_kernel<R, true> : mprolong_kernel<R, false>, grid_for(cnt, 256),
+              256, s, L.g, C.g, (const float*)zcv, z);
   });
   if (rc) return rc;
   for (int it = 0; it < h->post; ++it)

@@ -109,10 +109,11 @@ static int spmv_t(hpg_problem* h, int level, int R, const T* x, T* y, cudaStream
                                 make_coef<double>(h->beta), (unsigned)L.g.n_store, x, diag, y);
                   const bool vec = whole_groups<T, row_elems<T>()>(g, x, y);
                   if constexpr (sizeof(T) == 4) {   // R-vectors are FP32
-                    if (R == 8) return spmv_launch<T, 8, true>(h, g, x, diag, y, block, s);
-                    if (R == 4) return spmv_launch<T, 4, true>(h, g, x, diag, y, block, s);
-                    if (R == 2) return spmv_launch<T, 2, true>(h, g, x, diag, y, block, s);
-                    if (!vec) return spmv_launch<T, 1, false>(h, g, x, diag, y, block, s);
+                    auto fn = R == 8   ? (vec ? spmv_launch<T, 8, true> : spmv_launch<T, 8, false>)
+                              : R == 4 ? (vec ? spmv_launch<T, 4, true> : spmv_launch<T, 4, false>)
+                              : R == 2 ? (vec ? spmv_launch<T, 2, true> : spmv_launch<T, 2, false>)
+                              : vec    ? spmv_launch<T, 1, true> : spmv_launch<T, 1, false>;
+                    return fn(h, g, x, diag, y, block, s);
                   }
                   return spmv_launch<T, 1, true>(h, g, x, diag, y, block, s);
                 });

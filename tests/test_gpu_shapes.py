@@ -153,3 +153,22 @@ def test_rvector_vcycle_with_cell_diagonals_equals_single_vector(dims, R):
         batch.spmv_batch(p.h, 0, X, Y)
         for q in range(R):
             assert torch.equal(Y[:, q], p.spmv(X[:, q].contiguous())), q
+
+
+# R-vectors anywhere on a 4-byte boundary: the product and the V-cycle (small levels'
+# cluster, planes, colours) give what aligned vectors give and write nothing beside them
+@pytest.mark.parametrize("dims", [(24, 20, 28), (64, 48, 40), (45, 37, 41), (64, 64, 8)])
+@pytest.mark.parametrize("R", [2, 4, 8])
+@pytest.mark.parametrize("off", [1, 2, 3])
+def test_rvectors_off_a_vector_boundary(dims, R, off):
+    with hpg.Problem(*dims, beta=0.5) as p:
+        X = torch.stack([vec(p, torch.float32, 20 + q) for q in range(R)], dim=1).contiguous()
+        n = X.numel()
+        for f in (batch.spmv_batch, batch.vcycle_batch):
+            ref = torch.empty_like(X)
+            f(p.h, 0, X, ref)
+            xb, yb = (torch.zeros(n + 4, dtype=torch.float32, device=DEV) for _ in range(2))
+            xb[off:off + n] = X.reshape(-1)
+            f(p.h, 0, xb[off:off + n].view(-1, R), yb[off:off + n].view(-1, R))
+            assert torch.equal(yb[off:off + n].view(-1, R), ref)
+            assert not yb[:off].any() and not yb[off + n:].any()
