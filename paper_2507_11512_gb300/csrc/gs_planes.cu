@@ -13,54 +13,6 @@
 
 namespace hpg {
 
-// Quotients by a fixed divisor below 2^31 of dividends below 2^31 (Granlund and
-// Montgomery, PLDI 1994: the multiplier for 31-bit operands fits 32 bits).
-struct Div31 {
-  unsigned d, m, sh;
-  explicit Div31(unsigned n) : d(n), m(0), sh(0) {
-    if (n <= 1) return;
-    unsigned s = 1;
-    while ((1ULL << s) < n) ++s;
-    m = (unsigned)((1ULL << (31 + s)) / n + 1);
-    sh = s - 1;
-  }
-  __device__ __forceinline__ unsigned div(unsigned t) const { return m ? __umulhi(t, m) >> sh : t; }
-};
-
-// What a colour phase needs of its level, in elements of an R-vector.  A
-// neighbour's line part is told by which of its parities differ from the colour's:
-// flip f (bit 0 x, 1 y, 2 z) starts at o[f] and steps w[f] a line, wh[f] a plane; slot
-// s adds d[s].
-struct ColourPlan {
-  unsigned off, cnt, end;     // the colour's block (end: with padding rows)
-  Div31 across, lines;        // a line's element groups, a plane's lines
-  int px, py, pz, ny, nz, R, rshift;
-  int early;                  // whether the next kernel may start while this one runs
-  unsigned o[8], w[8], wh[8];
-  int d[kSlots];
-};
-static ColourPlan make_colour_plan(const SGeom& g, int colour, int V) {
-  const int px = colour_parity_x(colour), py = colour_parity_y(colour),
-            pz = colour_parity_z(colour);
-  ColourPlan q{g.off[colour], g.cnt[colour], g.end[colour],
-               Div31((unsigned)((px ? g.wo : g.we) / V)), Div31((unsigned)(py ? g.ho : g.he))};
-  q.px = px; q.py = py; q.pz = pz; q.ny = g.ny; q.nz = g.nz; q.R = g.R;
-  q.rshift = g.R == 8 ? 3 : g.R >> 1;
-  q.early = 1;
-  for (int f = 0; f < 8; ++f) {
-    const int x = px ^ (f & 1), y = py ^ (f >> 1 & 1), z = pz ^ (f >> 2);
-    q.o[f] = g.off[(x ^ 1) | (y ^ 1) << 1 | (z ^ 1) << 2];
-    q.w[f] = (unsigned)(x ? g.wo : g.we);
-    q.wh[f] = q.w[f] * (unsigned)(y ? g.ho : g.he);
-  }
-  for (int s = 0; s < kSlots; ++s) {
-    const int dx = s % 3 - 1, dy = (s / 3) % 3 - 1, dz = s / 9 - 1;
-    const int f = (dx & 1) | (dy & 1) << 1 | (dz & 1) << 2;
-    q.d[s] = ((px + dx) >> 1) * g.R + ((py + dy) >> 1) * (int)q.w[f] + ((pz + dz) >> 1) * (int)q.wh[f];
-  }
-  return q;
-}
-
 // One colour phase (Sec. 3.2.1), V consecutive elements of a line per thread (V
 // divides R, so that neighbour groups are aligned), in place: FP64 sweeps of larger
 // levels and levels whose planes do not fit (see symgs_t), and phases beside the
@@ -96,34 +48,17 @@ gs_colour_kernel(const __grid_constant__ ColourPlan g, const __grid_constant__ C
     }
     return;
   }
-  const unsigned q = g.across.div(t), e = (t - q * g.across.d) * V;
-  const unsigned K = g.lines.div(q), J = q - K * g.lines.d;
-  const int j = 2 * (int)J + g.py, k = 2 * (int)K + g.pz;
-  // whether the points before and after exist along x, y and z
-  const bool lo[3] = {g.px || e >= (unsigned)g.R, j > 0, k > 0};
-  const bool up[3] = {e + (unsigned)(g.px * g.R) < g.w[1], j + 1 < g.ny, k + 1 < g.nz};
-  const bool edge = !(lo[0] && up[0] && lo[1] && up[1] && lo[2] && up[2]);
-  unsigned base[8];
-#pragma unroll
-  for (int f = 0; f < 8; ++f) {
-    base[f] = g.o[f] + g.w[f] * J + g.wh[f] * K + e;
-    asm volatile("" : "+r"(base[f]));   // formed here, not after the wait
-  }
+  const ColourPlace at(g, t, V);
+  const bool edge = at.edge();
   const T dg = diag ? diag[row >> g.rshift] : T(0);
   pdl_wait();
   T x[kSlots][V], u[V];
 #pragma unroll
   for (int s = 0; s < kSlots; ++s) {
-    const int dx = s % 3 - 1, dy = (s / 3) % 3 - 1, dz = s / 9 - 1;
 #pragma unroll
     for (int v = 0; v < V; ++v) x[s][v] = T(0);
     if (s == kCentre ? MC >= 0 : !((kMask >> s) & 1u)) continue;
-    bool in = s != kCentre || edge;
-    if (dx) in = in && (dx < 0 ? lo[0] : up[0]);
-    if (dy) in = in && (dy < 0 ? lo[1] : up[1]);
-    if (dz) in = in && (dz < 0 ? lo[2] : up[2]);
-    const unsigned f = (dx & 1) | (dy & 1) << 1 | (dz & 1) << 2;
-    if (in) unpack(ld_dep(reinterpret_cast<const P*>(z + (base[f] + (unsigned)g.d[s]))), x[s]);
+    if (s == kCentre ? edge : at.in(s)) unpack(ld_dep(reinterpret_cast<const P*>(z + at.at(g, s))), x[s]);
   }
   unpack(ld_dep(reinterpret_cast<const P*>(r + row)), u);
 #pragma unroll

@@ -303,10 +303,10 @@ void destroy_profiler(hpg_problem* h);
 // serialization attribute when the previous operation on s was a kernel of
 // the chain (and not while profiling).
 template <typename... KArgs, typename... Args>
-cudaError_t kl(hpg_problem* h, void (*kern)(KArgs...), int grid, int block, cudaStream_t s,
+cudaError_t kl(hpg_problem* h, void (*kern)(KArgs...), dim3 grid, int block, cudaStream_t s,
                Args&&... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)block);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = s;

@@ -46,8 +46,7 @@ stencil_spmv_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coe
 
 // The same with one thread per storage row, for FP64 levels between these sizes,
 // whose FP64 work single rows spread most evenly over the SMs (rows against pairs
-// of lines: 40^3 6.2 / 7.0 us, 72^3 20.9 / 23.9, 96^3 44.7 / 45.5; 128^3 101 / 99, 16^3
-// 5.0 / 4.2).
+// of lines: 40^3 6.2 / 7.0 us, 72^3 20.9 / 23.9, 96^3 44.7 / 45.5; 128^3 101 / 99).
 constexpr long long kRowPoints64 = 60000, kRowPointsMax64 = 1500000;
 __global__ void __launch_bounds__(64)
 stencil_spmv_row_kernel(const __grid_constant__ SGeom g, const __grid_constant__ Coef<double> c,
@@ -62,6 +61,39 @@ stencil_spmv_row_kernel(const __grid_constant__ SGeom g, const __grid_constant__
     v = fma(a, ld_dep(x + q), v);
   });
   y[row] = point ? v : ld_dep(x + row);   // padding row: identity
+}
+
+// FP64 levels below kRowPoints64: one thread per point, a row of the grid of blocks per
+// colour.  Bound by launch and latency, so every load issues at once from addresses
+// formed before the wait (16^3 4.1 us by lines, 2.8 here; 36^3 5.6 / 4.9; against the rows
+// above 40^3 6.2 / 6.2, 64^3 15.6 / 17.2: the 72 registers leave too few threads an SM).
+struct ColourPlans { ColourPlan c[kColours]; };
+__global__ void __launch_bounds__(64)
+stencil_spmv_point_kernel(const __grid_constant__ ColourPlans P, const __grid_constant__ Coef<double> c,
+                        const double* x, const double* diag, double* y) {
+  pdl_trigger();
+  const ColourPlan& g = P.c[blockIdx.y];
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x, row = g.off + t;
+  if (row >= g.end) return;
+  if (t >= g.cnt) {   // padding row: identity
+    pdl_wait();
+    y[row] = ld_dep(x + row);
+    return;
+  }
+  const ColourPlace at(g, t, 1);
+  const double dg = diag ? diag[row] : kDiag;
+  pdl_wait();
+  double v[kSlots], acc = 0.0;
+#pragma unroll
+  for (int s = 0; s < kSlots; ++s) {
+    v[s] = 0.0;
+    if (at.in(s)) v[s] = ld_dep(x + at.at(g, s));
+  }
+#pragma unroll
+  for (int s = 0; s < kSlots; ++s)
+    acc = fma(s == kCentre ? dg : c.a[s % 3 - 1 + (s / 3) % 3 - 1 + s / 9 - 1 + 3], v[s], acc);
+  if (at.edge()) pad_slot(v[kCentre], acc);
+  y[row] = acc;
 }
 
 RowPlan make_row_plan(const SGeom& g, int elems, int lines) {
@@ -79,19 +111,34 @@ static cudaError_t spmv_launch(hpg_problem* h, const SGeom& g, const T* x, const
                                int block, cudaStream_t s) {
   constexpr int V = row_elems<T>();
   // lines a thread takes: as many as leave every SM enough threads (FP32 64^3 4.6 us
-  // with one, 3.3 with two; 96^3 9.9 / 5.8 / 5.4 with one, two, four)
+  // with one, 3.3 with two; 96^3 9.9 / 5.8 / 5.4 with one, two, four); FP64 levels come
+  // here large
   const long long groups = (long long)((g.we + V - 1) / V) * g.ny * g.nz;
-  const int lines = groups < 25000 || (sizeof(T) == 8 && groups < 50000) ? 1
-                    : sizeof(T) == 8 || groups < 150000                  ? 2 : kRowLines;
+  const int lines = sizeof(T) == 8 ? 2 : groups < 25000 ? 1 : groups < 150000 ? 2 : kRowLines;
   const RowPlan pl = make_row_plan(g, V, lines);
   // small blocks spread few threads over all SMs, and FP64 work evenly (an SM
   // has one FP64 unit, 16 cycles a warp instruction)
   if (sizeof(T) == 8 || (long long)pl.threads <= 256LL * h->num_sms) block = 64;
-  return kl(h, lines == 1   ? stencil_spmv_kernel<T, R, VEC, 1>
-               : lines == 2 ? stencil_spmv_kernel<T, R, VEC, 2>
-                            : stencil_spmv_kernel<T, R, VEC, kRowLines>,
+  auto fn = stencil_spmv_kernel<T, R, VEC, 2>;
+  if constexpr (sizeof(T) == 4) {
+    if (lines == 1) fn = stencil_spmv_kernel<T, R, VEC, 1>;
+    if (lines == kRowLines) fn = stencil_spmv_kernel<T, R, VEC, kRowLines>;
+  }
+  return kl(h, fn,
             grid_for((long long)pl.threads + pl.pad, block), block, s, g, make_coef<T>(h->beta),
             pl, x, diag, y);
+}
+
+static cudaError_t spmv_points(hpg_problem* h, const SGeom& g, const double* x,
+                               const double* diag, double* y, cudaStream_t s) {
+  ColourPlans P;
+  unsigned most = 0;
+  for (int c = 0; c < kColours; ++c) {
+    P.c[c] = make_colour_plan(g, c, 1);
+    most = std::max(most, g.end[c] - g.off[c]);
+  }
+  return kl(h, stencil_spmv_point_kernel, dim3((unsigned)grid_for(most, 64), kColours), 64, s, P,
+            make_coef<double>(h->beta), x, diag, y);
 }
 
 template <typename T>
@@ -103,10 +150,12 @@ static int spmv_t(hpg_problem* h, int level, int R, const T* x, T* y, cudaStream
   return launch(h, K_SPMV, level, sizeof(T) == 8 ? HPG_FP64 : HPG_FP32,
                 (double)L.n * R * 2.0 * sizeof(T) + (diag ? L.n * (double)sizeof(T) : 0.0), s,
                 "stencil_spmv_kernel", [&] {
-                  if constexpr (sizeof(T) == 8)
-                    if (L.n >= kRowPoints64 && L.n < kRowPointsMax64)
+                  if constexpr (sizeof(T) == 8) {
+                    if (L.n < kRowPoints64) return spmv_points(h, g, x, diag, y, s);
+                    if (L.n < kRowPointsMax64)
                       return kl(h, stencil_spmv_row_kernel, grid_for(L.g.n_store, 64), 64, s, g,
                                 make_coef<double>(h->beta), (unsigned)L.g.n_store, x, diag, y);
+                  }
                   const bool vec = whole_groups<T, row_elems<T>()>(g, x, y);
                   if constexpr (sizeof(T) == 4) {   // R-vectors are FP32
                     auto fn = R == 8   ? (vec ? spmv_launch<T, 8, true> : spmv_launch<T, 8, false>)

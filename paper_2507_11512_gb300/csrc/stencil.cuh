@@ -252,6 +252,93 @@ __device__ __forceinline__ bool for_row_slots(const SGeom& g, unsigned row, F&& 
   return true;
 }
 
+// Quotients by a fixed divisor below 2^31 of dividends below 2^31 (Granlund and
+// Montgomery, PLDI 1994: the multiplier for 31-bit operands fits 32 bits).
+struct Div31 {
+  unsigned d, m, sh;
+  explicit Div31(unsigned n = 1) : d(n), m(0), sh(0) {
+    if (n <= 1) return;
+    unsigned s = 1;
+    while ((1ULL << s) < n) ++s;
+    m = (unsigned)((1ULL << (31 + s)) / n + 1);
+    sh = s - 1;
+  }
+  __device__ __forceinline__ unsigned div(unsigned t) const { return m ? __umulhi(t, m) >> sh : t; }
+};
+
+// What a kernel with one thread per point of a colour needs of its level, in
+// elements of an R-vector.  A
+// neighbour's line part is told by which of its parities differ from the colour's:
+// flip f (bit 0 x, 1 y, 2 z) starts at o[f] and steps w[f] a line, wh[f] a plane; slot
+// s adds d[s].
+struct ColourPlan {
+  unsigned off, cnt, end;     // the colour's block (end: with padding rows)
+  Div31 across, lines;        // a line's element groups, a plane's lines
+  int px, py, pz, ny, nz, R, rshift;
+  int early;                  // whether the next kernel may start while this one runs
+  unsigned o[8], w[8], wh[8];
+  int d[kSlots];
+};
+inline ColourPlan make_colour_plan(const SGeom& g, int colour, int V) {
+  const int px = colour_parity_x(colour), py = colour_parity_y(colour),
+            pz = colour_parity_z(colour);
+  ColourPlan q{g.off[colour], g.cnt[colour], g.end[colour],
+               Div31((unsigned)((px ? g.wo : g.we) / V)), Div31((unsigned)(py ? g.ho : g.he))};
+  q.px = px; q.py = py; q.pz = pz; q.ny = g.ny; q.nz = g.nz; q.R = g.R;
+  q.rshift = g.R == 8 ? 3 : g.R >> 1;
+  q.early = 1;
+  for (int f = 0; f < 8; ++f) {
+    const int x = px ^ (f & 1), y = py ^ (f >> 1 & 1), z = pz ^ (f >> 2);
+    q.o[f] = g.off[(x ^ 1) | (y ^ 1) << 1 | (z ^ 1) << 2];
+    q.w[f] = (unsigned)(x ? g.wo : g.we);
+    q.wh[f] = q.w[f] * (unsigned)(y ? g.ho : g.he);
+  }
+  for (int s = 0; s < kSlots; ++s) {
+    const int dx = s % 3 - 1, dy = (s / 3) % 3 - 1, dz = s / 9 - 1;
+    const int f = (dx & 1) | (dy & 1) << 1 | (dz & 1) << 2;
+    q.d[s] = ((px + dx) >> 1) * g.R + ((py + dy) >> 1) * (int)q.w[f] + ((pz + dz) >> 1) * (int)q.wh[f];
+  }
+  return q;
+}
+
+// A thread's place in a colour (element p = V t of its block): line element e, line J
+// and plane K of the colour, whether the points before and after exist along x, y
+// and z, and the first element of each flip's line part at its place.
+struct ColourPlace {
+  bool lo[3], up[3];
+  unsigned base[8];
+  __device__ __forceinline__ ColourPlace(const ColourPlan& g, unsigned t, int V) {
+    const unsigned q = g.across.div(t), e = (t - q * g.across.d) * V;
+    const unsigned K = g.lines.div(q), J = q - K * g.lines.d;
+    const int j = 2 * (int)J + g.py, k = 2 * (int)K + g.pz;
+    lo[0] = g.px || e >= (unsigned)g.R;
+    up[0] = e + (unsigned)(g.px * g.R) < g.w[1];
+    lo[1] = j > 0, up[1] = j + 1 < g.ny;
+    lo[2] = k > 0, up[2] = k + 1 < g.nz;
+#pragma unroll
+    for (int f = 0; f < 8; ++f) {
+      base[f] = g.o[f] + g.w[f] * J + g.wh[f] * K + e;
+      asm volatile("" : "+r"(base[f]));   // formed here, not after the caller's wait
+    }
+  }
+  __device__ __forceinline__ bool edge() const {
+    return !(lo[0] && up[0] && lo[1] && up[1] && lo[2] && up[2]);
+  }
+  // neighbour at slot s: whether it exists, and its element
+  __device__ __forceinline__ bool in(int s) const {
+    const int d[3] = {s % 3 - 1, (s / 3) % 3 - 1, s / 9 - 1};
+    bool v = true;
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+      if (d[a]) v = v && (d[a] < 0 ? lo[a] : up[a]);
+    return v;
+  }
+  __device__ __forceinline__ unsigned at(const ColourPlan& g, int s) const {
+    const int dx = s % 3 - 1, dy = (s / 3) % 3 - 1, dz = s / 9 - 1;
+    return base[(dx & 1) | (dy & 1) << 1 | (dz & 1) << 2] + (unsigned)g.d[s];
+  }
+};
+
 // Lines a thread of a whole-grid product takes (stencil_rows), at most: they
 // share their neighbour lines in registers.
 constexpr int kRowLines = 4;

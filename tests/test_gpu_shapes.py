@@ -32,12 +32,12 @@ def vec(p, dtype, seed):
 
 
 def graph_us(call):
-    """Device time of a call: eight of them in a CUDA graph, the fastest of ten replays."""
+    """Device time of a call: 32 of them in a CUDA graph, the fastest of eleven replays."""
     call()
     torch.cuda.synchronize()
     g = torch.cuda.CUDAGraph()
     with torch.cuda.graph(g):
-        for _ in range(8):
+        for _ in range(32):
             call()
     best = float("inf")
     for _ in range(11):
@@ -46,7 +46,7 @@ def graph_us(call):
         g.replay()
         e1.record()
         torch.cuda.synchronize()
-        best = min(best, e0.elapsed_time(e1) * 1e3 / 8)
+        best = min(best, e0.elapsed_time(e1) * 1e3 / 32)
     return best
 
 
@@ -54,6 +54,8 @@ def case_us(op, prec, dims):
     with hpg.Problem(*dims, beta=0.4, levels=1 if op == "smooth" else 4) as p:
         r = vec(p, DTYPE[prec], 1)
         z = torch.zeros_like(r)
+        if op == "spmv":
+            return graph_us(lambda: hpg.spmv(p.h, 0, r, z))
         if op == "smooth":
             return graph_us(lambda: hpg.mg_smooth(p.h, 0, r, z, 1, False))
         return graph_us(lambda: hpg.mg_vcycle(p.h, 0, r, z))
@@ -75,6 +77,8 @@ TIMES = [
     # against 66 and 13)
     ("vcycle", "fp32", (90, 88, 4), (32, 32, 32), 1.4),
     ("smooth", "fp32", (64, 64, 4), (32, 32, 32), 1.6),
+    # a small product's launch and latency (4.1 us; 2.8 now, against 15.6)
+    ("spmv", "fp64", (16, 16, 16), (64, 64, 64), 0.23),
 ]
 
 
@@ -172,3 +176,36 @@ def test_rvectors_off_a_vector_boundary(dims, R, off):
             f(p.h, 0, xb[off:off + n].view(-1, R), yb[off:off + n].view(-1, R))
             assert torch.equal(yb[off:off + n].view(-1, R), ref)
             assert not yb[:off].any() and not yb[off + n:].any()
+
+
+# FP64 products by single points, by rows and by lines, with a diagonal per cell
+@pytest.mark.parametrize("dims", [(16, 16, 16), (33, 17, 24), (5, 1, 3), (1, 1, 40), (45, 37, 41),
+                                  (64, 63, 30), (130, 128, 100)])
+@pytest.mark.parametrize("theta", [False, True])
+def test_fp64_product_against_plain_torch(dims, theta):
+    nx, ny, nz = dims
+    n, beta = nx * ny * nz, -0.4
+    g = torch.Generator(device="cpu").manual_seed(3)
+    th = 0.9 + 0.2 * torch.rand(n, generator=g, dtype=torch.float64)
+    x = torch.randn(n, generator=g, dtype=torch.float64).to(DEV)
+
+    def product(v, b, diag):
+        vp = torch.nn.functional.pad(v.view(nz, ny, nx), (1, 1, 1, 1, 1, 1))
+        y = (diag * v).view(nz, ny, nx).clone()
+        for q in range(27):
+            dx, dy, dz = q % 3, q // 3 % 3, q // 9
+            if q != 13:
+                y += (-1.0 + b * (dx + dy + dz - 3) / 3.0) * vp[dz:dz + nz, dy:dy + ny, dx:dx + nx]
+        return y.reshape(-1)
+
+    diag = 26.0 * th.to(DEV) if theta else torch.full_like(x, 26.0)
+    with hpg.Problem(*dims, beta=beta, levels=1, theta=th.numpy() if theta else None) as p:
+        y = p.to_natural(p.spmv(p.to_storage(x)))
+        # padding rows are identity rows
+        pad = torch.ones(p.n_store(0), dtype=torch.float64, device=DEV)
+        pad[p.to_storage(torch.ones_like(x)) != 0] = 0
+        assert torch.equal(p.spmv(pad), pad)
+    # |A||x|: 26 theta and at most 1.4 a neighbour; 27 FMAs and the rounding of a
+    # coefficient make 28 u of it, twice that with the reference's own
+    scale = diag * x.abs() - 1.4 * product(x.abs(), 0.0, torch.zeros_like(x))
+    assert ((y - product(x, beta, diag)).abs() <= 2 * 28 * 2.0 ** -53 * scale).all()
