@@ -67,7 +67,7 @@ def get_shape(h, level, kind, nrhs):
 
 
 def tune(h, nrhs, stream=None):
-    """Autotunes the multi-right-hand-side launch shapes of every level."""
+    """hpg_batch_tune: times the block sizes of the level-0 SpMV and keeps the fastest."""
     check(load().hpg_batch_tune(h, nrhs, _stream(stream)), "hpg_batch_tune")
 
 
@@ -75,8 +75,8 @@ class BatchSolver:
     """Several Problems solved by one CUDA graph launch (hpg_batch_*)."""
 
     def __init__(self, problems, nrhs, restart=30, tune_shapes=False):
-        """tune_shapes: per-problem isolated tuning (hpg_batch_tune) before the
-        capture; for the batch itself prefer tune(), which times the batch."""
+        """tune_shapes: per-problem tuning of the SpMV (hpg_batch_tune) before the
+        capture."""
         self.problems = list(problems)
         self.nrhs = nrhs
         self.restart = restart
@@ -101,8 +101,9 @@ class BatchSolver:
         return [d[i * self.nrhs:(i + 1) * self.nrhs] for i in range(n)]
 
     def tune(self, Bs, Xs, tol=1e-9, maxit=10000, stream=None):
-        """hpg_batch_tune_solve: times whole batch solves of (Bs, Xs) per
-        candidate launch shape and keeps the fastest (Xs is overwritten)."""
+        """hpg_batch_tune_solve: recaptures the graph with the present shapes and times a
+        solve of (Bs, Xs) from zero (Xs is overwritten); the time is returned under each
+        number of lanes per row, which all launch the same kernels."""
         n = len(self.problems)
         bp = (ctypes.c_void_p * n)(*[_ptr(b) for b in Bs])
         xp = (ctypes.c_void_p * n)(*[_ptr(x) for x in Xs])
@@ -165,9 +166,8 @@ def main(argv=None):
     solver = BatchSolver(probs, a.nrhs)
     tune_ms = None
     if not a.no_tune:
-        tune_ms = solver.tune(Bs, Xs, tol=a.tol)
+        tune_ms = solver.tune(Bs, Xs, tol=a.tol)[1]
     create_s = time.perf_counter() - t1
-    shape = get_shape(probs[0].h, 0, KIND_GS, a.nrhs)
     times, infos = [], None
     for it in range(a.reps + 1):
         for x in Xs:
@@ -217,7 +217,7 @@ def main(argv=None):
         "rhs_solved_per_s": a.systems * a.nrhs / (ms / 1e3),
         "iterations_min_median_max": [min(its), sorted(its)[len(its) // 2], max(its)],
         "setup_s": setup_s, "tune_and_capture_s": create_s, "tuned": not a.no_tune,
-        "lanes_per_row": shape[0], "tuning_solve_ms_by_lanes_per_row": tune_ms,
+        "tuning_solve_ms": tune_ms,
         "roofline": {"bound": "hbm", "bytes": total_bytes, "achieved": gbs, "unit": "GB/s",
                      "peak": peak, "frac": gbs / peak if peak else None,
                      "timing": "library per-launch algorithmic bytes of every system's "

@@ -106,19 +106,31 @@ RowPlan make_row_plan(const SGeom& g, int elems, int lines) {
   return p;
 }
 
+// lines a thread takes: as many as leave every SM enough threads (FP32 64^3 4.6 us
+// with one, 3.3 with two; 96^3 9.9 / 5.8 / 5.4 with one, two, four); FP64 levels come
+// here large
+template <typename T> static RowPlan spmv_plan(const SGeom& g, int* lines) {
+  constexpr int V = row_elems<T>();
+  const long long groups = (long long)((g.we + V - 1) / V) * g.ny * g.nz;
+  *lines = sizeof(T) == 8 ? 2 : groups < 25000 ? 1 : groups < 150000 ? 2 : kRowLines;
+  return make_row_plan(g, V, *lines);
+}
+// whether the block size is the caller's: small blocks spread few threads over all SMs,
+// and FP64 work evenly (an SM has one FP64 unit, 16 cycles a warp instruction)
+template <typename T> static bool spmv_takes_block(const hpg_problem* h, const RowPlan& pl) {
+  return sizeof(T) == 4 && (long long)pl.threads > 256LL * h->num_sms;
+}
+bool stencil_spmv_takes_block(const hpg_problem* h, int level, int R) {
+  int lines;
+  return spmv_takes_block<float>(h, spmv_plan<float>(make_sgeom(h->lev[level].g, R), &lines));
+}
+
 template <typename T, int R, bool VEC>
 static cudaError_t spmv_launch(hpg_problem* h, const SGeom& g, const T* x, const T* diag, T* y,
                                int block, cudaStream_t s) {
-  constexpr int V = row_elems<T>();
-  // lines a thread takes: as many as leave every SM enough threads (FP32 64^3 4.6 us
-  // with one, 3.3 with two; 96^3 9.9 / 5.8 / 5.4 with one, two, four); FP64 levels come
-  // here large
-  const long long groups = (long long)((g.we + V - 1) / V) * g.ny * g.nz;
-  const int lines = sizeof(T) == 8 ? 2 : groups < 25000 ? 1 : groups < 150000 ? 2 : kRowLines;
-  const RowPlan pl = make_row_plan(g, V, lines);
-  // small blocks spread few threads over all SMs, and FP64 work evenly (an SM
-  // has one FP64 unit, 16 cycles a warp instruction)
-  if (sizeof(T) == 8 || (long long)pl.threads <= 256LL * h->num_sms) block = 64;
+  int lines;
+  const RowPlan pl = spmv_plan<T>(g, &lines);
+  if (!spmv_takes_block<T>(h, pl)) block = 64;
   auto fn = stencil_spmv_kernel<T, R, VEC, 2>;
   if constexpr (sizeof(T) == 4) {
     if (lines == 1) fn = stencil_spmv_kernel<T, R, VEC, 1>;

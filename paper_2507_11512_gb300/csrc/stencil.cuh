@@ -491,6 +491,8 @@ int stencil_spmv(hpg_problem* h, int level, int R, const float* x, float* y, cud
                  int block = 256);
 int stencil_spmv(hpg_problem* h, int level, int R, const double* x, double* y, cudaStream_t s,
                  int block = 256);
+// Whether an FP32 product of R vectors runs with the given block size.
+bool stencil_spmv_takes_block(const hpg_problem* h, int level, int R);
 int stencil_restrict(hpg_problem* h, int level, int R, const float* r, const float* z, float* rc,
                      float* zc0, cudaStream_t s);
 int stencil_restrict(hpg_problem* h, int level, int R, const double* r, const double* z,
