@@ -635,7 +635,9 @@ static int colour_phase_t(hpg_problem* h, int level, int R, int colour, bool fro
   const int nslots = __builtin_popcount(gs_slot_mask(colour, from_zero)) - 1;
   // two elements of an aligned R-vector share loads, addresses and tests
   const int V = R > 1 && (((uintptr_t)r | (uintptr_t)z) & 7u) == 0 ? 2 : 1;
-  ColourPlan q = make_colour_plan(g, colour, V);
+  ColourPlan q = make_colour_plan(
+      g, colour, Div31((unsigned)((colour_parity_x(colour) ? g.wo : g.we) / V)),
+      Div31((unsigned)(colour_parity_y(colour) ? g.ho : g.he)));
   q.early = colour_early<T>(n / V, h->num_sms);
   return launch(h, K_GS, level, sizeof(T) == 8 ? HPG_FP64 : HPG_FP32,
                 L.cnt[colour] * (2.0 + nslots / 26.0) * R * sizeof(T), s, "gs_colour_kernel",

@@ -67,12 +67,17 @@ stencil_spmv_row_kernel(const __grid_constant__ SGeom g, const __grid_constant__
 // colour.  Bound by launch and latency, so every load issues at once from addresses
 // formed before the wait (16^3 4.1 us by lines, 2.8 here; 36^3 5.6 / 4.9; against the rows
 // above 40^3 6.2 / 6.2, 64^3 15.6 / 17.2: the 72 registers leave too few threads an SM).
-struct ColourPlans { ColourPlan c[kColours]; };
+struct PointGeom {   // across, lines: by parity
+  SGeom g;
+  Div31 across[2], lines[2];
+};
 __global__ void __launch_bounds__(64)
-stencil_spmv_point_kernel(const __grid_constant__ ColourPlans P, const __grid_constant__ Coef<double> c,
-                        const double* x, const double* diag, double* y) {
+stencil_spmv_point_kernel(const __grid_constant__ PointGeom P, const __grid_constant__ Coef<double> c,
+                          const double* x, const double* diag, double* y) {
   pdl_trigger();
-  const ColourPlan& g = P.c[blockIdx.y];
+  const int colour = (int)blockIdx.y;
+  const ColourPlan g = make_colour_plan(P.g, colour, P.across[colour_parity_x(colour)],
+                                        P.lines[colour_parity_y(colour)]);
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x, row = g.off + t;
   if (row >= g.end) return;
   if (t >= g.cnt) {   // padding row: identity
@@ -143,12 +148,14 @@ static cudaError_t spmv_launch(hpg_problem* h, const SGeom& g, const T* x, const
 
 static cudaError_t spmv_points(hpg_problem* h, const SGeom& g, const double* x,
                                const double* diag, double* y, cudaStream_t s) {
-  ColourPlans P;
+  PointGeom P;
+  P.g = g;
+  P.across[0] = Div31((unsigned)g.we);
+  P.across[1] = Div31((unsigned)g.wo);
+  P.lines[0] = Div31((unsigned)g.he);
+  P.lines[1] = Div31((unsigned)g.ho);
   unsigned most = 0;
-  for (int c = 0; c < kColours; ++c) {
-    P.c[c] = make_colour_plan(g, c, 1);
-    most = std::max(most, g.end[c] - g.off[c]);
-  }
+  for (int c = 0; c < kColours; ++c) most = std::max(most, g.end[c] - g.off[c]);
   return kl(h, stencil_spmv_point_kernel, dim3((unsigned)grid_for(most, 64), kColours), 64, s, P,
             make_coef<double>(h->beta), x, diag, y);
 }

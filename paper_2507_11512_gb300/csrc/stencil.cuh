@@ -256,12 +256,11 @@ __device__ __forceinline__ bool for_row_slots(const SGeom& g, unsigned row, F&& 
 // Montgomery, PLDI 1994: the multiplier for 31-bit operands fits 32 bits).
 struct Div31 {
   unsigned d, m, sh;
-  explicit Div31(unsigned n = 1) : d(n), m(0), sh(0) {
+  Div31() = default;
+  __host__ explicit Div31(unsigned n) : d(n), m(0), sh(0) {
     if (n <= 1) return;
-    unsigned s = 1;
-    while ((1ULL << s) < n) ++s;
-    m = (unsigned)((1ULL << (31 + s)) / n + 1);
-    sh = s - 1;
+    sh = 31 - (unsigned)__builtin_clz(n - 1);   // 2^sh < n <= 2^(sh + 1)
+    m = (unsigned)((1ULL << (32 + sh)) / n + 1);
   }
   __device__ __forceinline__ unsigned div(unsigned t) const { return m ? __umulhi(t, m) >> sh : t; }
 };
@@ -279,24 +278,28 @@ struct ColourPlan {
   unsigned o[8], w[8], wh[8];
   int d[kSlots];
 };
-inline ColourPlan make_colour_plan(const SGeom& g, int colour, int V) {
+// across, lines: of the colour's x and y parity.
+__host__ __device__ inline ColourPlan make_colour_plan(const SGeom& g, int colour, Div31 across,
+                                                      Div31 lines) {
   const int px = colour_parity_x(colour), py = colour_parity_y(colour),
             pz = colour_parity_z(colour);
-  ColourPlan q{g.off[colour], g.cnt[colour], g.end[colour],
-               Div31((unsigned)((px ? g.wo : g.we) / V)), Div31((unsigned)(py ? g.ho : g.he))};
+  ColourPlan q{g.off[colour], g.cnt[colour], g.end[colour], across, lines};
   q.px = px; q.py = py; q.pz = pz; q.ny = g.ny; q.nz = g.nz; q.R = g.R;
   q.rshift = g.R == 8 ? 3 : g.R >> 1;
   q.early = 1;
+#pragma unroll
   for (int f = 0; f < 8; ++f) {
     const int x = px ^ (f & 1), y = py ^ (f >> 1 & 1), z = pz ^ (f >> 2);
     q.o[f] = g.off[(x ^ 1) | (y ^ 1) << 1 | (z ^ 1) << 2];
     q.w[f] = (unsigned)(x ? g.wo : g.we);
     q.wh[f] = q.w[f] * (unsigned)(y ? g.ho : g.he);
   }
+#pragma unroll
   for (int s = 0; s < kSlots; ++s) {
     const int dx = s % 3 - 1, dy = (s / 3) % 3 - 1, dz = s / 9 - 1;
-    const int f = (dx & 1) | (dy & 1) << 1 | (dz & 1) << 2;
-    q.d[s] = ((px + dx) >> 1) * g.R + ((py + dy) >> 1) * (int)q.w[f] + ((pz + dz) >> 1) * (int)q.wh[f];
+    const int f = (dx & 1) | (dy & 1) << 1;   // w and wh do not depend on the z parity
+    q.d[s] = ((px + dx) >> 1) * g.R + ((py + dy) >> 1) * (int)q.w[f] +
+             ((pz + dz) >> 1) * (int)q.wh[f];
   }
   return q;
 }
