@@ -31,12 +31,12 @@ if ROOT not in sys.path:
 METRIC = "GMRES-IR GFLOP/s and time-to-1e-9 residual, MxP vs FP64, 1 GB300; % HBM peak"
 FALLBACK_HBM_GBS = 6800.0
 
-# DRAM bytes (read + write) per launch of the level-0 FP32 Gauss-Seidel plane
-# kernel at 128^3, from one ncu capture of that kernel (None: not captured),
-# valid while the kernel's source text (the kernel and the helpers it inlines)
-# hashes to `sources_sha256`.
-GS_TRAFFIC = {"workload": "mxp_gmres30_128cube", "bytes_per_launch": None,
-              "sources_sha256": "0" * 64}
+# DRAM bytes (read + write, cold L2) per launch of the level-0 FP32 Gauss-Seidel
+# plane kernel at 128^3, the mean of a sweep's three launches in one ncu capture
+# (None: not captured), valid while the kernel's source text (the kernel and the
+# helpers it inlines) hashes to `sources_sha256`.
+GS_TRAFFIC = {"workload": "mxp_gmres30_128cube", "bytes_per_launch": 12631211.0,
+              "sources_sha256": "bb59e06dd094a4ac7b67f6e51564e73b4032ef5f708d3dc4d1d50d52b806781a"}
 # (file, first line of the block, text that ends it): the kernel's source
 GS_KERNEL_TEXT = (
     ("paper_2507_11512_gb300/csrc/gs_planes.cu", "enum PlaneKind", "// Shared memory of a plane CTA"),
@@ -407,7 +407,8 @@ def run_gpu(args):
     # graph-timed time per solve
     solve_bytes = sum(p["bytes"] for p in prof)
     solve_gbs = solve_bytes / (ms_max / args.steps / 1e3) / 1e9
-    roofline = {"bound": "hbm", "kernel": "gs_plane_kernel (level 0, fp32)",
+    roofline = {"bound": "instruction issue and latency (the vectors of 128^3 stay in L2)",
+                "kernel": "gs_plane_kernel (level 0, fp32)",
                 "achieved": gs_gbs, "peak": peak, "unit": "GB/s", "frac": gs_gbs / peak,
                 "peak_source": peak_src,
                 "traffic": traffic,
@@ -484,8 +485,7 @@ def run_gpu(args):
                        "l2": "working set larger than L2 (Krylov basis of %d vectors, %.0f MB)" % (
                            w.restart + 1, (w.restart + 1) * prob.n_store() *
                            {"fp32": 4}.get(args.basis, 2) / 1e6),
-                       "operator": "evaluated from the grid, beta and theta (FP64 sweeps of a "
-                                   "given iterate read the stored ELL matrix)",
+                       "operator": "evaluated from the grid, beta and theta",
                        "parallelism": "replicas" if world > 1 else "single"},
             "gpu_launches": launches, "clocks": clocks,
             "cpu_baseline": cpu,

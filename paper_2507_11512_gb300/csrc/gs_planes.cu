@@ -125,8 +125,8 @@ template <typename T, int V> static ColourFn<T> colour_fn(int colour, bool from_
 // addresses for that reason), FP64 by the FP64 rate; small ones by the chain of
 // load, phases and store.
 // One sweep on GB300, stored matrix with a launch per colour -> this: FP32 64^3 39
-// -> 13 us, 128^3 139 -> 30 us, 320^3 2.1 ms -> 495 us; FP64 64^3 66 -> 48 us, 96^3 229
-// -> 150 us.
+// -> 13 us, 128^3 139 -> 30 us, 320^3 2.1 ms -> 495 us; FP64 64^3 66 -> 48 us.  Where
+// whole planes leave SMs without work the sweep goes by colours (by_colours).
 enum PlaneKind { kOddFwd = 0, kEven = 1, kOddBwd = 2 };
 
 struct PlanePlan {
@@ -158,8 +158,8 @@ __device__ __forceinline__ void copy_wait() {
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
-// Threads of a plane CTA, at most (a line's element groups must fit); two such
-// CTAs of the FP32 kernels fit an SM.
+// Threads of a plane CTA, at most (a line's element groups must fit).  At the kernels'
+// 64 to 80 registers one such CTA fits an SM; plans for two take half the threads.
 constexpr int kPlaneThreads = 768;
 // Shared-memory layout of a CTA: z of the lines a-2 .. b+2 of the planes k-1, k
 // and k+1, each line as
@@ -497,15 +497,14 @@ constexpr int kMaxPlaneCtas = 8;                // portable cluster size
 // at most two CTAs per SM, with at least 8 lines each (a CTA recomputes up to 3
 // more).  FP64, whose time is the busiest SM's FP64 work: the split of up to 5 CTAs
 // with the fewest lines on that SM -- one CTA per SM up to 85 % of the SMs (clusters
-// do not reach all of them), else whole rounds of two (64^3 sweep 76 -> 48 us, 80^3
-// 112 -> 92, against 5 CTAs throughout).
-// Up to 8 where a CTA's lines would take more shared memory than two CTAs per SM
-// have.  (Measured, one sweep: 128^3 FP32 30 us with 4 CTAs per plane, 37 with 3 or
-// 8; 96^3 FP64 150 us with 5, 177 with 4, 187 with 8.)  About 384
-// threads a CTA, twice that where only one fits an SM.  The next kernel may
-// start early only after grids that leave most SMs idle: otherwise its waiting
-// CTAs take the free places unevenly (96^3 FP64 V-cycle 595 us with an early start
-// everywhere, 493 us with this rule; 8^3 sweep 11.5 us without any, 9.5 us with).
+// do not reach all of them), else whole rounds of two (64^3 sweep 76 -> 48 us against 5
+// CTAs throughout).  Up to 8 where a CTA's lines would take more shared memory than
+// two CTAs per SM have.  (Measured, one sweep: 128^3 FP32 30 us with 4 CTAs per plane,
+// 37 with 3 or 8.)  About 384 threads a CTA, twice that where only one fits an SM.
+// The next kernel may start early only after grids that leave most SMs idle:
+// otherwise its waiting CTAs take the free places unevenly (96^3 FP64 V-cycle by planes
+// 595 us with an early start everywhere, 493 with this rule; 8^3 sweep 11.5 us without
+// any, 9.5 with).
 // False: a line has more element groups than a CTA threads, or its lines do not
 // fit shared memory even so.
 template <typename T, int V>

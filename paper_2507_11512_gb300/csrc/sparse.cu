@@ -36,7 +36,8 @@ template <> struct Prec<double> {
 // every thread computes its row from shared memory alone; a gather reads
 // index col + delta[slot], delta being the shared-memory offset of the run
 // holding that slot's neighbours minus the run's start in the vector.  Same
-// slots, order and arithmetic as gs_phase_kernel: results equal bit for bit.
+// slots, order of products and division as the sweeps from the grid: results equal bit
+// for bit.
 // STREAM marks the matrix copies evict-first in L2.  The copy wait is
 // bounded: if it runs out the CTA sets `err` (the solve then reports
 // HPG_ERR_TIMEOUT), waits (bounded) once more for its copies and skips its
@@ -234,7 +235,8 @@ __device__ __forceinline__ void st_release(int* p, int v) {
   asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// One row of a colour phase, arithmetic as gs_phase_kernel; gathers via L2.
+// One row of a colour phase: the products of its 26 slots in slot order, then the
+// division; gathers via L2.
 template <typename T, bool STREAM, bool MASKED>
 __device__ __forceinline__ void pipe_row(const T* __restrict__ vals, const int* __restrict__ cols,
                                          long long ns, const T* __restrict__ r, T* z,
@@ -563,7 +565,7 @@ static int symgs(hpg_problem* h, int level, const T* r, T* z, bool from_zero, Sw
 // thread loads the next phase's matrix row and r_i into registers while the
 // current phase computes, so the L2 latency of the matrix is off the chain.
 // Phases, slot sets, summation order and division are those of the launched
-// phases (gs_phase_small_kernel), so z is equal bit for bit.
+// phases, so z is equal bit for bit.
 constexpr int kCtaSweepRows = 512;
 struct CtaSweepPhase {
   int row0, nrows, valid_end;
